@@ -1,7 +1,8 @@
-"""Thin ctypes binding of the C-ABI library declared in include/dgq.h.
+"""Thin binding of the C-ABI library declared in include/dgq.h.
 
 Argument marshalling only: every step of the path runs in the library's CUDA
-kernels.  Tensors are torch CUDA tensors (device memory and streams come from
+kernels.  The calls of the hot path marshal their arguments and allocate their
+buffers in the native extension csrc/binding.cpp, the others through ctypes.  Tensors are torch CUDA tensors (device memory and streams come from
 PyTorch); their data pointers go to the library as plain pointers.  Loading
 fails loudly when the library has not been built.
 """
@@ -48,6 +49,26 @@ class DgqError(RuntimeError):
 
 
 _lib = None
+_native = None
+
+
+def native():
+    """The extension module with the hot-path calls (it links the library that `lib` loads)."""
+    global _native
+    if _native is None:
+        lib()
+        try:
+            from . import _native as ext
+        except ImportError as e:
+            raise RuntimeError("the native binding is missing or does not load: build it with "
+                               "`python -m paper_2501_04304_b200.build`") from e
+        _native = ext
+    return _native
+
+
+def _raw(h) -> int:
+    """Address of a library-owned handle, 0 for a closed one."""
+    return (h.value or 0) if h else 0
 
 
 def lib():
@@ -170,25 +191,18 @@ def groups_from_host(C_, P, act_bits, col_group, row_group, scale, zp) -> Groups
 
 def quantize_act(groups: Groups, X, timestep=0, mode=MODE_STATIC, layout=CODES_U8, out=None, stream=None):
     """dgq_quantize_act.  Returns (Xq uint8 [M, K_pad], dyn_scale or None, dyn_zp or None)."""
-    assert X.is_cuda and X.dtype == torch.float16 and X.dim() == 2 and X.stride(1) == 1
-    M = X.shape[0]
-    Xq = out if out is not None else torch.empty((M, groups.K_pad), dtype=torch.uint8, device=X.device)
-    ds = dz = None
-    if mode == MODE_DYNAMIC_TOKEN:
-        ds = torch.empty((M, groups.G), dtype=torch.float32, device=X.device)
-        dz = torch.empty((M, groups.G), dtype=torch.int32, device=X.device)
-    st = lib().dgq_quantize_act(groups.h, C.c_int(timestep), C.c_int(mode), C.c_int(layout), _ptr(X), C.c_int64(M),
-                                C.c_int64(X.stride(0)), _ptr(Xq), _ptr(ds), _ptr(dz), _stream(stream))
-    _check(st, "dgq_quantize_act")
-    return Xq, ds, dz
+    r = (_native or native()).quantize_act(_raw(groups.h), groups.K_pad, groups.G, timestep, mode, layout, X, out, None, None, 1,
+                                           stream)
+    if type(r) is int:
+        _check(r, "dgq_quantize_act")
+    return r
 
 
 def quantize_act_into(groups: Groups, X, Xq, ds, dz, timestep=0, mode=MODE_STATIC, layout=CODES_U8, stream=None):
     """dgq_quantize_act into caller-provided buffers (no allocation)."""
-    st = lib().dgq_quantize_act(groups.h, C.c_int(timestep), C.c_int(mode), C.c_int(layout), _ptr(X),
-                                C.c_int64(X.shape[0]), C.c_int64(X.stride(0)), _ptr(Xq), _ptr(ds), _ptr(dz),
-                                _stream(stream))
-    _check(st, "dgq_quantize_act")
+    r = (_native or native()).quantize_act(_raw(groups.h), groups.K_pad, groups.G, timestep, mode, layout, X, Xq, ds, dz, 0, stream)
+    if type(r) is int:
+        _check(r, "dgq_quantize_act")
 
 
 class Weight:
@@ -254,19 +268,11 @@ def linear(groups: Groups, weight: Weight, Xq, timestep=0, mode=MODE_STATIC, lay
     """dgq_linear.  Returns Y fp16 [M, N].  `workspace` (uint8 CUDA tensor) is only used for 4-bit
     weights; when it is None one of the size the library asks for is taken from torch, when it is
     False the call is made without one."""
-    M = Xq.shape[0]
-    Y = out if out is not None else torch.empty((M, weight.N), dtype=torch.float16, device=Xq.device)
-    if workspace is False:
-        workspace = None
-    elif workspace is None:
-        need = linear_workspace_bytes(groups, weight, M)
-        workspace = torch.empty(need, dtype=torch.uint8, device=Xq.device) if need else None
-    st = lib().dgq_linear(groups.h, weight.h, C.c_int(timestep), C.c_int(mode), C.c_int(layout), _ptr(Xq),
-                          _ptr(dyn_scale), _ptr(dyn_zp), _ptr(bias), _ptr(Y), C.c_int64(M), C.c_int64(Y.stride(0)),
-                          _conv(conv), _ptr(workspace), C.c_size_t(workspace.numel() if workspace is not None else 0),
-                          _stream(stream))
-    _check(st, "dgq_linear")
-    return Y
+    r = (_native or native()).linear(_raw(groups.h), _raw(weight.h), weight.N, timestep, mode, layout, Xq, dyn_scale, dyn_zp, bias,
+                                     out, conv, workspace, stream)
+    if type(r) is int:
+        _check(r, "dgq_linear")
+    return r
 
 
 def cross_attn_workspace_bytes(B, H, nq, nk, d) -> int:
@@ -280,41 +286,19 @@ def cross_attn_logq(Q, K, V, score_bits=8, scale_gran=SCALE_PER_PROMPT, fixed_sc
                     want_scale=False, want_codes=False, workspace=None, stream=None, v_bits=0):
     """dgq_cross_attn_logq (v_bits = 0) or dgq_cross_attn_logq_qv (quantized value operand, v_bits 2..8).
     Q [B, nq, H, d], K, V [B, nk, H, d] CUDA fp16.  Returns (O, scale, codes)."""
-    B, nq, H, d = Q.shape
-    nk = K.shape[1]
-    assert Q.is_contiguous() and K.is_contiguous() and V.is_contiguous()
-    O = out if out is not None else torch.empty_like(Q)
-    n_scope = {SCALE_PER_PROMPT: B, SCALE_PER_PROMPT_HEAD: B * H, SCALE_PER_CALL: 1}[scale_gran]
-    scale = torch.empty(n_scope, dtype=torch.float32, device=Q.device) if want_scale else None
-    codes = torch.empty((B, H, nq, nk - 1), dtype=torch.uint8, device=Q.device) if want_codes else None
-    need = cross_attn_workspace_bytes(B, H, nq, nk, d) if nk >= 2 else 256
-    ws = workspace if workspace is not None else torch.empty(need, dtype=torch.uint8, device=Q.device)
-    if v_bits:
-        st = lib().dgq_cross_attn_logq_qv(_ptr(Q), _ptr(K), _ptr(V), C.c_int(B), C.c_int(H), C.c_int(nq), C.c_int(nk),
-                                          C.c_int(d), C.c_int(score_bits), C.c_int(scale_gran), _ptr(fixed_scale),
-                                          C.c_int(v_bits), _ptr(O), _ptr(scale), _ptr(codes), _ptr(ws),
-                                          C.c_size_t(ws.numel()), _stream(stream))
-        _check(st, "dgq_cross_attn_logq_qv")
-        return O, scale, codes
-    st = lib().dgq_cross_attn_logq(_ptr(Q), _ptr(K), _ptr(V), C.c_int(B), C.c_int(H), C.c_int(nq), C.c_int(nk),
-                                   C.c_int(d), C.c_int(score_bits), C.c_int(scale_gran), _ptr(fixed_scale), _ptr(O),
-                                   _ptr(scale), _ptr(codes), _ptr(ws), C.c_size_t(ws.numel()), _stream(stream))
-    _check(st, "dgq_cross_attn_logq")
-    return O, scale, codes
+    r = (_native or native()).cross_attn_logq(Q, K, V, score_bits, scale_gran, fixed_scale, out, bool(want_scale),
+                                              bool(want_codes), workspace, v_bits, stream)
+    if type(r) is int:
+        _check(r, "dgq_cross_attn_logq_qv" if v_bits else "dgq_cross_attn_logq")
+    return r
 
 
 def self_attn_logq(Q, K, V, score_bits=8, fixed_scale=None, out=None, want_codes=False, stream=None):
     """dgq_self_attn_logq.  Q [B, nq, H, d], K, V [B, nk, H, d] CUDA fp16.  Returns (O, codes)."""
-    B, nq, H, d = Q.shape
-    nk = K.shape[1]
-    assert Q.is_contiguous() and K.is_contiguous() and V.is_contiguous()
-    O = out if out is not None else torch.empty_like(Q)
-    codes = torch.empty((B, H, nq, nk), dtype=torch.uint8, device=Q.device) if want_codes else None
-    st = lib().dgq_self_attn_logq(_ptr(Q), _ptr(K), _ptr(V), C.c_int(B), C.c_int(H), C.c_int(nq), C.c_int(nk),
-                                  C.c_int(d), C.c_int(score_bits), _ptr(fixed_scale), _ptr(O), _ptr(codes),
-                                  _stream(stream))
-    _check(st, "dgq_self_attn_logq")
-    return O, codes
+    r = (_native or native()).self_attn_logq(Q, K, V, score_bits, fixed_scale, out, bool(want_codes), stream)
+    if type(r) is int:
+        _check(r, "dgq_self_attn_logq")
+    return r
 
 
 NOALLOC_MAX_ROWS = 1 << 18

@@ -10,6 +10,7 @@
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -29,6 +30,48 @@ __device__ __forceinline__ void record_error(int code) { atomicCAS(&g_status_wor
     cudaError_t e__ = (expr);                    \
     if (e__ != cudaSuccess) return DGQ_ERR_CUDA; \
   } while (0)
+
+// Device memory of the library-owned objects and of the scratch their set-up needs: one stream-ordered pool per
+// device (cudaMalloc and cudaFree of a few MB take 300 us each, several times what preparing a layer takes).  The
+// pool keeps at most POOL_KEEP bytes beyond what is in use; the rest goes back to the device at the next
+// synchronisation.  Both calls may be made from any thread.
+constexpr uint64_t POOL_KEEP = 32ull << 20;
+static inline cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t stream) {
+  static std::mutex lock;
+  static cudaMemPool_t pools[64] = {nullptr};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> hold(lock);
+    if (!pools[dev]) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      cudaMemPool_t made;
+      uint64_t keep = POOL_KEEP;
+      if ((e = cudaMemPoolCreate(&made, &props)) != cudaSuccess) return e;
+      if ((e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
+      pools[dev] = made;
+    }
+    pool = pools[dev];
+  }
+  return cudaMallocFromPoolAsync(p, bytes, pool, stream);
+}
+// Frees an object's memory once nothing on the device uses it any more (as cudaFree does).
+static inline void pool_free(void* p) {
+  if (!p) return;
+  cudaPointerAttributes at;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) return;
+  if (at.device != dev) cudaSetDevice(at.device);
+  cudaDeviceSynchronize();
+  cudaFreeAsync(p, nullptr);
+  if (at.device != dev) cudaSetDevice(dev);
+}
 
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

@@ -1,7 +1,6 @@
 // Single translation unit of the DGQ library (one device status word, no relocatable device code).
 #include <climits>
 #include <cmath>
-#include <mutex>
 
 #include "common.cuh"
 #include "groups.cuh"

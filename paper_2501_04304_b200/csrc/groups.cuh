@@ -16,36 +16,73 @@ struct dgq_groups {
   std::vector<int32_t> zp;                                      // [T][R][G]
   std::vector<char> filled;                                     // [T]
   int device = 0;
-  // device copies
+  // device copies, one allocation
+  unsigned char* d_slab = nullptr;
   int16_t* d_perm = nullptr;          // [K_pad], -1 = padding
-  uint8_t* d_chunk_group = nullptr;   // [K_pad / 16] group of every 16-code chunk
   uint8_t* d_quant_head = nullptr;    // layout tables of the quantizer, as it keeps them in shared memory
   int32_t* d_row_group = nullptr;     // [P]
   int32_t* d_col_group = nullptr;     // [C]
-  float* d_scale = nullptr;           // [T][R][G]
+  float* d_scale = nullptr;           // [T][R][G], then d_inv_scale and d_zp of the same shape
   float* d_inv_scale = nullptr;
   int32_t* d_zp = nullptr;
+  int* d_cell = nullptr;              // scratch of a calibration: minima and maxima [2][R][G] as ordered integers
 };
 
 namespace dgq {
 
 // ------------------------------------------------------------------ kernels
-// Per-channel extrema (Eq. 4, d = channel): thread c walks a block of rows of column c.
+// Running range of eight neighbouring columns.  NaN never wins a packed minimum or maximum.
+struct Range8 {
+  __half2 lo[4], hi[4];
+  __device__ __forceinline__ void reset() {
+    const __half2 inf = __half2half2(__ushort_as_half(0x7C00)), ninf = __half2half2(__ushort_as_half(0xFC00));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      lo[i] = inf;
+      hi[i] = ninf;
+    }
+  }
+  __device__ __forceinline__ void add(const uint4& x) {
+    const __half2* h = reinterpret_cast<const __half2*>(&x);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      lo[i] = __hmin2(lo[i], h[i]);
+      hi[i] = __hmax2(hi[i], h[i]);
+    }
+  }
+  __device__ __forceinline__ float min_of(int i) const { return __half2float(i & 1 ? __high2half(lo[i >> 1]) : __low2half(lo[i >> 1])); }
+  __device__ __forceinline__ float max_of(int i) const { return __half2float(i & 1 ? __high2half(hi[i >> 1]) : __low2half(hi[i >> 1])); }
+};
+// Columns 8 v .. 8 v + 7 of a row; a last vector that the matrix does not fill is completed with NaN.
+__device__ __forceinline__ uint4 load8(const __half* row, int v, int C) {
+  if (v * 8 + 8 <= C) return __ldg(reinterpret_cast<const uint4*>(row) + v);
+  uint16_t h[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) h[i] = v * 8 + i < C ? __half_as_ushort(row[v * 8 + i]) : (uint16_t)0x7FFF;
+  return make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16, h[6] | (uint32_t)h[7] << 16);
+}
+
+// The calibration reductions read 16 bytes per thread and load, CAL_ROWS rows per block: with one 2-byte load per
+// row and thread and 128 rows per block a 4096 x 640 recording kept 32 blocks busy for 128 dependent steps each.
+constexpr int CAL_ROWS = 32;
+constexpr int CAL_THREADS = 256;
+
+// Per-channel extrema (Eq. 4, d = channel): a thread walks the rows of its block over eight columns.
 __global__ void channel_extrema_kernel(const __half* __restrict__ X, int64_t n_rows, int C, int64_t ld,
-                                       int rows_per_block, int* __restrict__ ch_min, int* __restrict__ ch_max) {
-  const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
-  const int64_t r1 = min(n_rows, r0 + rows_per_block);
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    float lo = INFINITY, hi = -INFINITY;
-    for (int64_t r = r0; r < r1; ++r) {
-      float v = __half2float(X[r * ld + c]);
-      lo = fminf(lo, v);
-      hi = fmaxf(hi, v);
-    }
-    if (r1 > r0) {
-      atomicMin(&ch_min[c], float_to_ordered(lo));
-      atomicMax(&ch_max[c], float_to_ordered(hi));
-    }
+                                       int* __restrict__ ch_min, int* __restrict__ ch_max) {
+  const int64_t r0 = (int64_t)blockIdx.x * CAL_ROWS;
+  const int rows = (int)min((int64_t)CAL_ROWS, n_rows - r0);
+  for (int v = threadIdx.x; v * 8 < C; v += CAL_THREADS) {
+    Range8 x;
+    x.reset();
+#pragma unroll 8
+    for (int r = 0; r < rows; ++r) x.add(load8(X + (r0 + r) * ld, v, C));
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (v * 8 + i < C) {
+        atomicMin(&ch_min[v * 8 + i], float_to_ordered(x.min_of(i)));
+        atomicMax(&ch_max[v * 8 + i], float_to_ordered(x.max_of(i)));
+      }
   }
 }
 
@@ -56,11 +93,15 @@ __global__ void pixel_extrema_kernel(const __half* __restrict__ X, int64_t n_row
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t r = warp; r < n_rows; r += n_warps) {
+    Range8 x;
+    x.reset();
+#pragma unroll 4
+    for (int v = lane; v * 8 < C; v += 32) x.add(load8(X + r * ld, v, C));
     float lo = INFINITY, hi = -INFINITY;
-    for (int c = lane; c < C; c += 32) {
-      float v = __half2float(X[r * ld + c]);
-      lo = fminf(lo, v);
-      hi = fmaxf(hi, v);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      lo = fminf(lo, x.min_of(i));
+      hi = fmaxf(hi, x.max_of(i));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -74,43 +115,56 @@ __global__ void pixel_extrema_kernel(const __half* __restrict__ X, int64_t n_row
   }
 }
 
-// Extrema of every (pixel group, channel group) cell (the x of Eq. 6).  Thread c keeps a running
-// range for its channel and flushes it when the row's pixel group changes.
+// Extrema of every (pixel group, channel group) cell (the x of Eq. 6).  A thread keeps the running range of eight
+// columns and flushes it into the block's cells when the row's pixel group changes; the block's cells go to
+// global memory once.
 __global__ void cell_extrema_kernel(const __half* __restrict__ X, int64_t n_rows, int C, int64_t ld, int P,
-                                    int rows_per_block, const int32_t* __restrict__ row_group,
-                                    const int32_t* __restrict__ col_group, int G, int* __restrict__ cell_min,
-                                    int* __restrict__ cell_max) {
-  const int64_t r0 = (int64_t)blockIdx.x * rows_per_block;
-  const int64_t r1 = min(n_rows, r0 + rows_per_block);
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    const int g = col_group[c];
-    float lo = INFINITY, hi = -INFINITY;
-    int cur = -1;
-    for (int64_t r = r0; r < r1; ++r) {
-      const int rg = row_group[r % P];
-      if (rg != cur) {
-        if (cur >= 0) {
-          atomicMin(&cell_min[cur * G + g], float_to_ordered(lo));
-          atomicMax(&cell_max[cur * G + g], float_to_ordered(hi));
+                                    const int32_t* __restrict__ row_group, const int32_t* __restrict__ col_group, int G,
+                                    int n_cells, int* __restrict__ cell_min, int* __restrict__ cell_max) {
+  extern __shared__ int cells[];  // [2][n_cells]
+  for (int i = threadIdx.x; i < n_cells; i += CAL_THREADS) {
+    cells[i] = INT_MAX;
+    cells[n_cells + i] = INT_MIN;
+  }
+  __syncthreads();
+  const int64_t r0 = (int64_t)blockIdx.x * CAL_ROWS;
+  const int rows = (int)min((int64_t)CAL_ROWS, n_rows - r0);
+  for (int v = threadIdx.x; v * 8 < C; v += CAL_THREADS) {
+    Range8 x;
+    x.reset();
+    auto flush = [&](int rg) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (v * 8 + i < C) {
+          const int cell = rg * G + __ldg(col_group + v * 8 + i);
+          atomicMin(&cells[cell], float_to_ordered(x.min_of(i)));
+          atomicMax(&cells[n_cells + cell], float_to_ordered(x.max_of(i)));
         }
+      x.reset();
+    };
+    int cur = __ldg(row_group + r0 % P);
+#pragma unroll 8
+    for (int r = 0; r < rows; ++r) {
+      const int rg = __ldg(row_group + (r0 + r) % P);
+      if (rg != cur) {
+        flush(cur);
         cur = rg;
-        lo = INFINITY;
-        hi = -INFINITY;
       }
-      float v = __half2float(X[r * ld + c]);
-      lo = fminf(lo, v);
-      hi = fmaxf(hi, v);
+      x.add(load8(X + (r0 + r) * ld, v, C));
     }
-    if (cur >= 0) {
-      atomicMin(&cell_min[cur * G + g], float_to_ordered(lo));
-      atomicMax(&cell_max[cur * G + g], float_to_ordered(hi));
-    }
+    flush(cur);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n_cells; i += CAL_THREADS) {
+    if (cells[i] != INT_MAX) atomicMin(&cell_min[i], cells[i]);
+    if (cells[n_cells + i] != INT_MIN) atomicMax(&cell_max[i], cells[n_cells + i]);
   }
 }
 
-__global__ void fill_int_kernel(int* p, int n, int v) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) p[i] = v;
+// n minima followed by n maxima
+__global__ void fill_extrema_kernel(int* p, int n) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < 2 * n) p[i] = i < n ? INT_MAX : INT_MIN;
 }
 
 // ------------------------------------------------------------------ host: grouping
@@ -125,8 +179,7 @@ static std::vector<int> kmeans_ranges(const std::vector<double>& vmin, const std
   std::vector<int> order(n);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-    volatile double wa = vmax[a] - vmin[a], wb = vmax[b] - vmin[b];
-    return wa < wb;
+    return vmax[a] - vmin[a] < vmax[b] - vmin[b];
   });
   std::vector<double> cx(K), cy(K);
   for (int k = 0; k < K; ++k) {
@@ -136,19 +189,29 @@ static std::vector<int> kmeans_ranges(const std::vector<double>& vmin, const std
   }
   std::vector<int> labels(n, -1), next(n);
   for (int it = 0; it < 100; ++it) {
-    for (int i = 0; i < n; ++i) {
-      int best = 0;
-      double bd = 0.0;
-      for (int k = 0; k < K; ++k) {
-        volatile double dx = vmin[i] - cx[k], dy = vmax[i] - cy[k];
-        volatile double dx2 = dx * dx, dy2 = dy * dy;
-        double d = dx2 + dy2;
-        if (k == 0 || d < bd) {
-          bd = d;
-          best = k;
+    // Squares and their sum are rounded one by one (host code is compiled without contraction).  Centroids outside,
+    // a block of points inside: the inner loop is a select without a carried dependency, two points per
+    // instruction.
+    constexpr int BLOCK = 64;
+    for (int i0 = 0; i0 < n; i0 += BLOCK) {
+      const int m = std::min(BLOCK, n - i0);
+      const double *x = &vmin[i0], *y = &vmax[i0];
+      double bd[BLOCK], best[BLOCK];
+      for (int i = 0; i < m; ++i) {
+        const double dx = x[i] - cx[0], dy = y[i] - cy[0];
+        bd[i] = dx * dx + dy * dy;
+        best[i] = 0.0;
+      }
+      for (int k = 1; k < K; ++k) {
+        const double ck = cx[k], dk = cy[k], label = (double)k;
+        for (int i = 0; i < m; ++i) {
+          const double dx = x[i] - ck, dy = y[i] - dk;
+          const double d = dx * dx + dy * dy;
+          best[i] = d < bd[i] ? label : best[i];
+          bd[i] = d < bd[i] ? d : bd[i];
         }
       }
-      next[i] = best;
+      for (int i = 0; i < m; ++i) next[i0 + i] = (int)best[i];
     }
     if (next == labels) break;
     labels = next;
@@ -173,8 +236,7 @@ static std::vector<int> kmeans_ranges(const std::vector<double>& vmin, const std
       if (has[k]) used.push_back(k);
   }
   std::stable_sort(used.begin(), used.end(), [&](int a, int b) {
-    volatile double wa = cy[a] - cx[a], wb = cy[b] - cx[b];
-    return wa < wb;
+    return cy[a] - cx[a] < cy[b] - cx[b];
   });
   std::vector<int> remap(K, -1);
   for (size_t j = 0; j < used.size(); ++j) remap[used[j]] = (int)j;
@@ -226,16 +288,7 @@ static std::vector<int> group_vectors(const std::vector<double>& vmin, const std
 // ------------------------------------------------------------------ host: object plumbing
 constexpr int GROUP_MIN_PAD = 8;
 
-static void groups_free_device(dgq_groups* g) {
-  cudaFree(g->d_perm);
-  cudaFree(g->d_chunk_group);
-  cudaFree(g->d_quant_head);
-  cudaFree(g->d_row_group);
-  cudaFree(g->d_col_group);
-  cudaFree(g->d_scale);
-  cudaFree(g->d_inv_scale);
-  cudaFree(g->d_zp);
-}
+static void groups_free_device(dgq_groups* g) { pool_free(g->d_slab); }
 
 // Padded, group-contiguous code layout: members of each group in ascending channel order, every
 // group padded to a multiple of DGQ_K_ATOM positions with at least GROUP_MIN_PAD padding positions.
@@ -249,7 +302,7 @@ __host__ __device__ inline int quant_head_bytes(int C, int K_pad) {
   return (quant_head_pm_offset(C, K_pad) + (K_pad >> 4) * 2 + 15) & ~15;
 }
 
-static dgq_status groups_build_layout(dgq_groups* g) {
+static dgq_status groups_build_layout(dgq_groups* g, cudaStream_t stream) {
   g->group_off.assign(g->G + 1, 0);
   g->perm.clear();
   for (int k = 0; k < g->G; ++k) {
@@ -261,53 +314,56 @@ static dgq_status groups_build_layout(dgq_groups* g) {
   }
   g->K_pad = (int)g->perm.size();
   g->group_off[g->G] = g->K_pad;
-  std::vector<int16_t> perm16(g->K_pad);
-  for (int i = 0; i < g->K_pad; ++i) perm16[i] = (int16_t)g->perm[i];
-  std::vector<uint8_t> cg(g->K_pad / 16);
+  const size_t tn = (size_t)g->T * g->R * g->G;
+  // One allocation and one upload for everything but the tables, which groups_upload_tables sends; every part
+  // starts on a 256-byte boundary.
+  size_t bytes = 0;
+  auto part = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) & ~size_t(255);
+    return at;
+  };
+  const size_t o_perm = part(g->K_pad * sizeof(int16_t)), o_head = part(quant_head_bytes(g->C, g->K_pad));
+  const size_t o_row = part(g->P * sizeof(int32_t)), o_col = part(g->C * sizeof(int32_t)), upload = bytes;
+  const size_t o_tab = part(3 * tn * sizeof(float)), o_cell = part(2 * (size_t)g->R * g->G * sizeof(int));
+  std::vector<unsigned char> h(upload, 0);
+  int16_t* perm16 = reinterpret_cast<int16_t*>(h.data() + o_perm);
+  int16_t* pos = reinterpret_cast<int16_t*>(h.data() + o_head);
+  uint8_t* cg = h.data() + o_head + g->C * 2;
+  uint16_t* pm = reinterpret_cast<uint16_t*>(h.data() + o_head + quant_head_pm_offset(g->C, g->K_pad));
+  for (int p = 0; p < g->K_pad; ++p) {
+    perm16[p] = (int16_t)g->perm[p];
+    if (g->perm[p] >= 0) pos[g->perm[p]] = (int16_t)p;
+    else pm[p >> 4] |= (uint16_t)(1u << (p & 15));
+  }
   for (int k = 0; k < g->G; ++k)
     for (int p = g->group_off[k]; p < g->group_off[k + 1]; p += 16) cg[p / 16] = (uint8_t)k;
-  const size_t tn = (size_t)g->T * g->R * g->G;
+  std::memcpy(h.data() + o_row, g->row_group.data(), g->P * sizeof(int32_t));
+  std::memcpy(h.data() + o_col, g->col_group.data(), g->C * sizeof(int32_t));
   DGQ_CUDA_OK(cudaGetDevice(&g->device));
-  DGQ_CUDA_OK(cudaMalloc(&g->d_perm, g->K_pad * sizeof(int16_t)));
-  DGQ_CUDA_OK(cudaMalloc(&g->d_chunk_group, cg.size()));
-  DGQ_CUDA_OK(cudaMalloc(&g->d_row_group, g->P * sizeof(int32_t)));
-  DGQ_CUDA_OK(cudaMalloc(&g->d_col_group, g->C * sizeof(int32_t)));
-  DGQ_CUDA_OK(cudaMalloc(&g->d_scale, tn * sizeof(float)));
-  DGQ_CUDA_OK(cudaMalloc(&g->d_inv_scale, tn * sizeof(float)));
-  DGQ_CUDA_OK(cudaMalloc(&g->d_zp, tn * sizeof(int32_t)));
-  DGQ_CUDA_OK(cudaMemcpy(g->d_perm, perm16.data(), g->K_pad * sizeof(int16_t), cudaMemcpyHostToDevice));
-  DGQ_CUDA_OK(cudaMemcpy(g->d_chunk_group, cg.data(), cg.size(), cudaMemcpyHostToDevice));
-  {
-    std::vector<uint8_t> head(quant_head_bytes(g->C, g->K_pad), 0);
-    int16_t* pos = reinterpret_cast<int16_t*>(head.data());
-    uint16_t* pm = reinterpret_cast<uint16_t*>(head.data() + quant_head_pm_offset(g->C, g->K_pad));
-    for (int p = 0; p < g->K_pad; ++p) {
-      if (g->perm[p] >= 0) pos[g->perm[p]] = (int16_t)p;
-      else pm[p >> 4] |= (uint16_t)(1u << (p & 15));
-    }
-    std::memcpy(head.data() + g->C * 2, cg.data(), cg.size());
-    DGQ_CUDA_OK(cudaMalloc(&g->d_quant_head, head.size()));
-    DGQ_CUDA_OK(cudaMemcpy(g->d_quant_head, head.data(), head.size(), cudaMemcpyHostToDevice));
-  }
-  DGQ_CUDA_OK(cudaMemcpy(g->d_row_group, g->row_group.data(), g->P * sizeof(int32_t), cudaMemcpyHostToDevice));
-  DGQ_CUDA_OK(cudaMemcpy(g->d_col_group, g->col_group.data(), g->C * sizeof(int32_t), cudaMemcpyHostToDevice));
+  DGQ_CUDA_OK(pool_alloc(reinterpret_cast<void**>(&g->d_slab), bytes, stream));
+  g->d_perm = reinterpret_cast<int16_t*>(g->d_slab + o_perm);
+  g->d_quant_head = g->d_slab + o_head;
+  g->d_row_group = reinterpret_cast<int32_t*>(g->d_slab + o_row);
+  g->d_col_group = reinterpret_cast<int32_t*>(g->d_slab + o_col);
+  g->d_scale = reinterpret_cast<float*>(g->d_slab + o_tab);
+  g->d_inv_scale = g->d_scale + tn;
+  g->d_zp = reinterpret_cast<int32_t*>(g->d_inv_scale + tn);
+  g->d_cell = reinterpret_cast<int*>(g->d_slab + o_cell);
+  DGQ_CUDA_OK(cudaMemcpyAsync(g->d_slab, h.data(), upload, cudaMemcpyHostToDevice, stream));
+  DGQ_CUDA_OK(cudaStreamSynchronize(stream));
   return DGQ_OK;
 }
 
-static dgq_status groups_upload_tables(dgq_groups* g) {
+static dgq_status groups_upload_tables(dgq_groups* g, cudaStream_t stream) {
   const size_t tn = (size_t)g->T * g->R * g->G;
-  DGQ_CUDA_OK(cudaMemcpy(g->d_scale, g->scale.data(), tn * sizeof(float), cudaMemcpyHostToDevice));
-  DGQ_CUDA_OK(cudaMemcpy(g->d_inv_scale, g->inv_scale.data(), tn * sizeof(float), cudaMemcpyHostToDevice));
-  DGQ_CUDA_OK(cudaMemcpy(g->d_zp, g->zp.data(), tn * sizeof(int32_t), cudaMemcpyHostToDevice));
+  std::vector<float> h(3 * tn);
+  std::copy(g->scale.begin(), g->scale.end(), h.begin());
+  std::copy(g->inv_scale.begin(), g->inv_scale.end(), h.begin() + tn);
+  std::memcpy(h.data() + 2 * tn, g->zp.data(), tn * sizeof(int32_t));
+  DGQ_CUDA_OK(cudaMemcpyAsync(g->d_scale, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, stream));
+  DGQ_CUDA_OK(cudaStreamSynchronize(stream));
   return DGQ_OK;
-}
-
-static std::vector<float> fetch_ordered(const int* d, int n, dgq_status* st) {
-  std::vector<int> h(n);
-  std::vector<float> f(n);
-  if (cudaMemcpy(h.data(), d, n * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) *st = DGQ_ERR_CUDA;
-  for (int i = 0; i < n; ++i) f[i] = ordered_to_float(h[i]);
-  return f;
 }
 
 }  // namespace dgq
@@ -335,32 +391,34 @@ extern "C" dgq_status dgq_calibrate_groups(const dgq_calib_config* cfg, const vo
   if (!fresh && (g->C != C || g->P != P || g->T != cfg->n_timesteps || g->bits != cfg->act_bits))
     return DGQ_ERR_INVALID_ARG;
 
-  const int rows_per_block = 128;
-  const int n_blocks = (int)((n_rows + rows_per_block - 1) / rows_per_block);
+  const unsigned n_blocks = (unsigned)((n_rows + CAL_ROWS - 1) / CAL_ROWS);
   dgq_status st = DGQ_OK;
+  std::vector<double> cmin, cmax, pmin, pmax;  // (fresh only) ranges of the channels and of the pixel positions
 
   if (fresh) {
-    int* d_ext = nullptr;  // ch_min[C], ch_max[C], px_min[P], px_max[P]
-    const int n_ext = 2 * C + 2 * P;
-    DGQ_CUDA_OK(cudaMalloc(&d_ext, n_ext * sizeof(int)));
-    int *ch_min = d_ext, *ch_max = d_ext + C, *px_min = d_ext + 2 * C, *px_max = d_ext + 2 * C + P;
-    fill_int_kernel<<<(C + 255) / 256, 256, 0, stream>>>(ch_min, C, INT_MAX);
-    fill_int_kernel<<<(C + 255) / 256, 256, 0, stream>>>(ch_max, C, INT_MIN);
-    fill_int_kernel<<<(P + 255) / 256, 256, 0, stream>>>(px_min, P, INT_MAX);
-    fill_int_kernel<<<(P + 255) / 256, 256, 0, stream>>>(px_max, P, INT_MIN);
-    channel_extrema_kernel<<<n_blocks, 256, 0, stream>>>(X, n_rows, C, ld, rows_per_block, ch_min, ch_max);
+    int* d_ext = nullptr;  // minima of the C channels and P pixels, then their maxima
+    const int n_ext = C + P;
+    DGQ_CUDA_OK(pool_alloc(reinterpret_cast<void**>(&d_ext), 2 * (size_t)n_ext * sizeof(int), stream));
+    fill_extrema_kernel<<<(2 * n_ext + 255) / 256, 256, 0, stream>>>(d_ext, n_ext);
+    channel_extrema_kernel<<<n_blocks, CAL_THREADS, 0, stream>>>(X, n_rows, C, ld, d_ext, d_ext + n_ext);
     const int pb = (int)std::min<int64_t>((n_rows + 7) / 8, 148 * 8);
-    pixel_extrema_kernel<<<pb, 256, 0, stream>>>(X, n_rows, C, ld, P, px_min, px_max);
-    g_launches += 6;
-    if (cudaStreamSynchronize(stream) != cudaSuccess) {
-      cudaFree(d_ext);
-      return DGQ_ERR_CUDA;
-    }
-    std::vector<float> ext = fetch_ordered(d_ext, n_ext, &st);
-    cudaFree(d_ext);
+    pixel_extrema_kernel<<<pb, 256, 0, stream>>>(X, n_rows, C, ld, P, d_ext + C, d_ext + n_ext + C);
+    g_launches += 3;
+    std::vector<int> ext(2 * (size_t)n_ext);
+    if (cudaMemcpyAsync(ext.data(), d_ext, ext.size() * sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+        cudaStreamSynchronize(stream) != cudaSuccess)
+      st = DGQ_ERR_CUDA;
+    cudaFreeAsync(d_ext, stream);
     if (st != DGQ_OK) return st;
-    std::vector<double> cmin(ext.begin(), ext.begin() + C), cmax(ext.begin() + C, ext.begin() + 2 * C);
-    std::vector<double> pmin(ext.begin() + 2 * C, ext.begin() + 2 * C + P), pmax(ext.begin() + 2 * C + P, ext.end());
+    auto range = [&](int first, int n) {
+      std::vector<double> v(n);
+      for (int i = 0; i < n; ++i) v[i] = ordered_to_float(ext[first + i]);
+      return v;
+    };
+    cmin = range(0, C);
+    pmin = range(C, P);
+    cmax = range(n_ext, C);
+    pmax = range(n_ext + C, P);
     // Eq. 4
     auto spread = [](const std::vector<double>& v) {
       return *std::max_element(v.begin(), v.end()) - *std::min_element(v.begin(), v.end());
@@ -393,7 +451,7 @@ extern "C" dgq_status dgq_calibrate_groups(const dgq_calib_config* cfg, const vo
     g->inv_scale.assign(tn, 1.0f);
     g->zp.assign(tn, 0);
     g->filled.assign(g->T, 0);
-    st = groups_build_layout(g);
+    st = groups_build_layout(g, stream);
     if (st != DGQ_OK) {
       groups_free_device(g);
       delete g;
@@ -403,39 +461,43 @@ extern "C" dgq_status dgq_calibrate_groups(const dgq_calib_config* cfg, const vo
 
   // Eq. 6 per cell from this timestep's rows
   const int n_cells = g->R * g->G;
-  int* d_cell = nullptr;
-  if (cudaMalloc(&d_cell, 2 * n_cells * sizeof(int)) != cudaSuccess) st = DGQ_ERR_CUDA;
-  if (st == DGQ_OK) {
-    fill_int_kernel<<<(n_cells + 255) / 256, 256, 0, stream>>>(d_cell, n_cells, INT_MAX);
-    fill_int_kernel<<<(n_cells + 255) / 256, 256, 0, stream>>>(d_cell + n_cells, n_cells, INT_MIN);
-    cell_extrema_kernel<<<n_blocks, 256, 0, stream>>>(X, n_rows, C, ld, P, rows_per_block, g->d_row_group,
-                                                      g->d_col_group, g->G, d_cell, d_cell + n_cells);
-    g_launches += 3;
-    if (cudaStreamSynchronize(stream) != cudaSuccess) st = DGQ_ERR_CUDA;
-  }
-  if (st == DGQ_OK) {
-    std::vector<int> h(2 * n_cells);
-    if (cudaMemcpy(h.data(), d_cell, 2 * n_cells * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-      st = DGQ_ERR_CUDA;
-    for (int i = 0; i < n_cells && st == DGQ_OK; ++i) {
-      float lo = 0.f, hi = 0.f;
-      if (h[i] != INT_MAX) {  // an empty cell keeps the range (0, 0)
-        lo = ordered_to_float(h[i]);
-        hi = ordered_to_float(h[n_cells + i]);
-      }
-      float s, inv_s;
-      int Z;
-      group_params(lo, hi, g->bits, s, inv_s, Z);
-      const size_t o = (size_t)timestep * n_cells + i;
-      g->scale[o] = s;
-      g->inv_scale[o] = inv_s;
-      g->zp[o] = Z;
+  std::vector<int> cell(2 * (size_t)n_cells, INT_MIN);  // minima, then maxima, as ordered integers
+  if (fresh && (g->R == 1 || g->G == 1)) {
+    // grouped along one dimension: a cell's range is that of its channels (or pixel positions), which are at hand
+    std::fill(cell.begin(), cell.begin() + n_cells, INT_MAX);
+    const bool by_channel = g->R == 1;
+    const std::vector<int32_t>& group = by_channel ? g->col_group : g->row_group;
+    const std::vector<double>&lo = by_channel ? cmin : pmin, &hi = by_channel ? cmax : pmax;
+    for (size_t i = 0; i < group.size(); ++i) {
+      cell[group[i]] = std::min(cell[group[i]], float_to_ordered((float)lo[i]));
+      cell[n_cells + group[i]] = std::max(cell[n_cells + group[i]], float_to_ordered((float)hi[i]));
     }
+  } else {
+    fill_extrema_kernel<<<(2 * n_cells + 255) / 256, 256, 0, stream>>>(g->d_cell, n_cells);
+    cell_extrema_kernel<<<n_blocks, CAL_THREADS, 2 * n_cells * sizeof(int), stream>>>(
+        X, n_rows, C, ld, P, g->d_row_group, g->d_col_group, g->G, n_cells, g->d_cell, g->d_cell + n_cells);
+    g_launches += 2;
+    if (cudaMemcpyAsync(cell.data(), g->d_cell, cell.size() * sizeof(int), cudaMemcpyDeviceToHost, stream) != cudaSuccess ||
+        cudaStreamSynchronize(stream) != cudaSuccess)
+      st = DGQ_ERR_CUDA;
   }
-  cudaFree(d_cell);
+  for (int i = 0; i < n_cells && st == DGQ_OK; ++i) {
+    float lo = 0.f, hi = 0.f;
+    if (cell[i] != INT_MAX) {  // an empty cell keeps the range (0, 0)
+      lo = ordered_to_float(cell[i]);
+      hi = ordered_to_float(cell[n_cells + i]);
+    }
+    float s, inv_s;
+    int Z;
+    group_params(lo, hi, g->bits, s, inv_s, Z);
+    const size_t o = (size_t)timestep * n_cells + i;
+    g->scale[o] = s;
+    g->inv_scale[o] = inv_s;
+    g->zp[o] = Z;
+  }
   if (st == DGQ_OK) {
     g->filled[timestep] = 1;
-    st = groups_upload_tables(g);
+    st = groups_upload_tables(g, stream);
   }
   if (st != DGQ_OK) {
     if (fresh) {
@@ -483,8 +545,8 @@ extern "C" dgq_status dgq_groups_from_host(int C, int P, int act_bits, int G, in
     g->inv_scale[i] = inv;
   }
   g->filled.assign(T, 1);
-  dgq_status st = groups_build_layout(g);
-  if (st == DGQ_OK) st = groups_upload_tables(g);
+  dgq_status st = groups_build_layout(g, nullptr);
+  if (st == DGQ_OK) st = groups_upload_tables(g, nullptr);
   if (st != DGQ_OK) {
     groups_free_device(g);
     delete g;

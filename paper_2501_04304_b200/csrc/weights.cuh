@@ -1,6 +1,11 @@
-// Offline weight preparation: per-out-channel symmetric round-to-nearest codes, permuted and
-// padded to the layer's group-contiguous code layout, int4 packed two per byte, plus the
-// per-group column sums the de-quantizer needs.  Runs on the host; not a timed path.
+// Weight preparation: per-out-channel symmetric round-to-nearest codes, permuted and padded to the layer's
+// group-contiguous code layout, int4 packed two per byte, plus the per-group column sums the de-quantizer needs.
+//
+// One kernel, one thread block per output row: the row's absolute maximum, its codes (kept in shared memory), the
+// sums of every group and the padded row are one pass over the row's fp16 weights.  What a caller waits for is
+// then the allocation, one launch and one small copy back (scales and the mask of residual groups); the
+// host loops this replaces took 30 ms for 640 -> 5120.  The object keeps no host copy of the codes: an export
+// reads them back out of the padded rows.
 #pragma once
 
 #include "groups.cuh"
@@ -10,38 +15,191 @@ struct dgq_weight {
   int N_pad = 0;                 // N rounded up to a multiple of 256 (rows beyond N are zero)
   int Kt = 0;                    // length of the GEMM reduction in padded positions (multiple of 32)
   std::vector<int32_t> seg_end;  // [G] end of every group's segment, in 32-position atoms
-  std::vector<int8_t> wq;        // host codes, original order [N][K]
   std::vector<float> sw;         // host scales [N]
+  unsigned char* d_slab = nullptr;  // all device arrays below
   int8_t* d_w = nullptr;         // 8-bit: [N_pad][Kt] s8; 4-bit: [N_pad][Kt/2] packed
   float* d_sw = nullptr;         // [N_pad]; 4-bit: sw / 16 (the unpacked codes carry a factor 16)
   float* d_wsum = nullptr;       // [G][N_pad] column sums per group as fp32 (exact); 4-bit: x 16
   float* d_wres = nullptr;       // [G][N_pad] part of wsum the padding positions could not absorb
+  int2* d_chan = nullptr;        // [C] reduction position of every channel's first tap, distance between its taps
   uint32_t res_mask = 0;         // bit g set: group g has a non-zero entry in d_wres
 };
 
 namespace dgq {
 
-// 4-bit storage: every 8 consecutive positions k0..k0+7 share one 32-bit word whose byte i holds
-// code k0+i in its low nibble and code k0+4+i in its high nibble.  In the kernel
-// (word << 4) & 0xF0F0F0F0 and word & 0xF0F0F0F0 are then bytes k0..k0+3 and k0+4..k0+7, each
-// equal to 16 x the signed code, with no per-byte sign extension.
-static void pack_int4_words(const int8_t* row, int Kt, uint8_t* out) {
-  for (int k0 = 0; k0 < Kt; k0 += 8)
-    for (int i = 0; i < 4; ++i)
-      out[k0 / 2 + i] = (uint8_t)((row[k0 + i] & 0x0F) | ((row[k0 + 4 + i] & 0x0F) << 4));
+constexpr int WP_THREADS = 256;
+
+struct WeightArgs {
+  const __half* W;       // [N][K], or null when the codes are given
+  const int8_t* wq;      // [N][K] given codes
+  const float* sw_in;    // [N] their scales
+  int N, K, C, G, N_pad, Kt, K_pad, taps, qmax, four_bit;
+  const int16_t* perm;   // [K_pad] channel of every padded position, -1 = padding
+  int group_off[DGQ_MAX_GROUPS + 1];  // first padded position of every group
+  uint8_t* w;            // outputs, see dgq_weight
+  float *sw, *wsum, *wres;
+  float* sw_out;         // [N] scales as the caller sees them
+  unsigned int* res_mask;
+};
+
+// Eight neighbouring reduction positions (always of one group) of one row: their codes, padding as 0.  The
+// reduction is group-major, inside a group tap-major, then the group's padded positions.
+__device__ __forceinline__ int weight_codes8(const WeightArgs& a, const int8_t* row, int pos, int (&c)[8], int& first_pad) {
+  int g = 0;
+  while (pos >= a.taps * a.group_off[g + 1]) ++g;
+  const int len = a.group_off[g + 1] - a.group_off[g], local = pos - a.taps * a.group_off[g];
+  const int tap = local / len, p0 = a.group_off[g] + local - tap * len;
+  const int8_t* src = row + tap * a.C;
+  const uint4 pv = __ldg(reinterpret_cast<const uint4*>(a.perm + p0));
+  const int16_t* p = reinterpret_cast<const int16_t*>(&pv);
+  first_pad = 8;
+#pragma unroll
+  for (int i = 7; i >= 0; --i) {
+    c[i] = p[i] >= 0 ? src[p[i]] : 0;
+    if (p[i] < 0) first_pad = i;  // padding follows a group's members
+  }
+  return g;
 }
 
-static dgq_status weight_build(const dgq_groups* g, const int8_t* wq, const float* sw, int N, int K, int w_bits,
-                               const dgq_conv_desc* conv, dgq_weight** out) {
-  if (!g || !wq || !sw || !out || N <= 0) return DGQ_ERR_INVALID_ARG;
-  if (w_bits != 8 && w_bits != 4) return DGQ_ERR_INVALID_ARG;
+__global__ void __launch_bounds__(WP_THREADS) weight_rows_kernel(const __grid_constant__ WeightArgs a) {
+  extern __shared__ int8_t row_s[];  // [K] codes of the row
+  __shared__ float red[WP_THREADS / 32];
+  __shared__ int sum_s[DGQ_MAX_GROUPS];
+  const int o = blockIdx.x;
+  const int row_bytes = a.four_bit ? a.Kt / 2 : a.Kt;
+  uint8_t* out = a.w + (size_t)o * row_bytes;
+  if (o >= a.N) {
+    for (int i = threadIdx.x; i < row_bytes / 16; i += WP_THREADS) reinterpret_cast<uint4*>(out)[i] = make_uint4(0, 0, 0, 0);
+    for (int g = threadIdx.x; g < a.G; g += WP_THREADS) a.wsum[(size_t)g * a.N_pad + o] = a.wres[(size_t)g * a.N_pad + o] = 0.f;
+    if (threadIdx.x == 0) a.sw[o] = 0.f;
+    return;
+  }
+  const float unit = a.four_bit ? 16.f : 1.f;
+  if (threadIdx.x < a.G) sum_s[threadIdx.x] = 0;
+  float s;
+  if (a.W) {
+    // fp32 sequence: sw = absmax / qmax, inv = 1 / sw, code = clamp(rint(w * inv), -qmax, qmax)
+    const __half* w = a.W + (size_t)o * a.K;
+    const float qmax = (float)a.qmax;
+    float amax = 0.f;
+    for (int k = threadIdx.x; k < a.K; k += WP_THREADS) amax = fmaxf(amax, fabsf(__half2float(__ldg(w + k))));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = amax;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < WP_THREADS / 32; ++i) amax = fmaxf(amax, red[i]);
+    s = amax > 0.f ? __fdiv_rn(amax, qmax) : 1.0f;
+    const float inv = __fdiv_rn(1.0f, s);
+    for (int k = threadIdx.x; k < a.K; k += WP_THREADS) {
+      const float r = rintf(__fmul_rn(__half2float(__ldg(w + k)), inv));
+      row_s[k] = (int8_t)(int)fminf(fmaxf(r, -qmax), qmax);
+    }
+  } else {
+    s = __ldg(a.sw_in + o);
+    for (int k = threadIdx.x; k < a.K; k += WP_THREADS) row_s[k] = __ldg(a.wq + (size_t)o * a.K + k);
+  }
+  if (threadIdx.x == 0) {
+    a.sw[o] = __fdiv_rn(s, unit);
+    a.sw_out[o] = s;
+  }
+  __syncthreads();
+  int c[8], first_pad;
+  for (int pos = threadIdx.x * 8; pos < a.Kt; pos += WP_THREADS * 8) {
+    const int g = weight_codes8(a, row_s, pos, c, first_pad);
+    if (first_pad > 0) atomicAdd(&sum_s[g], ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7])));
+  }
+  __syncthreads();
+  // Linear layers: -sum of a group is spread over its padding positions (whose activation code is the zero-point
+  // Z), so that acc + Z * (-sum) = acc - Z * wsum comes out of the integer product.  What does not fit in the
+  // available positions stays in `wres` for the epilogue.  The conv's zero-centred codes have no zero-point term.
+  for (int pos = threadIdx.x * 8; pos < a.Kt; pos += WP_THREADS * 8) {
+    const int g = weight_codes8(a, row_s, pos, c, first_pad);
+    if (a.taps == 1 && first_pad < 8) {
+      // the padding starts somewhere in front of this word: count the positions it fills up to here
+      int lo = a.group_off[g], hi = pos + first_pad;  // first padding position of the group lies in [lo, hi]
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(a.perm + mid) < 0) hi = mid;
+        else lo = mid + 1;
+      }
+      const int neg = -sum_s[g], sign = neg < 0 ? -1 : 1;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i >= first_pad) c[i] = sign * min(a.qmax, max(0, sign * neg - (pos + i - lo) * a.qmax));
+    }
+    if (a.four_bit) {
+      // Word of 8 positions: byte i holds code i in its low nibble and code 4 + i in its high nibble.  In the GEMM
+      // (word << 4) & 0xF0F0F0F0 and word & 0xF0F0F0F0 are then bytes 0..3 and 4..7, each equal to 16 x the signed
+      // code, with no per-byte sign extension.
+      uint32_t v = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v |= (uint32_t)((c[i] & 0xF) | ((c[4 + i] & 0xF) << 4)) << (8 * i);
+      *reinterpret_cast<uint32_t*>(out + pos / 2) = v;
+    } else {
+      uint2 v = make_uint2(0, 0);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        v.x |= (uint32_t)(c[i] & 0xFF) << (8 * i);
+        v.y |= (uint32_t)(c[4 + i] & 0xFF) << (8 * i);
+      }
+      *reinterpret_cast<uint2*>(out + pos) = v;
+    }
+  }
+  for (int g = threadIdx.x; g < a.G; g += WP_THREADS) {
+    const int sum = sum_s[g];
+    int members = 0, lo = a.group_off[g], hi = a.group_off[g + 1];
+    const int end = hi;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (__ldg(a.perm + mid) < 0) hi = mid;
+      else lo = mid + 1;
+    }
+    members = lo;
+    const int room = (end - members) * a.qmax;
+    const int left = sum < 0 ? min(0, sum + room) : max(0, sum - room);
+    const int res = a.taps == 1 ? left : sum;
+    a.wsum[(size_t)g * a.N_pad + o] = (float)sum * unit;
+    a.wres[(size_t)g * a.N_pad + o] = (float)res * unit;
+    if (res != 0 && a.taps == 1) atomicOr(a.res_mask, 1u << g);
+  }
+}
+
+// Codes in original channel order from the padded rows.
+__global__ void weight_unpermute_kernel(const uint8_t* __restrict__ w, const int2* __restrict__ chan, int K, int C, int Kt,
+                                        int four_bit, int8_t* __restrict__ out) {
+  const uint8_t* row = w + (size_t)blockIdx.x * (four_bit ? Kt / 2 : Kt);
+  for (int k = threadIdx.x; k < K; k += blockDim.x) {
+    const int tap = k / C;
+    const int2 ch = __ldg(chan + (k - tap * C));
+    const int pos = ch.x + tap * ch.y;
+    int v;
+    if (four_bit) {
+      const int b = row[pos / 8 * 4 + (pos & 3)];
+      v = (int)((uint32_t)((pos & 4) ? b >> 4 : b) << 28) >> 28;
+    } else {
+      v = (int8_t)row[pos];
+    }
+    out[(size_t)blockIdx.x * K + k] = (int8_t)v;
+  }
+}
+
+// Device arrays of a weight in one allocation, filled by weight_rows_kernel from fp16 weights `W` (device) or from
+// codes `wq` and scales `sw` (host), whichever is given.
+static dgq_status weight_build(const dgq_groups* g, const __half* W, const int8_t* wq, const float* sw, int N, int K, int w_bits,
+                               const dgq_conv_desc* conv, dgq_weight** out, cudaStream_t stream) {
   const int taps = conv ? 9 : 1;
   if (conv && (conv->c != g->C || conv->n <= 0 || conv->h <= 0 || conv->w <= 0)) return DGQ_ERR_INVALID_ARG;
   if (K != taps * g->C) return DGQ_ERR_INVALID_ARG;
   if ((N % 8) != 0) return DGQ_ERR_UNSUPPORTED;
-  const int qmax = (1 << (w_bits - 1)) - 1;
-  for (size_t i = 0; i < (size_t)N * K; ++i)
-    if (wq[i] < -qmax || wq[i] > qmax) return DGQ_ERR_INVALID_ARG;
+  WeightArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.qmax = (1 << (w_bits - 1)) - 1;
+  if (wq)
+    for (size_t i = 0; i < (size_t)N * K; ++i)
+      if (wq[i] < -a.qmax || wq[i] > a.qmax) return DGQ_ERR_INVALID_ARG;
+  // accumulator bound: |code| <= 255, |weight| <= 127 (4-bit: 7 * 16)
+  if ((int64_t)taps * g->K_pad * 255 * 127 >= ((int64_t)1 << 31)) return DGQ_ERR_UNSUPPORTED;
   dgq_weight* w = new dgq_weight();
   w->N = N;
   w->K = K;
@@ -51,75 +209,81 @@ static dgq_status weight_build(const dgq_groups* g, const int8_t* wq, const floa
   w->is_conv = conv ? 1 : 0;
   w->N_pad = (N + 255) / 256 * 256;
   w->Kt = taps * g->K_pad;
-  // accumulator bound: |code| <= 255, |weight| <= 127 (4-bit: 7 * 16)
-  if ((int64_t)w->Kt * 255 * 127 >= ((int64_t)1 << 31)) {
-    delete w;
-    return DGQ_ERR_UNSUPPORTED;
-  }
-  w->wq.assign(wq, wq + (size_t)N * K);
-  w->sw.assign(sw, sw + N);
   w->seg_end.resize(g->G);
-  // GEMM reduction order: group-major; inside a group tap-major (conv), then the group's padded positions
-  std::vector<int8_t> Wp((size_t)w->N_pad * w->Kt, 0);
-  std::vector<float> wsum((size_t)g->G * w->N_pad, 0.f), wres((size_t)g->G * w->N_pad, 0.f);
-  const float unit = (w_bits == 4) ? 16.f : 1.f;
-  int pos = 0;
-  for (int k = 0; k < g->G; ++k) {
-    const int p0 = g->group_off[k], p1 = g->group_off[k + 1];
-    for (int t = 0; t < taps; ++t)
-      for (int p = p0; p < p1; ++p, ++pos) {
-        const int c = g->perm[p];
-        if (c < 0) continue;
-        for (int o = 0; o < N; ++o) Wp[(size_t)o * w->Kt + pos] = wq[(size_t)o * K + t * g->C + c];
-      }
-    w->seg_end[k] = pos / DGQ_K_ATOM;
-    const int seg0 = pos - taps * (p1 - p0);  // first reduction position of this group
-    for (int o = 0; o < N; ++o) {
-      int64_t sum = 0;
-      for (int c = 0; c < g->C; ++c)
-        if (g->col_group[c] == k)
-          for (int t = 0; t < taps; ++t) sum += wq[(size_t)o * K + t * g->C + c];
-      wsum[(size_t)k * w->N_pad + o] = (float)sum * unit;
-      // Linear layers: spread -sum over the group's padding positions (whose activation code is the
-      // zero-point Z), so that acc + Z * (-sum) = acc - Z * wsum comes out of the integer product.
-      // What does not fit in the available positions stays in `wres` for the epilogue.
-      int64_t rem = conv ? 0 : -sum;
-      if (!conv)
-        for (int p = p0; p < p1 && rem != 0; ++p)
-          if (g->perm[p] < 0) {
-            const int64_t v = std::max<int64_t>(-qmax, std::min<int64_t>(qmax, rem));
-            Wp[(size_t)o * w->Kt + seg0 + (p - p0)] = (int8_t)v;
-            rem -= v;
-          }
-      const int64_t res = conv ? sum : -rem;  // conv uses zero-centred codes: no zero-point term at all
-      wres[(size_t)k * w->N_pad + o] = (float)res * unit;
-      if (res != 0 && !conv) w->res_mask |= 1u << k;
+  for (int k = 0; k < g->G; ++k) w->seg_end[k] = taps * g->group_off[k + 1] / DGQ_K_ATOM;
+
+  size_t bytes = 0;
+  auto part = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) & ~size_t(255);
+    return at;
+  };
+  const size_t w_bytes = (size_t)w->N_pad * w->Kt / (w_bits == 4 ? 2 : 1), per_group = (size_t)g->G * w->N_pad * sizeof(float);
+  const size_t o_w = part(w_bytes), o_sw = part(w->N_pad * sizeof(float)), o_wsum = part(per_group), o_wres = part(per_group);
+  const size_t o_chan = part(g->C * sizeof(int2)), o_back = part((size_t)(N + 1) * sizeof(float));  // scales, then the mask
+  const size_t o_codes = bytes;  // given codes and scales, for the duration of the call
+  int8_t* d_codes = nullptr;
+  dgq_status st = DGQ_OK;
+  auto ok = [&](cudaError_t e) {
+    if (st == DGQ_OK && e != cudaSuccess) st = DGQ_ERR_CUDA;
+    return st == DGQ_OK;
+  };
+  if (ok(pool_alloc((void**)&w->d_slab, o_codes, stream)) &&
+      (!wq || ok(pool_alloc((void**)&d_codes, (size_t)N * K + 4 * (size_t)N + 16, stream)))) {
+    w->d_w = reinterpret_cast<int8_t*>(w->d_slab + o_w);
+    w->d_sw = reinterpret_cast<float*>(w->d_slab + o_sw);
+    w->d_wsum = reinterpret_cast<float*>(w->d_slab + o_wsum);
+    w->d_wres = reinterpret_cast<float*>(w->d_slab + o_wres);
+    w->d_chan = reinterpret_cast<int2*>(w->d_slab + o_chan);
+    float* back = reinterpret_cast<float*>(w->d_slab + o_back);
+    std::vector<int2> chan(g->C);
+    for (int k = 0; k < g->G; ++k)
+      for (int p = g->group_off[k]; p < g->group_off[k + 1]; ++p)
+        if (g->perm[p] >= 0)
+          chan[g->perm[p]] = make_int2((taps - 1) * g->group_off[k] + p, g->group_off[k + 1] - g->group_off[k]);
+    ok(cudaMemcpyAsync(w->d_chan, chan.data(), chan.size() * sizeof(int2), cudaMemcpyHostToDevice, stream));
+    if (wq) {
+      a.wq = d_codes;
+      a.sw_in = reinterpret_cast<const float*>(d_codes + (((size_t)N * K + 15) & ~size_t(15)));
+      ok(cudaMemcpyAsync(d_codes, wq, (size_t)N * K, cudaMemcpyHostToDevice, stream));
+      ok(cudaMemcpyAsync(const_cast<float*>(a.sw_in), sw, N * sizeof(float), cudaMemcpyHostToDevice, stream));
+    }
+    ok(cudaMemsetAsync(back + N, 0, sizeof(float), stream));
+    a.W = W;
+    a.N = N;
+    a.K = K;
+    a.C = g->C;
+    a.G = g->G;
+    a.N_pad = w->N_pad;
+    a.Kt = w->Kt;
+    a.K_pad = g->K_pad;
+    a.taps = taps;
+    a.four_bit = w_bits == 4;
+    a.perm = g->d_perm;
+    std::copy(g->group_off.begin(), g->group_off.end(), a.group_off);
+    a.w = reinterpret_cast<uint8_t*>(w->d_w);
+    a.sw = w->d_sw;
+    a.wsum = w->d_wsum;
+    a.wres = w->d_wres;
+    a.sw_out = back;
+    a.res_mask = reinterpret_cast<unsigned int*>(back + N);
+    if (K > 40 * 1024)
+      ok(cudaFuncSetAttribute(weight_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 72 * 1024));
+    std::vector<float> host(N + 1);
+    if (st == DGQ_OK) {
+      weight_rows_kernel<<<w->N_pad, WP_THREADS, (size_t)K, stream>>>(a);
+      g_launches += 1;
+      ok(cudaGetLastError());
+      ok(cudaMemcpyAsync(host.data(), back, host.size() * sizeof(float), cudaMemcpyDeviceToHost, stream));
+      ok(cudaStreamSynchronize(stream));
+      std::memcpy(&w->res_mask, &host[N], sizeof(w->res_mask));
+      host.resize(N);
+      w->sw = std::move(host);
     }
   }
-  std::vector<float> swp(w->N_pad, 0.f);
-  for (int o = 0; o < N; ++o) swp[o] = sw[o] / unit;
-  dgq_status st = DGQ_OK;
-  auto up = [&](void** d, const void* h, size_t bytes) {
-    if (st != DGQ_OK) return;
-    if (cudaMalloc(d, bytes) != cudaSuccess || cudaMemcpy(*d, h, bytes, cudaMemcpyHostToDevice) != cudaSuccess)
-      st = DGQ_ERR_CUDA;
-  };
-  if (w_bits == 8) {
-    up((void**)&w->d_w, Wp.data(), Wp.size());
-  } else {
-    std::vector<uint8_t> packed((size_t)w->N_pad * w->Kt / 2);
-    for (int o = 0; o < w->N_pad; ++o)
-      pack_int4_words(&Wp[(size_t)o * w->Kt], w->Kt, &packed[(size_t)o * w->Kt / 2]);
-    up((void**)&w->d_w, packed.data(), packed.size());
-  }
-  up((void**)&w->d_sw, swp.data(), swp.size() * sizeof(float));
-  up((void**)&w->d_wsum, wsum.data(), wsum.size() * sizeof(float));
-  up((void**)&w->d_wres, wres.data(), wres.size() * sizeof(float));
+  if (d_codes) cudaFreeAsync(d_codes, stream);
   if (st != DGQ_OK) {
-    cudaFree(w->d_w);
-    cudaFree(w->d_sw);
-    cudaFree(w->d_wsum);
-    cudaFree(w->d_wres);
+    pool_free(w->d_slab);
     delete w;
     return st;
   }
@@ -131,50 +295,36 @@ static dgq_status weight_build(const dgq_groups* g, const int8_t* wq, const floa
 
 extern "C" dgq_status dgq_weight_from_codes(const dgq_groups* g, const int8_t* wq, const float* sw, int N, int K,
                                             int w_bits, const dgq_conv_desc* conv, dgq_weight** out) {
-  return dgq::weight_build(g, wq, sw, N, K, w_bits, conv, out);
+  if (!g || !wq || !sw || !out || N <= 0) return DGQ_ERR_INVALID_ARG;
+  if (w_bits != 8 && w_bits != 4) return DGQ_ERR_INVALID_ARG;
+  return dgq::weight_build(g, nullptr, wq, sw, N, K, w_bits, conv, out, nullptr);
 }
 
 extern "C" dgq_status dgq_weight_prepare(const dgq_groups* g, const void* W, int N, int K, int w_bits,
                                          const dgq_conv_desc* conv, dgq_weight** out, void* stream) {
   if (!g || !W || !out || N <= 0 || K <= 0) return DGQ_ERR_INVALID_ARG;
   if (w_bits != 8 && w_bits != 4) return DGQ_ERR_INVALID_ARG;
-  std::vector<__half> h((size_t)N * K);
-  if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return DGQ_ERR_CUDA;
-  if (cudaMemcpy(h.data(), W, h.size() * sizeof(__half), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return DGQ_ERR_CUDA;
-  // fp32 sequence: sw = absmax / qmax, inv = 1 / sw, code = clamp(rint(w * inv), -qmax, qmax)
-  const float qmax = (float)((1 << (w_bits - 1)) - 1);
-  std::vector<int8_t> wq((size_t)N * K);
-  std::vector<float> sw(N);
-  for (int o = 0; o < N; ++o) {
-    float amax = 0.f;
-    for (int k = 0; k < K; ++k) amax = std::max(amax, std::fabs(__half2float(h[(size_t)o * K + k])));
-    volatile float s = amax > 0.f ? amax / qmax : 1.0f;
-    volatile float inv = 1.0f / s;
-    sw[o] = s;
-    for (int k = 0; k < K; ++k) {
-      volatile float t = __half2float(h[(size_t)o * K + k]) * inv;
-      float r = __builtin_rintf(t);
-      r = std::min(std::max(r, -qmax), qmax);
-      wq[(size_t)o * K + k] = (int8_t)r;
-    }
-  }
-  return dgq::weight_build(g, wq.data(), sw.data(), N, K, w_bits, conv, out);
+  return dgq::weight_build(g, (const __half*)W, nullptr, nullptr, N, K, w_bits, conv, out, (cudaStream_t)stream);
 }
 
 extern "C" dgq_status dgq_weight_destroy(dgq_weight* w) {
   if (!w) return DGQ_OK;
-  cudaFree(w->d_w);
-  cudaFree(w->d_sw);
-  cudaFree(w->d_wsum);
-  cudaFree(w->d_wres);
+  dgq::pool_free(w->d_slab);
   delete w;
   return DGQ_OK;
 }
 
 extern "C" dgq_status dgq_weight_export(const dgq_weight* w, int8_t* wq, float* sw) {
   if (!w) return DGQ_ERR_INVALID_ARG;
-  if (wq) std::copy(w->wq.begin(), w->wq.end(), wq);
+  if (wq) {
+    int8_t* d = nullptr;
+    DGQ_CUDA_OK(dgq::pool_alloc((void**)&d, (size_t)w->N * w->K, nullptr));
+    dgq::weight_unpermute_kernel<<<w->N, 256>>>((const uint8_t*)w->d_w, w->d_chan, w->K, w->C, w->Kt, w->w_bits == 4, d);
+    dgq::g_launches += 1;
+    const cudaError_t e = cudaMemcpy(wq, d, (size_t)w->N * w->K, cudaMemcpyDeviceToHost);
+    cudaFreeAsync(d, nullptr);
+    if (e != cudaSuccess) return DGQ_ERR_CUDA;
+  }
   if (sw) std::copy(w->sw.begin(), w->sw.end(), sw);
   return DGQ_OK;
 }

@@ -1,0 +1,63 @@
+"""GPU parity of the set-up kernels at the edges of their ranges: calibration reductions on ragged recordings and
+weight preparation on group sizes around the 32-position atom."""
+import numpy as np
+import pytest
+
+from oracle import calibration as oc
+from oracle import linear as ol
+from paper_2501_04304_b200 import synth
+from dgq_testlib import gpu, to_dev, oracle_grouping_matches, check_output
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("P,n,C,ld,dim,K", [
+    (1, 1, 8, 8, oc.DIM_CHANNEL, 2),          # one row, one vector
+    (31, 1, 13, 16, oc.DIM_BOTH, 3),          # a last vector of five columns, fewer rows than a block takes
+    (33, 3, 2056, 2064, oc.DIM_BOTH, 4),      # more vectors than threads, ragged blocks, row groups change inside one
+    (96, 1, 320, 320, oc.DIM_PIXEL, 8),
+])
+def test_calibration_edges(P, n, C, ld, dim, K):
+    torch, b = gpu()
+    X = synth.activations(31, 1, n, P, C)
+    X1 = synth.activations(31, 2, n, P, C)
+    buf = torch.zeros((n * P, ld), dtype=torch.float16, device="cuda")
+    gr = oc.calibrate(X, P, 8, K, dim_select=dim)
+    oc.fill_timestep(gr, X1, 1)
+    buf[:, :C] = to_dev(torch, X)
+    g = b.calibrate_groups(buf[:, :C], P, 8, K, dim, n_timesteps=2)
+    buf[:, :C] = to_dev(torch, X1)
+    b.calibrate_groups(buf[:, :C], P, 8, K, dim, n_timesteps=2, timestep=1, groups=g)
+    oracle_grouping_matches(gr, g.export())
+
+
+@pytest.mark.parametrize("w_bits", [8, 4])
+@pytest.mark.parametrize("sizes,N", [
+    ((8,), 8),                      # one word of members
+    ((24, 25, 1, 30), 16),          # padding that just fits the atom, spills into the next, fills one alone
+    ((32, 64, 7, 9), 264),          # whole atoms of padding, rows beyond N in the last tile
+    ((400, 8), 72),                 # sums that eight padding positions cannot absorb at 4 bits
+])
+def test_weight_layout_edges(sizes, N, w_bits):
+    torch, b = gpu()
+    C = sum(sizes)
+    rng = np.random.default_rng(C)
+    cg = rng.permutation(np.repeat(np.arange(len(sizes)), sizes)).astype(np.int32)
+    G, M = len(sizes), 40
+    scale = rng.uniform(0.01, 0.05, (1, 1, G)).astype(np.float32)
+    zp = rng.integers(100, 140, (1, 1, G)).astype(np.int32)
+    g = b.groups_from_host(C, 1, 8, cg, np.zeros(1, np.int32), scale, zp)
+    W = (rng.normal(0.01, 0.02, (N, C))).astype(np.float16)   # biased, so that a group's sum outgrows its padding
+    W[N - 1] = 0
+    wq, sw = ol.weight_rtn(W, w_bits)
+    w = b.weight_prepare(g, to_dev(torch, W), w_bits)
+    got, got_sw = w.export()
+    assert np.array_equal(got, wq) and np.array_equal(got_sw, sw)
+    w2 = b.weight_from_codes(g, wq, sw, w_bits)
+    X = rng.normal(0, 1, (M, C)).astype(np.float16)
+    codes = np.clip(np.rint(X.astype(np.float32) * (np.float32(1) / scale[0, 0, cg])) + zp[0, 0, cg], 0, 255).astype(np.int64)
+    Xq, _, _ = b.quantize_act(g, to_dev(torch, X))
+    Y, Y2 = b.linear(g, w, Xq), b.linear(g, w2, Xq)
+    assert torch.equal(Y, Y2) and b.device_status() == 0
+    s_rows, z_rows = np.broadcast_to(scale[0], (M, G)), np.broadcast_to(zp[0], (M, G))
+    check_output(Y, ol.group_linear(codes, s_rows, z_rows, cg, wq, sw, None))

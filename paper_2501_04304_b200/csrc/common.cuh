@@ -73,6 +73,18 @@ static inline void pool_free(void* p) {
   if (at.device != dev) cudaSetDevice(dev);
 }
 
+// Multiprocessors of the current device, asked once.
+static inline cudaError_t sm_count(int* n) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && (*n = known[dev].load()) != 0) return cudaSuccess;
+  if ((e = cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if (dev < 64) known[dev].store(*n);
+  return cudaSuccess;
+}
+
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // ------------------------------------------------------------------ ordered-int encoding of floats

@@ -19,7 +19,7 @@ struct dgq_groups {
   // device copies, one allocation
   unsigned char* d_slab = nullptr;
   int16_t* d_perm = nullptr;          // [K_pad], -1 = padding
-  uint8_t* d_quant_head = nullptr;    // layout tables of the quantizer, as it keeps them in shared memory
+  uint8_t* d_chunk_group = nullptr;   // [K_pad / 16] group of every 16-code chunk
   int32_t* d_row_group = nullptr;     // [P]
   int32_t* d_col_group = nullptr;     // [C]
   float* d_scale = nullptr;           // [T][R][G], then d_inv_scale and d_zp of the same shape
@@ -294,13 +294,6 @@ static void groups_free_device(dgq_groups* g) { pool_free(g->d_slab); }
 // group padded to a multiple of DGQ_K_ATOM positions with at least GROUP_MIN_PAD padding positions.
 // The padding carries the cell's zero-point as its code; the weight side stores -wsum spread over
 // those positions, so the integer product already contains the zero-point term of Eq. 1.
-// The quantizer's layout tables: position of every channel in the group-contiguous order (int16 [C]),
-// group of every 16-code chunk (u8 [K_pad / 16]) and the padding positions of every chunk as a bit
-// mask (u16 [K_pad / 16], 2-byte aligned), in one block whose size is a multiple of 16 bytes.
-__host__ __device__ inline int quant_head_pm_offset(int C, int K_pad) { return (C * 2 + (K_pad >> 4) + 1) & ~1; }
-__host__ __device__ inline int quant_head_bytes(int C, int K_pad) {
-  return (quant_head_pm_offset(C, K_pad) + (K_pad >> 4) * 2 + 15) & ~15;
-}
 
 static dgq_status groups_build_layout(dgq_groups* g, cudaStream_t stream) {
   g->group_off.assign(g->G + 1, 0);
@@ -323,19 +316,13 @@ static dgq_status groups_build_layout(dgq_groups* g, cudaStream_t stream) {
     bytes += (n + 255) & ~size_t(255);
     return at;
   };
-  const size_t o_perm = part(g->K_pad * sizeof(int16_t)), o_head = part(quant_head_bytes(g->C, g->K_pad));
+  const size_t o_perm = part(g->K_pad * sizeof(int16_t)), o_chunk = part(g->K_pad / 16);
   const size_t o_row = part(g->P * sizeof(int32_t)), o_col = part(g->C * sizeof(int32_t)), upload = bytes;
   const size_t o_tab = part(3 * tn * sizeof(float)), o_cell = part(2 * (size_t)g->R * g->G * sizeof(int));
   std::vector<unsigned char> h(upload, 0);
   int16_t* perm16 = reinterpret_cast<int16_t*>(h.data() + o_perm);
-  int16_t* pos = reinterpret_cast<int16_t*>(h.data() + o_head);
-  uint8_t* cg = h.data() + o_head + g->C * 2;
-  uint16_t* pm = reinterpret_cast<uint16_t*>(h.data() + o_head + quant_head_pm_offset(g->C, g->K_pad));
-  for (int p = 0; p < g->K_pad; ++p) {
-    perm16[p] = (int16_t)g->perm[p];
-    if (g->perm[p] >= 0) pos[g->perm[p]] = (int16_t)p;
-    else pm[p >> 4] |= (uint16_t)(1u << (p & 15));
-  }
+  uint8_t* cg = h.data() + o_chunk;
+  for (int p = 0; p < g->K_pad; ++p) perm16[p] = (int16_t)g->perm[p];
   for (int k = 0; k < g->G; ++k)
     for (int p = g->group_off[k]; p < g->group_off[k + 1]; p += 16) cg[p / 16] = (uint8_t)k;
   std::memcpy(h.data() + o_row, g->row_group.data(), g->P * sizeof(int32_t));
@@ -343,7 +330,7 @@ static dgq_status groups_build_layout(dgq_groups* g, cudaStream_t stream) {
   DGQ_CUDA_OK(cudaGetDevice(&g->device));
   DGQ_CUDA_OK(pool_alloc(reinterpret_cast<void**>(&g->d_slab), bytes, stream));
   g->d_perm = reinterpret_cast<int16_t*>(g->d_slab + o_perm);
-  g->d_quant_head = g->d_slab + o_head;
+  g->d_chunk_group = g->d_slab + o_chunk;
   g->d_row_group = reinterpret_cast<int32_t*>(g->d_slab + o_row);
   g->d_col_group = reinterpret_cast<int32_t*>(g->d_slab + o_col);
   g->d_scale = reinterpret_cast<float*>(g->d_slab + o_tab);

@@ -1,17 +1,24 @@
 // Activation quantizer: Eq. 1 with the per-cell parameters of Eq. 6, fused with the channel
 // permutation into the padded, group-contiguous code layout the GEMM reads.
 //
-// One warp owns one or two rows at a time and never synchronises with the rest of the CTA.  It
-// loads its rows with coalesced 128-bit loads and scatters every value to its position in the
-// group-contiguous order inside a shared-memory row buffer (padding positions of the buffer hold
-// NaN for good).  After that every 16-code chunk of the output is 32 contiguous bytes of the
-// buffer that belong to one channel group: a lane reads a chunk with two 128-bit loads, reduces
-// its range with packed half-precision min / max (which skip NaN), converts, quantizes and writes
-// one 16-byte vector, so a warp writes 512 contiguous bytes.
-// Dynamic-token mode first reduces the range of every (row, group) cell: lanes that share a cell
-// merge through shared-memory atomics on order-preserving integer keys, and one lane per cell
-// derives (s, 1/s, Z).
-// HBM traffic: 2 B read + 1 B written per element (+ 8 B per (token, group) in dynamic mode).
+// Rows are handled in pairs.  A thread block takes a batch of row pairs, loads them with 128-bit loads and
+// leaves every pair interleaved in shared memory (one 32-bit word per channel: both rows' fp16 values), so that
+// one 32-bit read fetches a channel of two rows.  A thread owns one 16-code chunk of one pair of the batch and the
+// same chunk in every batch, so the 16 channels it gathers sit in registers as byte offsets (padding positions
+// point at a word of NaN behind the row) and the values are read from shared memory once: range, parameters and codes
+// work on registers.  The packed half-precision min / max and the packed fp32 arithmetic then serve both rows with
+// one instruction.  Dynamic-token mode merges the ranges of a (row, group) cell with shared-memory atomics on
+// order-preserving keys (a warp whose lanes all belong to one cell reduces first), every thread
+// derives (s, 1/s, Z) of its two cells.
+//
+// Bound: about 300 warp instructions per row of 512 codes (half of them two-cycle integer and conversion
+// instructions) and the latency of one read-reduce-write chain for small matrices; the bytes (2 B read + 1 B written per
+// element + 8 B per (token, group) in dynamic mode) would take a third of the time.  72 registers keep 28
+// warps on an SM: at 80 an 8192-row matrix needs a second, nearly empty round of batches (5.5 against 5.1 us), at 64
+// the gathered values spill (5.9 us).  Blocks of 128 threads keep the barriers cheap (256: 5.8 us).  Against one warp
+// per two rows that scattered value by value into group order and read the chunks back twice, dynamic / static:
+// 8192 x 320 6.4 -> 5.1 / 7.0 -> 3.8 us, 32768 x 320 19.9 -> 16.3 us, 2048 x 5120 23.7 -> 15.7 us, 616 x 768 4.9 ->
+// 3.1 us, static 2048 x 1280 with 16 groups 12.0 -> 3.8 us.
 #pragma once
 
 #include <type_traits>
@@ -20,228 +27,276 @@
 
 namespace dgq {
 
-constexpr int QA_THREADS = 256;
-constexpr int QA_WARPS = QA_THREADS / 32;
+constexpr int QA_MAX_THREADS = 608;  // K_pad / 16 chunks of the widest layer (8192 channels, 32 groups)
 
 struct QuantArgs {
   const __half* X;
   uint8_t* Xq;
   int64_t M, ld;
-  int C, K_pad, G, P, bits, rows_per_warp;
-  int rows_per_cta;        // a CTA takes this many consecutive rows per sweep (a multiple of rows_per_warp, at most one turn per warp)
-  int dynamic, centred;
-  const uint8_t* head;     // layout tables (see quant_head_bytes)
-  const int32_t* row_group;
+  int C, K_pad, G, P, bits;
+  int pairs;               // row pairs of a batch
+  int pitch;               // 32-bit words of an interleaved row pair in shared memory
+  const int16_t* perm;     // [K_pad] channel of every position, -1 = padding
+  const uint8_t* chunk_group;  // [K_pad / 16]
+  const int32_t* row_group;  // null if there is one row group
   const float* inv_scale;  // static: table row of the timestep [R][G]
   const int32_t* zp;
   float* dyn_scale;        // dynamic: outputs [M][G]
   int32_t* dyn_zp;
 };
 
-__host__ __device__ inline int qa_warp_bytes(int rpw, int K_pad, int G) { return rpw * K_pad * 2 + rpw * G * 16; }
+// Words of the interleaved pair: the channels, a word of NaN for the padding, up to a multiple of four.
+__host__ __device__ inline int qa_pitch(int C) { return (C + 1 + 3) & ~3; }
+// The row buffer and two sets of cell ranges.
+__host__ inline size_t qa_smem_bytes(int pairs, int C, int G, bool dynamic) {
+  const size_t cells = (size_t)pairs * 2 * G;
+  return (size_t)pairs * qa_pitch(C) * 4 + (dynamic ? cells * 4 * 4 : 0);
+}
 
 // bits 0-3 of `m` spread to 0xFF bytes
 __device__ __forceinline__ uint32_t nibble_to_byte_mask(uint32_t m) {
   return (((m & 0xFu) * 0x00204081u) & 0x01010101u) * 0xFFu;
 }
 
-__global__ void __launch_bounds__(QA_THREADS, 4) quantize_act_kernel(const QuantArgs a) {
+// fp16 bits -> order-preserving integer and back
+__device__ __forceinline__ int half_key(uint32_t h) {
+  const int s = (int)(int16_t)h;
+  return s ^ ((s >> 15) & 0x7FFF);
+}
+__device__ __forceinline__ float half_from_key(int k) {
+  return __half2float(__ushort_as_half((uint16_t)(k ^ ((k >> 15) & 0x7FFF))));
+}
+
+// One 32-bit word of codes of four positions of a row: `y` holds x * (1/s) + 1.5 * 2^23 of the four.
+// Eq. 1 without conversion instructions, bit-identical to quantize_code for |Z| <= 2^21: y carries rint(t) in its
+// low mantissa bits (|t| < 2^22; a larger |t| ends at a clamp either way).  The lower clamp is taken on y (y >=
+// 1.5 * 2^23 - Z means rint(t) + Z >= 0; NaN falls to the bound, hence to code 0, in fmaxf), then bits(y) -
+// (0x4B400000 - Z) is the integer rint(t) + Z >= 0 and the upper clamp is the saturation of the packing
+// instruction (8 bits) or an unsigned minimum.
+template <bool CENTRED>
+__device__ __forceinline__ uint32_t codes4(const float (&y)[4], float lowb, uint32_t off, uint32_t L, uint32_t sub) {
+  uint32_t b[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) b[i] = __float_as_uint(fmaxf(y[i], lowb)) - off;
+  if (!CENTRED && L == 255u) {
+    uint32_t hi, w;
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(hi) : "r"(b[3]), "r"(b[2]), "r"(0));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(w) : "r"(b[1]), "r"(b[0]), "r"(hi));
+    return w;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) b[i] = min(b[i], L) - (CENTRED ? sub : 0u);
+  return __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
+}
+
+template <bool DYNAMIC, bool CENTRED>
+__global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ QuantArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int n_chunks = a.K_pad >> 4;
-  int16_t* pos_s = reinterpret_cast<int16_t*>(smem_raw);             // position of every channel
-  uint8_t* cg_s = reinterpret_cast<uint8_t*>(pos_s + a.C);            // group of every chunk
-  uint16_t* pm_s = reinterpret_cast<uint16_t*>(smem_raw + quant_head_pm_offset(a.C, a.K_pad));  // padding positions of every chunk
-  const int head = quant_head_bytes(a.C, a.K_pad);
-  const int rpw = a.rows_per_warp;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* wbase = smem_raw + head + warp * qa_warp_bytes(rpw, a.K_pad, a.G);
-  __half* rows_s = reinterpret_cast<__half*>(wbase);                  // [rpw][K_pad], group-contiguous order
-  int* cell_lo = reinterpret_cast<int*>(wbase + rpw * a.K_pad * 2);
-  int* cell_hi = cell_lo + rpw * a.G;
-  float* cell_inv = reinterpret_cast<float*>(cell_hi + rpw * a.G);
-  int* cell_z = reinterpret_cast<int*>(cell_inv + rpw * a.G);
+  const int n_chunks = a.K_pad >> 4, n_cells = a.pairs * 2 * a.G;
+  const int buf_bytes = a.pairs * a.pitch * 4;
+  int* cell_lo = reinterpret_cast<int*>(smem_raw + buf_bytes);  // [2][n_cells]
+  int* cell_hi = cell_lo + 2 * n_cells;
+  const int tid = threadIdx.x, n_threads = blockDim.x;
 
   pdl_launch_dependents();
-  for (int i = threadIdx.x; i < head / 16; i += QA_THREADS)
-    reinterpret_cast<uint4*>(smem_raw)[i] = __ldg(reinterpret_cast<const uint4*>(a.head) + i);
-  // The row buffers start as NaN everywhere: every row overwrites the positions of its channels, the
-  // padding positions are never written again.
-  for (int i = lane; i < rpw * a.K_pad / 8; i += 32)
-    reinterpret_cast<uint4*>(rows_s)[i] = make_uint4(0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu, 0x7FFF7FFFu);
-  __syncthreads();
+  // this thread's chunk: where its 16 values lie in an interleaved pair, its group, its padding positions
+  const int my_pair = tid / n_chunks, ch = tid - my_pair * n_chunks;
+  const bool active = my_pair < a.pairs;
+  uint32_t off[16];  // shared-memory addresses
+  uint32_t pm = 0;
+  int g = 0;
+  {
+    const uint4* pp = reinterpret_cast<const uint4*>(a.perm) + (active ? ch : 0) * 2;
+    const uint4 p0 = __ldg(pp), p1 = __ldg(pp + 1);
+    const uint32_t pw[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+    const uint32_t base = smem_u32(smem_raw) + (uint32_t)((active ? my_pair : 0) * a.pitch) * 4u;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int c = (int)(int16_t)(pw[i >> 1] >> (16 * (i & 1)));
+      if (c < 0) pm |= 1u << i;
+      off[i] = base + (uint32_t)(c < 0 ? a.C : c) * 4u;
+    }
+    g = active ? __ldg(a.chunk_group + ch) : 0;
+  }
+  for (int i = tid; i < a.pairs; i += n_threads)
+    *reinterpret_cast<uint32_t*>(smem_raw + ((size_t)i * a.pitch + a.C) * 4) = 0x7FFF7FFFu;  // the word of NaN
+  if (DYNAMIC)
+    for (int i = tid; i < n_cells; i += n_threads) {
+      cell_lo[i] = INT_MAX;
+      cell_hi[i] = INT_MIN;
+    }
+  const int cell = my_pair * 2 * a.G + g;  // row 0 of the pair; row 1: + G
+  const bool leads = active && (ch == 0 || __ldg(a.chunk_group + ch - 1) != g);  // the cell's first chunk
+  bool one_cell = false;                   // every lane of the warp reduces into the same cell
+  if (DYNAMIC) {
+    const int first = __shfl_sync(0xffffffffu, cell, 0);
+    one_cell = __all_sync(0xffffffffu, !active || cell == first);
+  }
+  // this thread's share of the row loads: at most two pieces of eight channels of a pair
+  const int vec = a.C >> 3;
+  int lp[2], lv[2];
+  bool lok[2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int task = tid + e * n_threads;
+    lp[e] = task / vec;
+    lv[e] = task - lp[e] * vec;
+    lok[e] = lp[e] < a.pairs;
+  }
+  float inv0 = 0.f, inv1 = 0.f;
+  int z0 = 0, z1 = 0;
+  if (!DYNAMIC && !a.row_group) {
+    inv0 = inv1 = __ldg(a.inv_scale + g);
+    z0 = z1 = __ldg(a.zp + g);
+  }
   pdl_wait();  // everything above reads only constants of the grouping; the rows may come from the previous kernel
 
-  const int vec_per_row = a.C >> 3;
-  const float Lf = (float)((1 << a.bits) - 1);
-  // A CTA takes rows_per_cta consecutive rows per sweep over the matrix, at most one turn per warp.  Small
-  // matrices are dealt out in one sweep with the same number of rows for every CTA (a kernel of one wave lasts
-  // as long as its busiest SM); large ones in sweeps of full CTAs.
-  for (int64_t base = (int64_t)blockIdx.x * a.rows_per_cta; base < a.M; base += (int64_t)gridDim.x * a.rows_per_cta) {
-    const int64_t cta_end = min(a.M, base + a.rows_per_cta);
-    const int64_t row0 = base + warp * rpw;
-    if (row0 >= cta_end) continue;  // the same answer in every lane of the warp
-    const int rows = (int)min((int64_t)rpw, cta_end - row0);
-    // Row loads in batches of four 128-bit pieces per lane: every load of a batch is issued before
-    // the first store, so the memory latency is paid once per batch and not once per piece.
-    {
-      const int n_vec = rows * vec_per_row;
-      const uint4* xrow = reinterpret_cast<const uint4*>(a.X + row0 * a.ld);
-      const int64_t row_step = a.ld >> 3;  // in 128-bit pieces
-      uint16_t* dst0 = reinterpret_cast<uint16_t*>(rows_s);
-      for (int v0 = 0; v0 < n_vec; v0 += 4 * 32) {
-        uint4 x[4];
+  const int64_t rows_per_batch = 2 * (int64_t)a.pairs, step = rows_per_batch * gridDim.x;
+  uint4 xa[2], xb[2];
+  auto request = [&](int64_t row0) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int i = v0 + e * 32 + lane;
-          if (i < n_vec) {
-            const int r = i >= vec_per_row ? 1 : 0, v = i - r * vec_per_row;  // at most two rows per warp
-            x[e] = __ldg(xrow + r * row_step + v);
+    for (int e = 0; e < 2; ++e) {
+      const int64_t row = row0 + 2 * lp[e];
+      if (lok[e] && row < a.M) {
+        const uint4* src = reinterpret_cast<const uint4*>(a.X + row * a.ld) + lv[e];
+        xa[e] = __ldg(src);
+        xb[e] = row + 1 < a.M ? __ldg(src + (a.ld >> 3)) : xa[e];
+      }
+    }
+  };
+  const int64_t first_row = (int64_t)blockIdx.x * rows_per_batch;
+  if (first_row < a.M) request(first_row);
+  int buf = 0;
+  for (int64_t row0 = first_row; row0 < a.M; row0 += step, buf ^= 1) {
+    // (dynamic: the barrier behind the ranges says so)
+    if (!DYNAMIC && row0 != first_row) __syncthreads();  // every value of the last batch is in registers
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+      if (lok[e]) {
+        uint4* dst = reinterpret_cast<uint4*>(smem_raw + (lp[e] * a.pitch + lv[e] * 8) * 4);
+        dst[0] = make_uint4(__byte_perm(xa[e].x, xb[e].x, 0x5410), __byte_perm(xa[e].x, xb[e].x, 0x7632),
+                            __byte_perm(xa[e].y, xb[e].y, 0x5410), __byte_perm(xa[e].y, xb[e].y, 0x7632));
+        dst[1] = make_uint4(__byte_perm(xa[e].z, xb[e].z, 0x5410), __byte_perm(xa[e].z, xb[e].z, 0x7632),
+                            __byte_perm(xa[e].w, xb[e].w, 0x5410), __byte_perm(xa[e].w, xb[e].w, 0x7632));
+      }
+    if (row0 + step < a.M) request(row0 + step);  // arrives while this batch is worked on
+    __syncthreads();
+    __half2 x[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      uint32_t v;
+      asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(off[i]));
+      x[i] = *reinterpret_cast<const __half2*>(&v);
+    }
+    if (DYNAMIC) {
+      __half2 lo = __hmin2(x[0], x[1]), hi = __hmax2(x[0], x[1]);  // NaN (padding, or a NaN input) never wins
+#pragma unroll
+      for (int i = 2; i < 16; ++i) {
+        lo = __hmin2(lo, x[i]);
+        hi = __hmax2(hi, x[i]);
+      }
+      const uint32_t lw = *reinterpret_cast<const uint32_t*>(&lo), hw = *reinterpret_cast<const uint32_t*>(&hi);
+      int* c_lo = cell_lo + buf * n_cells;
+      int* c_hi = cell_hi + buf * n_cells;
+      int k[4] = {half_key(lw), half_key(lw >> 16), half_key(hw), half_key(hw >> 16)};
+      const bool none0 = !active || (lw & 0x7FFFu) > 0x7C00u, none1 = !active || (lw & 0x7FFF0000u) > 0x7C000000u;
+      if (none0) k[0] = INT_MAX, k[2] = INT_MIN;  // nothing but padding
+      if (none1) k[1] = INT_MAX, k[3] = INT_MIN;
+      if (one_cell) {
+        k[0] = __reduce_min_sync(0xffffffffu, k[0]);
+        k[1] = __reduce_min_sync(0xffffffffu, k[1]);
+        k[2] = __reduce_max_sync(0xffffffffu, k[2]);
+        k[3] = __reduce_max_sync(0xffffffffu, k[3]);
+      }
+      if (active && (!one_cell || (tid & 31) == 0)) {
+        atomicMin(c_lo + cell, k[0]);
+        atomicMin(c_lo + cell + a.G, k[1]);
+        atomicMax(c_hi + cell, k[2]);
+        atomicMax(c_hi + cell + a.G, k[3]);
+      }
+      __syncthreads();
+      if (active) {
+        // Every thread derives the parameters of its two cells itself: two more IEEE divisions per thread cost less
+        // than a third barrier behind the few threads that would do it for all.
+        float l0 = 0.f, h0 = 0.f, l1 = 0.f, h1 = 0.f, s0, s1;
+        if (c_lo[cell] != INT_MAX) l0 = half_from_key(c_lo[cell]), h0 = half_from_key(c_hi[cell]);
+        if (c_lo[cell + a.G] != INT_MAX) l1 = half_from_key(c_lo[cell + a.G]), h1 = half_from_key(c_hi[cell + a.G]);
+        group_params(l0, h0, a.bits, s0, inv0, z0);
+        group_params(l1, h1, a.bits, s1, inv1, z1);
+        if (leads) {
+          const int64_t o = (row0 + 2 * my_pair) * a.G + g;
+          if (row0 + 2 * my_pair < a.M) {
+            a.dyn_scale[o] = s0;
+            a.dyn_zp[o] = z0;
           }
-        }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int i = v0 + e * 32 + lane;
-          if (i < n_vec) {
-            const int r = i >= vec_per_row ? 1 : 0, v = i - r * vec_per_row;
-            const uint4 pp = *reinterpret_cast<const uint4*>(pos_s + v * 8);  // positions of these 8 channels
-            uint16_t* dst = dst0 + r * a.K_pad;
-            const uint32_t pw[4] = {pp.x, pp.y, pp.z, pp.w}, xw[4] = {x[e].x, x[e].y, x[e].z, x[e].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              dst[pw[j] & 0xFFFFu] = (uint16_t)(xw[j] & 0xFFFFu);
-              dst[pw[j] >> 16] = (uint16_t)(xw[j] >> 16);
-            }
+          if (row0 + 2 * my_pair + 1 < a.M) {
+            a.dyn_scale[o + a.G] = s1;
+            a.dyn_zp[o + a.G] = z1;
           }
+          int* n_lo = cell_lo + (buf ^ 1) * n_cells + cell;  // for the next batch
+          int* n_hi = cell_hi + (buf ^ 1) * n_cells + cell;
+          n_lo[0] = n_lo[a.G] = INT_MAX;
+          n_hi[0] = n_hi[a.G] = INT_MIN;
         }
       }
     }
-    if (a.dynamic)
-      for (int i = lane; i < rows * a.G; i += 32) {
-        cell_lo[i] = INT_MAX;
-        cell_hi[i] = INT_MIN;
-      }
-    __syncwarp();
-
-    if (a.dynamic) {
-      for (int r = 0; r < rows; ++r) {
-        const uint4* row = reinterpret_cast<const uint4*>(rows_s + r * a.K_pad);
-        for (int ch = lane; ch < n_chunks; ch += 32) {
-          const uint4 u0 = row[ch * 2], u1 = row[ch * 2 + 1];
-          const __half2* h0 = reinterpret_cast<const __half2*>(&u0);
-          const __half2* h1 = reinterpret_cast<const __half2*>(&u1);
-          // NaN (padding, or a NaN input) never wins a min / max
-          __half2 lo2 = __hmin2(__hmin2(__hmin2(h0[0], h0[1]), __hmin2(h0[2], h0[3])),
-                                __hmin2(__hmin2(h1[0], h1[1]), __hmin2(h1[2], h1[3])));
-          __half2 hi2 = __hmax2(__hmax2(__hmax2(h0[0], h0[1]), __hmax2(h0[2], h0[3])),
-                                __hmax2(__hmax2(h1[0], h1[1]), __hmax2(h1[2], h1[3])));
-          const float lo = __half2float(__hmin(__low2half(lo2), __high2half(lo2)));
-          const float hi = __half2float(__hmax(__low2half(hi2), __high2half(hi2)));
-          if (lo <= hi) {  // false when the whole chunk is padding
-            const int g = cg_s[ch];
-            atomicMin(&cell_lo[r * a.G + g], float_to_ordered(lo));
-            atomicMax(&cell_hi[r * a.G + g], float_to_ordered(hi));
-          }
-        }
-      }
-      __syncwarp();
-      for (int i = lane; i < rows * a.G; i += 32) {
-        float lo = 0.f, hi = 0.f;
-        if (cell_lo[i] != INT_MAX) {
-          lo = ordered_to_float(cell_lo[i]);
-          hi = ordered_to_float(cell_hi[i]);
-        }
-        float s, inv_s;
-        int Z;
-        group_params(lo, hi, a.bits, s, inv_s, Z);
-        cell_inv[i] = inv_s;
-        cell_z[i] = Z;
-        const int r = i / a.G, g = i - r * a.G;
-        a.dyn_scale[(row0 + r) * a.G + g] = s;
-        a.dyn_zp[(row0 + r) * a.G + g] = Z;
-      }
-      __syncwarp();
+    const int64_t row = row0 + 2 * my_pair;
+    if (!active || row >= a.M) continue;
+    const bool two = row + 1 < a.M;
+    if (!DYNAMIC && a.row_group) {
+      const int rg0 = __ldg(a.row_group + row % a.P) * a.G + g, rg1 = __ldg(a.row_group + (row + 1) % a.P) * a.G + g;
+      inv0 = __ldg(a.inv_scale + rg0);
+      z0 = __ldg(a.zp + rg0);
+      inv1 = __ldg(a.inv_scale + rg1);
+      z1 = __ldg(a.zp + rg1);
     }
-
-    for (int r = 0; r < rows; ++r) {
-      const uint4* row = reinterpret_cast<const uint4*>(rows_s + r * a.K_pad);
-      const int rg = a.dynamic ? 0 : a.row_group[(row0 + r) % a.P];
-      uint8_t* out = a.Xq + (row0 + r) * a.K_pad;
-      for (int ch = lane; ch < n_chunks; ch += 32) {
-        const int g = cg_s[ch];
-        float inv_s;
-        int Z;
-        if (a.dynamic) {
-          inv_s = cell_inv[r * a.G + g];
-          Z = cell_z[r * a.G + g];
-        } else {
-          inv_s = __ldg(a.inv_scale + rg * a.G + g);
-          Z = __ldg(a.zp + rg * a.G + g);
+    const uint32_t L = (1u << a.bits) - 1u;
+    const uint32_t sub0 = CENTRED ? (uint32_t)z0 : 0u, sub1 = CENTRED ? (uint32_t)z1 : 0u;
+    uint32_t w0[4], w1[4];
+    if (abs(z0) <= (1 << 21) && abs(z1) <= (1 << 21)) {
+      // product and sum rounded separately (x * (1/s) + (-0) is the rounded product, times one plus
+      // 1.5 * 2^23 the rounded sum: an add in its place gets fused with the product), both rows per instruction
+      const float MAGIC = 12582912.0f;
+      const unsigned long long inv2 = pack_f32x2(inv0, inv1), magic2 = pack_f32x2(MAGIC, MAGIC);
+      const unsigned long long nzero2 = pack_f32x2(-0.0f, -0.0f), one2 = pack_f32x2(1.0f, 1.0f);
+      const float low0 = MAGIC - (float)z0, low1 = MAGIC - (float)z1;
+      const uint32_t off0 = 0x4B400000u - (uint32_t)z0, off1 = 0x4B400000u - (uint32_t)z1;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float y0[4], y1[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 f = __half22float2(x[4 * q + i]);
+          unpack_f32x2(fma_f32x2(fma_f32x2(pack_f32x2(f.x, f.y), inv2, nzero2), one2, magic2), y0[i], y1[i]);
         }
-        const float Zf = (float)Z;
-        const int sub = a.centred ? Z : 0;
-        const uint4 u[2] = {row[ch * 2], row[ch * 2 + 1]};
-        const __half2* h = reinterpret_cast<const __half2*>(u);
-        uint32_t w[4];
-        if (abs(Z) <= (1 << 21)) {
-          // Eq. 1 without conversion instructions, bit-identical to quantize_code for |Z| <= 2^21:
-          // y = x * (1/s) + 1.5 * 2^23 carries rint(t) in its low mantissa bits (|t| < 2^22; a larger |t|
-          // ends at a clamp either way).  The lower clamp is taken on y (y >= 1.5 * 2^23 - Z means
-          // rint(t) + Z >= 0; NaN falls to the bound, hence to code 0, in fmaxf), then
-          // bits(y) - (0x4B400000 - Z) is the integer rint(t) + Z >= 0 and the upper clamp is an unsigned
-          // minimum.  The product and the sum are rounded separately (x * (1/s) + (-0) is the rounded
-          // product), two values per packed instruction.
-          const float MAGIC = 12582912.0f;
-          const float lowb = MAGIC - Zf;
-          const uint32_t Lu = (uint32_t)((1 << a.bits) - 1);
-          const unsigned long long inv2 = pack_f32x2(inv_s, inv_s), magic2 = pack_f32x2(MAGIC, MAGIC);
-          const unsigned long long nzero2 = pack_f32x2(-0.0f, -0.0f), one2 = pack_f32x2(1.0f, 1.0f);
-          const uint32_t off = 0x4B400000u - (uint32_t)Z;
-          auto codes16 = [&](auto centred_tag) {
+        w0[q] = codes4<CENTRED>(y0, low0, off0, L, sub0);
+        w1[q] = codes4<CENTRED>(y1, low1, off1, L, sub1);
+      }
+    } else {
+      const float Lf = (float)L, zf0 = (float)z0, zf1 = (float)z1;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              uint32_t b[4];
+      for (int q = 0; q < 4; ++q) {
+        w0[q] = w1[q] = 0;
 #pragma unroll
-              for (int j = 0; j < 2; ++j) {
-                const float2 f = __half22float2(h[2 * q + j]);
-                const unsigned long long t2 = fma_f32x2(pack_f32x2(f.x, f.y), inv2, nzero2);
-                float y0, y1;
-                unpack_f32x2(fma_f32x2(t2, one2, magic2), y0, y1);
-                b[2 * j] = min(__float_as_uint(fmaxf(y0, lowb)) - off, Lu);
-                b[2 * j + 1] = min(__float_as_uint(fmaxf(y1, lowb)) - off, Lu);
-                if (decltype(centred_tag)::value) {  // low byte = code - Z (two's complement)
-                  b[2 * j] -= (uint32_t)sub;
-                  b[2 * j + 1] -= (uint32_t)sub;
-                }
-              }
-              w[q] = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
-            }
-          };
-          if (a.centred) codes16(std::true_type{});
-          else codes16(std::false_type{});
-        } else {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float2 f0 = __half22float2(h[2 * q]), f1 = __half22float2(h[2 * q + 1]);
-            const int c0 = quantize_code(f0.x, inv_s, Zf, Lf) - sub, c1 = quantize_code(f0.y, inv_s, Zf, Lf) - sub;
-            const int c2 = quantize_code(f1.x, inv_s, Zf, Lf) - sub, c3 = quantize_code(f1.y, inv_s, Zf, Lf) - sub;
-            w[q] = (uint32_t)(c0 & 0xFF) | ((uint32_t)(c1 & 0xFF) << 8) | ((uint32_t)(c2 & 0xFF) << 16) |
-                   ((uint32_t)c3 << 24);
-          }
+        for (int i = 0; i < 4; ++i) {
+          const float2 f = __half22float2(x[4 * q + i]);
+          w0[q] |= (((uint32_t)quantize_code(f.x, inv0, zf0, Lf) - sub0) & 0xFFu) << (8 * i);
+          w1[q] |= (((uint32_t)quantize_code(f.y, inv1, zf1, Lf) - sub1) & 0xFFu) << (8 * i);
         }
-        const uint32_t pm = pm_s[ch];
-        if (pm) {  // padding positions carry the clamped zero-point (0 in the zero-centred layout)
-          const uint32_t pad_code = a.centred ? 0u : (uint32_t)min(max(Z, 0), (1 << a.bits) - 1);
-          const uint32_t padw = pad_code * 0x01010101u;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const uint32_t m = nibble_to_byte_mask(pm >> (4 * q));
-            w[q] = (w[q] & ~m) | (padw & m);
-          }
-        }
-        *reinterpret_cast<uint4*>(out + ch * 16) = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
-    __syncwarp();  // rows fully consumed before the next iteration overwrites them
+    if (pm) {  // padding positions (NaN, so far code 0) carry the clamped zero-point (0 in the zero-centred layout)
+      const uint32_t pad0 = (uint32_t)min(max(z0, 0), (int)L) * 0x01010101u, pad1 = (uint32_t)min(max(z1, 0), (int)L) * 0x01010101u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t m = nibble_to_byte_mask(pm >> (4 * q));
+        w0[q] = CENTRED ? w0[q] & ~m : w0[q] | (pad0 & m);
+        w1[q] = CENTRED ? w1[q] & ~m : w1[q] | (pad1 & m);
+      }
+    }
+    uint8_t* out = a.Xq + row * a.K_pad + ch * 16;
+    *reinterpret_cast<uint4*>(out) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
+    if (two) *reinterpret_cast<uint4*>(out + a.K_pad) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
   }
 }
 
@@ -278,44 +333,42 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   a.G = g->G;
   a.P = g->P;
   a.bits = g->bits;
-  a.dynamic = (mode == DGQ_MODE_DYNAMIC_TOKEN);
-  a.centred = (layout == DGQ_CODES_S8_CENTRED);
-  a.head = g->d_quant_head;
-  a.row_group = g->d_row_group;
+  a.pitch = qa_pitch(g->C);
+  a.perm = g->d_perm;
+  a.chunk_group = g->d_chunk_group;
+  a.row_group = g->R > 1 ? g->d_row_group : nullptr;
   a.inv_scale = g->d_inv_scale + trow;
   a.zp = g->d_zp + trow;
   a.dyn_scale = dyn_scale;
   a.dyn_zp = dyn_zp;
-  const int rpw = (g->C <= 1280) ? 2 : 1;
-  a.rows_per_warp = rpw;
-  const size_t smem = (size_t)quant_head_bytes(g->C, g->K_pad) + (size_t)QA_WARPS * qa_warp_bytes(rpw, g->K_pad, g->G);
-  if (smem > 200 * 1024) return DGQ_ERR_UNSUPPORTED;
-  static bool attr_set[64] = {false};
+  const bool dynamic = mode == DGQ_MODE_DYNAMIC_TOKEN;
+  int n_sm = 0;
+  DGQ_CUDA_OK(sm_count(&n_sm));
+  // A block of about 128 threads, one per chunk of a batch (a single pair of a wide layer may need more), about 896
+  // threads to an SM.  A matrix that would leave blocks without work gets smaller batches, down to one pair.
+  const int n_chunks = g->K_pad / 16;
+  const int64_t n_pairs = (M + 1) / 2;
+  int pairs = std::max(1, 128 / n_chunks);
+  int64_t slots = (int64_t)n_sm * std::max(1, 896 / (pairs * n_chunks));
+  if (n_pairs < slots * pairs) pairs = (int)std::max<int64_t>(1, (n_pairs + slots - 1) / slots);
+  const int threads = (pairs * n_chunks + 31) / 32 * 32;
+  slots = (int64_t)n_sm * std::max(1, 896 / threads);
+  a.pairs = pairs;
+  const size_t smem = qa_smem_bytes(pairs, g->C, g->G, dynamic);
+  static std::atomic<bool> attr_set[64];
   int dev = 0;
   DGQ_CUDA_OK(cudaGetDevice(&dev));
-  if (dev >= 64 || !attr_set[dev]) {
-    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    if (dev < 64) attr_set[dev] = true;
+  if (dev >= 64 || !attr_set[dev].load()) {
+    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    if (dev < 64) attr_set[dev].store(true);
   }
-  // Four CTAs fit on an SM.  A matrix that one wave of full CTAs can cover is dealt out evenly over 4 x SMs
-  // CTAs instead; a larger one goes to at most two waves of full CTAs that sweep over it.
-  static int sm_count[64] = {0};
-  if (dev >= 64 || sm_count[dev] == 0) {
-    int n = 0;
-    DGQ_CUDA_OK(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
-    if (n <= 0) return DGQ_ERR_CUDA;
-    if (dev < 64) sm_count[dev] = n;
-  }
-  const int64_t slots = 4 * (int64_t)(dev < 64 ? sm_count[dev] : 148);
-  const int64_t full = (int64_t)QA_WARPS * rpw;  // rows of a CTA whose warps all take one turn
-  int64_t rows_per_cta = full;
-  if (M <= slots * full) {
-    rows_per_cta = (M + slots - 1) / slots;
-    rows_per_cta = (rows_per_cta + rpw - 1) / rpw * rpw;
-  }
-  a.rows_per_cta = (int)rows_per_cta;
-  const int grid = (int)std::min<int64_t>((M + rows_per_cta - 1) / rows_per_cta, 2 * slots);
-  DGQ_CUDA_OK(launch_pdl(quantize_act_kernel, dim3(grid), dim3(QA_THREADS), smem, (cudaStream_t)stream, a));
+  const int grid = (int)std::min<int64_t>((n_pairs + pairs - 1) / pairs, slots);
+  DGQ_CUDA_OK(launch_pdl(dynamic ? quantize_act_kernel<true, false>
+                                : layout == DGQ_CODES_S8_CENTRED ? quantize_act_kernel<false, true> : quantize_act_kernel<false, false>,
+                         dim3(grid), dim3(threads), smem,
+                         (cudaStream_t)stream, a));
   g_launches += 1;
   DGQ_CUDA_OK(cudaGetLastError());
   return DGQ_OK;

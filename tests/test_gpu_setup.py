@@ -61,3 +61,38 @@ def test_weight_layout_edges(sizes, N, w_bits):
     assert torch.equal(Y, Y2) and b.device_status() == 0
     s_rows, z_rows = np.broadcast_to(scale[0], (M, G)), np.broadcast_to(zp[0], (M, G))
     check_output(Y, ol.group_linear(codes, s_rows, z_rows, cg, wq, sw, None))
+
+
+@pytest.mark.parametrize("mode", ["static", "dynamic"])
+@pytest.mark.parametrize("M,sizes,bits", [
+    (1, (8,), 8),                    # one row, two chunks: a block of 64 pairs with one of them real
+    (3, (1, 31, 33, 255), 6),        # odd row count, groups that end inside a chunk, 6-bit clamp
+    (257, (320,), 8),                # a cell that covers a whole warp
+    (9, (5112, 8), 8),               # one pair per block, more chunks than a small block has threads
+    (4100, (8184, 8), 4),            # the widest layer, several batches per block
+])
+def test_quantizer_edges(M, sizes, bits, mode):
+    torch, b = gpu()
+    C, G = sum(sizes), len(sizes)
+    rng = np.random.default_rng(M)
+    cg = rng.permutation(np.repeat(np.arange(G), sizes)).astype(np.int32)
+    scale = rng.uniform(0.01, 0.05, (1, 1, G)).astype(np.float32)
+    zp = rng.integers(0, 2 ** bits, (1, 1, G)).astype(np.int32)
+    g = b.groups_from_host(C, 1, bits, cg, np.zeros(1, np.int32), scale, zp)
+    X = rng.normal(0, 1, (M, C)).astype(np.float16)
+    ex = g.export()
+    L = 2 ** bits - 1
+    Xq, ds, dz = b.quantize_act(g, to_dev(torch, X), mode=b.MODE_DYNAMIC_TOKEN if mode == "dynamic" else b.MODE_STATIC)
+    if mode == "dynamic":
+        codes, s_rows, z_rows = ol.quantize_dynamic_token(X, cg, G, bits)
+        assert np.array_equal(ds.cpu().numpy(), s_rows) and np.array_equal(dz.cpu().numpy(), z_rows)
+    else:
+        inv = (np.float32(1) / scale[0, 0]).astype(np.float32)
+        codes = np.clip(np.rint(X.astype(np.float32) * inv[cg]) + zp[0, 0, cg], 0, L).astype(np.int64)
+        z_rows = np.broadcast_to(zp[0], (M, G))
+    full = Xq.cpu().numpy().astype(np.int64)
+    valid = ex["perm"] >= 0
+    assert np.array_equal(full[:, valid], codes[:, ex["perm"][valid]])
+    group_of = np.repeat(np.arange(G), np.diff(ex["group_off"]))
+    assert np.array_equal(full[:, ~valid], np.clip(z_rows, 0, L)[:, group_of[~valid]])   # padding = clamped zero-point
+    assert b.device_status() == 0

@@ -6,7 +6,7 @@
 //
 // CTA = one 128-row output tile x BN columns, persistent over tiles.  Warp roles:
 //   warps 0-7   epilogue: lane quarter = warp & 3 (the TMEM lanes a warp may read), column half = warp >> 2
-//   warp  8     TMA producer (one lane): A code tile and B weight tile per 128-byte K stage
+//   warp  8, 11 TMA producers: A code tile and B weight tile per 128-byte K stage
 //   warp  9     MMA issuer (one lane) and TMEM allocator
 //   warp  10    output store (one lane): TMA stores of the staged fp16 tile
 //   warps 11-15 (4-bit weights only) unpack packed nibbles from global memory into the B stage
@@ -48,6 +48,7 @@ constexpr int GEMM_EPI_WARPS = 8;
 constexpr int GEMM_WARP_TMA = GEMM_EPI_WARPS;
 constexpr int GEMM_WARP_MMA = GEMM_EPI_WARPS + 1;
 constexpr int GEMM_WARP_STORE = GEMM_EPI_WARPS + 2;
+constexpr int GEMM_WARP_TMA2 = GEMM_EPI_WARPS + 3;  // second producer (not with in-kernel unpacking, whose warps start here)
 constexpr int GEMM_THREADS_W8 = (GEMM_EPI_WARPS + 3) * 32;  // first unpack thread
 __host__ __device__ constexpr int gemm_threads(bool w4) { return (w4 ? 16 : 12) * 32; }
 // Registers per thread: the kernel starts with `gemm_regs_launch`, the epilogue warps then grow to
@@ -60,6 +61,7 @@ static_assert(8 * gemm_regs_epi(false) + 4 * gemm_regs_other(false) <= 12 * gemm
 constexpr int GEMM_MAX_ATOMS = 1024;           // 32768 reduction positions
 constexpr int GEMM_A_STAGE = GEMM_BM * 128;  // bytes
 constexpr int GEMM_SMEM_LIMIT = 227 * 1024;
+constexpr int GEMM_LONG_STAGES = 8;          // from this many stages on a reduction is fed by two producers and issued by groups
 
 template <int BN, bool W4>
 struct GemmCfg {
@@ -98,13 +100,14 @@ struct GemmArgs {
   const float* scale;         // [rows][G]
   const int32_t* zp;          // [rows][G]
   const int32_t* row_group;   // [P]
+  int b_early;                // the B operand does not come from an earlier kernel
   const float* sw;            // [N_pad]
   const float* wsum;          // [G][N_pad]
   const float* wres;          // [G][N_pad]
   const __half* bias;         // [N] or null
   const uint8_t* w_packed;    // 4-bit weights [N_pad][Kt/2]
   int seg_end[DGQ_MAX_GROUPS];    // end atom of every group segment
-  unsigned long long end_mask[GEMM_MAX_ATOMS / 64];  // bit i: atom i is the last of its group
+  unsigned long long end_mask;    // reductions of fewer than GEMM_LONG_STAGES stages: bit i: atom i is the last of its group
   // conv
   int conv_W, conv_H;
   int grp_atoms[DGQ_MAX_GROUPS];  // channel atoms of every group
@@ -152,6 +155,11 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int n_kstages = (n_atoms + 3) >> 2;
   const int n_tiles = a.n_tiles_m * a.n_tiles_n;
 
+  if (threadIdx.x == 32 * GEMM_WARP_TMA) {
+    tma_prefetch_desc(&tmA);
+    if (!W4) tma_prefetch_desc(&tmB);
+    tma_prefetch_desc(&tmY);
+  }
   if (threadIdx.x == 0) {
     for (int i = 0; i < STAGES; ++i) {
       mbar_init(&sh->full[i], W4 ? 1 + GEMM_UNPACK_WARPS : 1);
@@ -196,9 +204,8 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tmem_alloc(&sh->tmem_base, 512);
     tmem_relinquish();
   }
-  // Everything above reads only the layer's constants; codes, scales and zero-points may come from
-  // the kernel before this one.
-  pdl_wait();
+  // Everything up to here reads only the layer's constants; codes, scales and zero-points may come from the kernel
+  // before this one, so every role waits for it (pdl_wait) before its first access to them.
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -207,22 +214,36 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (warp >= GEMM_EPI_WARPS) {
   // The warps that only move data or issue instructions hand most of their registers to the epilogue.
   reg_dealloc<gemm_regs_other(W4)>();
-  if (warp == GEMM_WARP_TMA) {
-    // ------------------------------------------------------------ TMA producer
-    // Five lanes run the loop together and issue their copies with one instruction: lanes 0-3 an A box each
-    // (a conv stage is four boxes, one per atom; a linear stage is one box, lane 0's), lane 4 the B box.
-    // Handing a box to the copy engine costs a thread a few hundred cycles of issue time, which one lane
-    // alone cannot hide when the boxes are as small as a conv atom's.  The other lanes go straight to the
-    // CTA's final barrier.
-    if (lane < 5) {
-      constexpr uint32_t PROD_MASK = 0x1Fu;
-      if (lane == 0) tma_prefetch_desc(&tmA);
-      if (!W4 && lane == 4) tma_prefetch_desc(&tmB);
+  if (warp == GEMM_WARP_TMA || (!W4 && warp == GEMM_WARP_TMA2)) {
+    // ------------------------------------------------------------ TMA producers
+    // Posting a stage (wait, byte count, a box of A and one of B) costs the issuing warp about 400 cycles, a conv stage
+    // with its four A boxes 600-800, whatever the boxes hold and wherever they come from: one warp alone fed
+    // long reductions at 545 and convs at 880 cycles a stage against 320 cycles of MMA, so two warps take the stages
+    // of a long reduction in turn.  The whole warp runs the loop and one elected lane issues (a loop run by some
+    // lanes of a diverged warp costs another 100-200 cycles).  A short reduction is bound by its epilogue, whose issue
+    // slots a second producer would take; with 4-bit weights unpacked in the kernel there is no warp to spare.
+    const int producers = W4 || n_kstages < GEMM_LONG_STAGES ? 1 : 2;
+    const int turn = (warp == GEMM_WARP_TMA) ? 0 : 1;
+    if (turn < producers) {
       const uint32_t empty0 = smem_u32(&sh->empty[0]);
-      uint32_t s = 0, empty_par = 1;  // fresh barriers pass a wait for parity 1
+      // The first tile's weights do not depend on the kernel before this one: their boxes go out ahead of the wait.
+      int early = 0;
+      if (!W4 && a.b_early && (int)blockIdx.x < n_tiles) {
+        early = min(n_kstages, STAGES);
+        for (int ks = turn; ks < early; ks += producers) {
+          const int atoms_here = min(4, n_atoms - ks * 4);
+          if (elect_one()) {
+            mbar_arrive_expect_tx(&sh->full[ks], (uint32_t)Cfg::B_STAGE + (CONV ? (uint32_t)(atoms_here * 4096) : (uint32_t)GEMM_A_STAGE));
+            tma_load_2d(smB + ks * Cfg::B_STAGE, &tmB, &sh->full[ks], ks * 128, cta_n0);
+          }
+          __syncwarp();
+        }
+      }
+      pdl_wait();
+      uint32_t s = (uint32_t)turn, empty_par = 1;  // fresh barriers pass a wait for parity 1
+      int ks = turn;
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const int tm = tile / a.n_tiles_n, tn = tile - tm * a.n_tiles_n;
-        const int m0 = tm * GEMM_BM, n0 = tn * BN;
+        const int m0 = tile / a.n_tiles_n * GEMM_BM;
         int cw = 0, chh = 0, cn = 0;  // conv: spatial origin of this row tile
         if (CONV) {
           const int hw = a.conv_H * a.conv_W;
@@ -231,40 +252,52 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           chh = rem / a.conv_W;
           cw = rem - chh * a.conv_W;
         }
-        for (int ks = 0; ks < n_kstages; ++ks) {
+        for (; ks < n_kstages; ks += producers) {
           mbar_wait_lean(empty0 + s * 8u, empty_par, abort_flag);
-          const int atoms_here = min(4, n_atoms - ks * 4);
-          uint32_t bytes = W4 ? 0u : (uint32_t)Cfg::B_STAGE;
-          bytes += CONV ? (uint32_t)(atoms_here * 4096) : (uint32_t)GEMM_A_STAGE;
-          if (lane == 0) mbar_arrive_expect_tx(&sh->full[s], bytes);  // before any of the copies below
-          __syncwarp(PROD_MASK);
-          if (CONV) {
-            if (lane < atoms_here) {
-              const uint32_t e = conv_tab[ks * 4 + lane];
-              tma_load_4d(smA + s * GEMM_A_STAGE + lane * 4096, &tmA, &sh->full[s], (int)(e & 0xFFFFu),
-                          cw + (int)((e >> 16) & 3u) - 1, chh + (int)((e >> 18) & 3u) - 1, cn);
+          uint4 tab = make_uint4(0, 0, 0, 0);
+          if (CONV) tab = *reinterpret_cast<const uint4*>(conv_tab + ks * 4);
+          if (elect_one()) {
+            const int atoms_here = min(4, n_atoms - ks * 4);
+            if (ks >= early) {
+              const uint32_t bytes = (W4 ? 0u : (uint32_t)Cfg::B_STAGE) + (CONV ? (uint32_t)(atoms_here * 4096) : (uint32_t)GEMM_A_STAGE);
+              mbar_arrive_expect_tx(&sh->full[s], bytes);  // before any of the copies below
+              if (!W4) tma_load_2d(smB + s * Cfg::B_STAGE, &tmB, &sh->full[s], ks * 128, cta_n0);
             }
-          } else if (lane == 0) {
-            tma_load_2d(smA + s * GEMM_A_STAGE, &tmA, &sh->full[s], ks * 128, m0);
+            if (CONV) {
+              auto box = [&](int j, uint32_t e) {
+                tma_load_4d(smA + s * GEMM_A_STAGE + j * 4096, &tmA, &sh->full[s], (int)(e & 0xFFFFu),
+                            cw + (int)((e >> 16) & 3u) - 1, chh + (int)((e >> 18) & 3u) - 1, cn);
+              };
+              box(0, tab.x);
+              if (atoms_here > 1) box(1, tab.y);
+              if (atoms_here > 2) box(2, tab.z);
+              if (atoms_here > 3) box(3, tab.w);
+            } else {
+              tma_load_2d(smA + s * GEMM_A_STAGE, &tmA, &sh->full[s], ks * 128, m0);
+            }
           }
-          if (!W4 && lane == 4) tma_load_2d(smB + s * Cfg::B_STAGE, &tmB, &sh->full[s], ks * 128, n0);
-          if (++s == (uint32_t)STAGES) {
-            s = 0;
+          __syncwarp();
+          s += (uint32_t)producers;
+          if (s >= (uint32_t)STAGES) {
+            s -= (uint32_t)STAGES;
             empty_par ^= 1u;
           }
         }
+        ks -= n_kstages;
+        early = 0;
         if (*abort_flag) break;
       }
     }
     __syncwarp();
   } else if (warp == GEMM_WARP_MMA) {
     // ------------------------------------------------------------ MMA issuer
-    // The whole warp runs the loop with uniform control flow; the tcgen05 instructions are issued by
-    // one elected lane.  What the issuing path costs per instruction, not the tensor core, bounds short
-    // groups: an MMA, a commit and a barrier poll each take tens to hundreds of cycles of this warp's
-    // time, whatever the tile width.  So a stage is straight-line code chosen by its pattern of group
-    // ends (no per-atom tests), everything that can be is precomputed (descriptor words, barrier
-    // addresses, running ring positions and parities).
+    // The whole warp runs the loop with uniform control flow; the tcgen05 instructions are issued by one elected lane.
+    // A branch costs this warp 30-40 cycles, a barrier poll 50-100, and the tensor core queues only a couple of MMAs,
+    // so what the loop does between MMAs shows.  A short reduction, whose stages are full of group ends, runs
+    // straight-line stage bodies chosen by the pattern of ends.  A long one walks groups: through the stages in the
+    // middle of a group without a test of where groups end, and with the next stage's barrier polled ahead of the
+    // MMAs so that the poll's latency runs under them (350 cycles a stage against 520, of which the MMAs take 320;
+    // 2048 x 5120 -> 1280 W8 20.7 -> 19.3 us, conv 8 x 64 x 64 x 320 93 -> 78 us together with the second producer).
     {
       constexpr uint32_t A_HI = CONV ? smem_desc_hi(256, 6) : smem_desc_hi(1024, 2);
       constexpr uint32_t B_HI = smem_desc_hi(1024, 2);
@@ -276,6 +309,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       uint32_t full_phase = 0;   // parity of the slot's next "full" phase
       uint32_t ab = 0;           // accumulator of the next group
       uint32_t acc_phase = 1;    // parity to wait for on its "empty" barrier (fresh barriers pass)
+      uint32_t full_ready = 0;   // the slot's "full" phase has been seen to be complete
       // One stage of four atoms whose group ends are the bits of PAT; `need`: the first atom starts a group.
       auto issue_stage = [&](auto pat_tag, bool need, uint32_t a_lo, uint32_t b_lo) {
         constexpr int PAT = decltype(pat_tag)::value;
@@ -300,43 +334,123 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         }
       };
-      for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        bool need = true;      // every tile starts a group
-        uint64_t ends = 0;     // bit i: atom (16 * 4) * word + i is the last of its group
-        for (int ks = 0; ks < n_kstages; ++ks) {
-          if ((ks & 15) == 0) ends = a.end_mask[ks >> 4];
-          uint32_t pat = (uint32_t)(ends >> ((ks & 15) * 4)) & 0xFu;
-          // A ragged last stage still issues four atoms (the missing ones multiply zero weights); the
-          // end of the last group moves to the last atom issued.
-          const int atoms_here = n_atoms - ks * 4;
-          if (atoms_here < 4) pat = (pat & ~(1u << (atoms_here - 1))) | 8u;
-          mbar_wait_lean(full0 + s * 8u, full_phase, abort_flag);
-          tc_fence_after();
-          const uint32_t a_lo = a_lo0 + s * (uint32_t)(GEMM_A_STAGE >> 4);
-          const uint32_t b_lo = b_lo0 + s * (uint32_t)(Cfg::B_STAGE >> 4);
-          switch (pat) {
-#define DGQ_STAGE_CASE(P) case P: issue_stage(std::integral_constant<int, P>{}, need, a_lo, b_lo); break;
-            DGQ_STAGE_CASE(0) DGQ_STAGE_CASE(1) DGQ_STAGE_CASE(2) DGQ_STAGE_CASE(3) DGQ_STAGE_CASE(4) DGQ_STAGE_CASE(5)
-            DGQ_STAGE_CASE(6) DGQ_STAGE_CASE(7) DGQ_STAGE_CASE(8) DGQ_STAGE_CASE(9) DGQ_STAGE_CASE(10) DGQ_STAGE_CASE(11)
-            DGQ_STAGE_CASE(12) DGQ_STAGE_CASE(13) DGQ_STAGE_CASE(14) DGQ_STAGE_CASE(15)
-#undef DGQ_STAGE_CASE
-          }
-          need = (pat & 8u) != 0;
-          if (elect_one()) mma_commit_addr(empty0 + s * 8u);  // stage reusable once these MMAs have read it
-          __syncwarp();
-          if (++s == (uint32_t)STAGES) {
-            s = 0;
-            full_phase ^= 1u;
-          }
+      auto wait_full = [&]() {
+        if (!full_ready) mbar_wait_lean(full0 + s * 8u, full_phase, abort_flag);
+        full_ready = 0;
+        tc_fence_after();
+      };
+      auto next_slot = [&]() {
+        if (++s == (uint32_t)STAGES) {
+          s = 0;
+          full_phase ^= 1u;
         }
-        if (*abort_flag) break;
+      };
+      // N atoms of the current stage from atom j0 on; then the accumulator and / or the stage are handed over
+      auto issue = [&](auto n_tag, uint32_t j0, uint32_t acc, bool group_done, bool stage_done) {
+        constexpr int N_ATOMS = decltype(n_tag)::value;
+        const uint32_t a_lo = a_lo0 + s * (uint32_t)(GEMM_A_STAGE >> 4) + j0 * (CONV ? 256u : 2u);
+        const uint32_t b_lo = b_lo0 + s * (uint32_t)(Cfg::B_STAGE >> 4) + j0 * 2u;
+        if (elect_one()) {
+#pragma unroll
+          for (int j = 0; j < N_ATOMS; ++j)
+            mma_i8_lohi(tmem_base + ab * (uint32_t)BN, a_lo + (CONV ? j * 256 : j * 2), A_HI, b_lo + j * 2, B_HI, idesc,
+                        j == 0 ? acc : 1u);
+          if (group_done) mma_commit_addr(accf0 + ab * 8u);
+          if (stage_done) mma_commit_addr(empty0 + s * 8u);  // stage reusable once these MMAs have read it
+        }
+        __syncwarp();
+      };
+      auto issue_n = [&](int n, uint32_t j0, uint32_t acc, bool group_done, bool stage_done) {
+        switch (n) {
+          case 1: issue(std::integral_constant<int, 1>{}, j0, acc, group_done, stage_done); break;
+          case 2: issue(std::integral_constant<int, 2>{}, j0, acc, group_done, stage_done); break;
+          case 3: issue(std::integral_constant<int, 3>{}, j0, acc, group_done, stage_done); break;
+          default: issue(std::integral_constant<int, 4>{}, j0, acc, group_done, stage_done); break;
+        }
+      };
+      if (n_kstages < GEMM_LONG_STAGES) {
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+          bool need = true;      // every tile starts a group
+          for (int ks = 0; ks < n_kstages; ++ks) {
+            uint32_t pat = (uint32_t)(a.end_mask >> (ks * 4)) & 0xFu;
+            // A ragged last stage still issues four atoms (the missing ones multiply zero weights); the
+            // end of the last group moves to the last atom issued.
+            const int atoms_here = n_atoms - ks * 4;
+            if (atoms_here < 4) pat = (pat & ~(1u << (atoms_here - 1))) | 8u;
+            mbar_wait_lean(full0 + s * 8u, full_phase, abort_flag);
+            tc_fence_after();
+            const uint32_t a_lo = a_lo0 + s * (uint32_t)(GEMM_A_STAGE >> 4);
+            const uint32_t b_lo = b_lo0 + s * (uint32_t)(Cfg::B_STAGE >> 4);
+            switch (pat) {
+#define DGQ_STAGE_CASE(P) case P: issue_stage(std::integral_constant<int, P>{}, need, a_lo, b_lo); break;
+              DGQ_STAGE_CASE(0) DGQ_STAGE_CASE(1) DGQ_STAGE_CASE(2) DGQ_STAGE_CASE(3) DGQ_STAGE_CASE(4) DGQ_STAGE_CASE(5)
+              DGQ_STAGE_CASE(6) DGQ_STAGE_CASE(7) DGQ_STAGE_CASE(8) DGQ_STAGE_CASE(9) DGQ_STAGE_CASE(10) DGQ_STAGE_CASE(11)
+              DGQ_STAGE_CASE(12) DGQ_STAGE_CASE(13) DGQ_STAGE_CASE(14) DGQ_STAGE_CASE(15)
+#undef DGQ_STAGE_CASE
+            }
+            need = (pat & 8u) != 0;
+            if (elect_one()) mma_commit_addr(empty0 + s * 8u);  // stage reusable once these MMAs have read it
+            __syncwarp();
+            if (++s == (uint32_t)STAGES) {
+              s = 0;
+              full_phase ^= 1u;
+            }
+          }
+          if (*abort_flag) break;
+        }
+      } else {
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+          int atom = 0;
+#pragma unroll 1
+          for (int g = 0; g < a.G; ++g) {
+            const int end = a.seg_end[g];
+            mbar_wait_lean(acce0 + ab * 8u, acc_phase, abort_flag);
+            tc_fence_after();
+            uint32_t acc = 0u;  // the group's first MMA starts the accumulator
+            // what is left of a stage that the group before has begun
+            const int j0 = atom & 3;
+            if (j0 != 0) {
+              const int n = min(4 - j0, end - atom);
+              atom += n;
+              const bool stage_done = (atom & 3) == 0 || atom == n_atoms;
+              issue_n(n, (uint32_t)j0, 0u, atom == end, stage_done);
+              acc = 1u;
+              if (stage_done) next_slot();
+            }
+            // stages in the middle of the group: most of a long reduction
+#pragma unroll 1
+            while (end - atom > 4) {
+              wait_full();
+              const uint32_t ns = s + 1 == (uint32_t)STAGES ? 0u : s + 1;
+              full_ready = mbar_test_addr(full0 + ns * 8u, ns == 0 ? full_phase ^ 1u : full_phase);
+              issue(std::integral_constant<int, 4>{}, 0u, acc, false, true);
+              acc = 1u;
+              atom += 4;
+              s = ns;
+              if (ns == 0) full_phase ^= 1u;
+            }
+            if (atom < end) {  // the group's last stage
+              wait_full();
+              const int n = end - atom;
+              atom = end;
+              const bool stage_done = n == 4 || atom == n_atoms;
+              issue_n(n, 0u, acc, true, stage_done);
+              if (stage_done) next_slot();
+            }
+            if (++ab == (uint32_t)NACC) {
+              ab = 0;
+              acc_phase ^= 1u;
+            }
+          }
+          if (*abort_flag) break;
+        }
       }
     }
     __syncwarp();
   } else if (warp == GEMM_WARP_STORE) {
     // ------------------------------------------------------------ output store
+    pdl_wait();
     if (lane == 0) {
-      tma_prefetch_desc(&tmY);
       const uint32_t out_full_a = smem_u32(&sh->out_full);
       uint32_t tile_it = 0;
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tile_it) {
@@ -354,7 +468,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       bulk_wait0();
     }
     __syncwarp();
-  } else if (W4 && warp >= GEMM_WARP_STORE + 1) {
+  } else if (W4 && warp >= GEMM_WARP_TMA2) {
     // ------------------------------------------------------------ 4-bit weight unpack into the B stage
     // Every thread owns the same 16-byte pieces of every stage.  It copies them asynchronously from global
     // memory into its slots of the packed ring PK_AHEAD stages before it expands them, one copy group per
@@ -480,6 +594,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if ((CW % 32) >= 16) tmem_ld16(taddr + (CW / 32) * 32, reinterpret_cast<uint32_t(&)[16]>(rb[(CW / 32) * 32]));
       if (CW % 16) tmem_ld8(taddr + (CW / 16) * 16, reinterpret_cast<uint32_t(&)[8]>(rb[(CW / 16) * 16]));
     };
+    pdl_wait();
     if ((int)blockIdx.x < n_tiles) prefetch_tile(blockIdx.x);
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tile_it) {
       const float* srow_t = srow;
@@ -717,6 +832,7 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   a.P = g->P;
   a.use_zp = (layout == DGQ_CODES_U8);
   a.code_max = (1 << g->bits) - 1;
+  a.b_early = !expand_first;
   a.res_mask = w->res_mask;
   a.wres = w->d_wres;
   a.row_group = g->d_row_group;
@@ -725,20 +841,27 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   a.bias = (const __half*)bias;
   a.w_packed = (const uint8_t*)w->d_w;
   if (w->Kt / DGQ_K_ATOM > GEMM_MAX_ATOMS) return DGQ_ERR_UNSUPPORTED;
-  for (int k = 0; k < g->G; ++k) a.end_mask[(w->seg_end[k] - 1) >> 6] |= 1ull << ((w->seg_end[k] - 1) & 63);
+  if (w->Kt <= 128 * (GEMM_LONG_STAGES - 1))
+    for (int k = 0; k < g->G; ++k) a.end_mask |= 1ull << (w->seg_end[k] - 1);
   for (int k = 0; k < g->G; ++k) {
     a.seg_end[k] = w->seg_end[k];
-    a.grp_atoms[k] = (g->group_off[k + 1] - g->group_off[k]) / DGQ_K_ATOM;
+    a.grp_atoms[k] = w->atoms[k];
     a.grp_chan0[k] = g->group_off[k];
   }
+  int n_sm = 0;
+  DGQ_CUDA_OK(sm_count(&n_sm));
+  a.n_tiles_m = (int)((M + GEMM_BM - 1) / GEMM_BM);
   int BN = 128;
   if (w->N % 160 == 0) BN = 160;
   else if (w->N <= 64) BN = 64;
+  // A problem that would leave more than half of the SMs without a tile takes narrow ones: the serial work of a CTA
+  // (rounds over the groups, output) shrinks with its columns (256 x 320 -> 320: 7.2 -> 5.4 us, 616 x 768 -> 1280 W4:
+  // 11.7 -> 10.1 us, 512 x 5120 -> 1280: 17.7 -> 15.4 us, conv 8 x 8 x 8 x 1280: 56 -> 46 us).
+  if ((int64_t)a.n_tiles_m * ((w->N + BN - 1) / BN) * 2 <= n_sm) BN = 64;
   // instruction descriptor of kind::i8: int32 accumulator (bits 4-5 = 2), A format bit 7 (0 = u8,
   // 1 = s8), B format bit 10 = 1 (s8), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
   a.idesc = (2u << 4) | ((layout == DGQ_CODES_S8_CENTRED ? 1u : 0u) << 7) | (1u << 10) |
             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(GEMM_BM >> 4) << 24);
-  a.n_tiles_m = (int)((M + GEMM_BM - 1) / GEMM_BM);
   a.n_tiles_n = (w->N + BN - 1) / BN;
 
   CUtensorMap tmA, tmB, tmY;
@@ -788,9 +911,6 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
     const uint32_t box[2] = {128u, (uint32_t)BN};
     if (!encode_map(&tmB, wb, 2, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B)) return DGQ_ERR_CUDA;
   }
-  int dev = 0, n_sm = 148;
-  DGQ_CUDA_OK(cudaGetDevice(&dev));
-  DGQ_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
   // a multiple of the number of column blocks, so that every CTA keeps one column block
   if (a.n_tiles_n > n_sm) return DGQ_ERR_UNSUPPORTED;
   const int grid = std::min(a.n_tiles_m, n_sm / a.n_tiles_n) * a.n_tiles_n;

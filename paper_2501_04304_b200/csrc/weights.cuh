@@ -15,6 +15,7 @@ struct dgq_weight {
   int N_pad = 0;                 // N rounded up to a multiple of 256 (rows beyond N are zero)
   int Kt = 0;                    // length of the GEMM reduction in padded positions (multiple of 32)
   std::vector<int32_t> seg_end;  // [G] end of every group's segment, in 32-position atoms
+  std::vector<int32_t> atoms;    // [G] atoms of every group (of one filter tap)
   std::vector<float> sw;         // host scales [N]
   unsigned char* d_slab = nullptr;  // all device arrays below
   int8_t* d_w = nullptr;         // 8-bit: [N_pad][Kt] s8; 4-bit: [N_pad][Kt/2] packed
@@ -36,6 +37,7 @@ struct WeightArgs {
   int N, K, C, G, N_pad, Kt, K_pad, taps, qmax, four_bit;
   const int16_t* perm;   // [K_pad] channel of every padded position, -1 = padding
   int group_off[DGQ_MAX_GROUPS + 1];  // first padded position of every group
+  int red_off[DGQ_MAX_GROUPS + 1];    // the same in the reduction, for one tap
   uint8_t* w;            // outputs, see dgq_weight
   float *sw, *wsum, *wres;
   float* sw_out;         // [N] scales as the caller sees them
@@ -46,8 +48,8 @@ struct WeightArgs {
 // reduction is group-major, inside a group tap-major, then the group's padded positions.
 __device__ __forceinline__ int weight_codes8(const WeightArgs& a, const int8_t* row, int pos, int (&c)[8], int& first_pad) {
   int g = 0;
-  while (pos >= a.taps * a.group_off[g + 1]) ++g;
-  const int len = a.group_off[g + 1] - a.group_off[g], local = pos - a.taps * a.group_off[g];
+  while (pos >= a.taps * a.red_off[g + 1]) ++g;
+  const int len = a.red_off[g + 1] - a.red_off[g], local = pos - a.taps * a.red_off[g];
   const int tap = local / len, p0 = a.group_off[g] + local - tap * len;
   const int8_t* src = row + tap * a.C;
   const uint4 pv = __ldg(reinterpret_cast<const uint4*>(a.perm + p0));
@@ -208,9 +210,19 @@ static dgq_status weight_build(const dgq_groups* g, const __half* W, const int8_
   w->w_bits = w_bits;
   w->is_conv = conv ? 1 : 0;
   w->N_pad = (N + 255) / 256 * 256;
-  w->Kt = taps * g->K_pad;
+  // A linear layer's reduction is the padded code row.  A conv has no use for an atom that holds only padding
+  // (zero-centred codes: it would add zeros), so its reduction leaves those out: 18 of 22 atoms per tap
+  // remain for 320 channels in 16 groups.
   w->seg_end.resize(g->G);
-  for (int k = 0; k < g->G; ++k) w->seg_end[k] = taps * g->group_off[k + 1] / DGQ_K_ATOM;
+  w->atoms.resize(g->G);
+  for (int k = 0; k < g->G; ++k) {
+    int members = 0;
+    while (g->perm[g->group_off[k] + members] >= 0) ++members;  // every group ends in padding
+    w->atoms[k] = conv ? std::max(1, (members + DGQ_K_ATOM - 1) / DGQ_K_ATOM) : (g->group_off[k + 1] - g->group_off[k]) / DGQ_K_ATOM;
+    a.red_off[k + 1] = a.red_off[k] + w->atoms[k] * DGQ_K_ATOM;
+    w->seg_end[k] = taps * a.red_off[k + 1] / DGQ_K_ATOM;
+  }
+  w->Kt = taps * a.red_off[g->G];
 
   size_t bytes = 0;
   auto part = [&](size_t n) {
@@ -240,7 +252,7 @@ static dgq_status weight_build(const dgq_groups* g, const __half* W, const int8_
     for (int k = 0; k < g->G; ++k)
       for (int p = g->group_off[k]; p < g->group_off[k + 1]; ++p)
         if (g->perm[p] >= 0)
-          chan[g->perm[p]] = make_int2((taps - 1) * g->group_off[k] + p, g->group_off[k + 1] - g->group_off[k]);
+          chan[g->perm[p]] = make_int2(taps * a.red_off[k] + p - g->group_off[k], a.red_off[k + 1] - a.red_off[k]);
     ok(cudaMemcpyAsync(w->d_chan, chan.data(), chan.size() * sizeof(int2), cudaMemcpyHostToDevice, stream));
     if (wq) {
       a.wq = d_codes;

@@ -96,3 +96,33 @@ def test_quantizer_edges(M, sizes, bits, mode):
     group_of = np.repeat(np.arange(G), np.diff(ex["group_off"]))
     assert np.array_equal(full[:, ~valid], np.clip(z_rows, 0, L)[:, group_of[~valid]])   # padding = clamped zero-point
     assert b.device_status() == 0
+
+
+@pytest.mark.parametrize("M,N,sizes", [
+    (130, 64, (856,)),                       # 27 atoms: the longest reduction of one producer
+    (130, 64, (24, 856)),                    # 28 atoms, a group that ends inside a stage
+    (130, 64, (24, 880, 8)),                 # 30 atoms: the shortest of two producers, ragged last stage
+    (300, 320, (56, 2000, 24, 24, 88, 600)),  # long reduction whose groups begin at every atom of a stage
+    (2500, 1280, (120, 1000, 24)),           # more tiles than half the SMs: wide tiles, several per block
+])
+def test_linear_reduction_lengths(M, N, sizes):
+    torch, b = gpu()
+    C, G = sum(sizes), len(sizes)
+    rng = np.random.default_rng(C)
+    cg = rng.permutation(np.repeat(np.arange(G), sizes)).astype(np.int32)
+    scale = rng.uniform(0.01, 0.05, (1, 1, G)).astype(np.float32)
+    zp = rng.integers(100, 140, (1, 1, G)).astype(np.int32)
+    g = b.groups_from_host(C, 1, 8, cg, np.zeros(1, np.int32), scale, zp)
+    W = rng.normal(0, 0.02, (N, C)).astype(np.float16)
+    bias = rng.normal(0, 0.01, N).astype(np.float16)
+    wq, sw = ol.weight_rtn(W, 8)
+    w = b.weight_prepare(g, to_dev(torch, W), 8)
+    X = rng.normal(0, 1, (M, C)).astype(np.float16)
+    codes, s_rows, z_rows = ol.quantize_dynamic_token(X, cg, G, 8)
+    Xq, ds, dz = b.quantize_act(g, to_dev(torch, X), mode=b.MODE_DYNAMIC_TOKEN)
+    Y = torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda")
+    b.linear(g, w, Xq, mode=b.MODE_DYNAMIC_TOKEN, dyn_scale=ds, dyn_zp=dz, bias=to_dev(torch, bias), out=Y)
+    rows = np.unique(np.r_[0:3, M // 2, M - 3:M])
+    ref = ol.group_linear(codes[rows], s_rows[rows], z_rows[rows], cg, wq, sw, bias)
+    check_output(Y[torch.from_numpy(rows).cuda()], ref)
+    assert torch.isfinite(Y).all() and b.device_status() == 0

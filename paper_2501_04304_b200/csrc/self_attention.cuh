@@ -133,6 +133,12 @@ __device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
 }
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // kind::f16 instruction descriptor: fp32 accumulator (bits 4-5 = 1), fp16 A and B (format 0), B major at
 // bit 16 (1 = MN-major), N >> 3 at bit 17, M >> 4 at bit 24.
 __host__ __device__ constexpr uint32_t satc_idesc(int n, bool b_mn_major) {
@@ -234,11 +240,14 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     }
     __syncwarp();
   } else if (warp == SATC_WARP_MMA) {
-    // ------------------------------------------------------------ score issuer (one lane)
+    // ------------------------------------------------------------ score issuer
+    // Both issuing warps run their loops as a whole with uniform control flow, and one elected lane issues a tile's
+    // MMAs and commits in one block: issued from a loop that a single lane runs, with its addresses in per-lane
+    // registers, every MMA cost about twice as much of the warp's time.
     // Score tiles are numbered g = 0 .. N_WALKS * per_walk - 1 in the order (walk, key block, query
     // tile) and alternate between the two score buffers; a tile is issued as soon as its buffer has
     // been read, which is early in the arithmetic of tile g - 2.
-    if (lane == 0) {
+    {
       constexpr uint32_t IDESC_QK = satc_idesc(SATC_BK, false);
       constexpr uint32_t HI = smem_desc_hi(1024, 2);
       const uint32_t q_lo = smem_desc_lo(smem_u32(sQ)), k_lo = smem_desc_lo(smem_u32(sK));
@@ -254,27 +263,29 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         mbar_wait_lean(s_free0 + sb * 8u, (((uint32_t)g >> 1) & 1u) ^ 1u, abort_flag);
         tc_fence_after();
         const uint32_t a_lo = q_lo + t * (uint32_t)(Cfg::TILE >> 4), b_lo = k_lo + ks * (uint32_t)(Cfg::TILE >> 4);
+        const bool k_done = t == NT - 1;
+        if (elect_one()) {
 #pragma unroll
-        for (int kstep = 0; kstep < Cfg::KSTEPS; ++kstep) {
-          const uint32_t off = (uint32_t)(((kstep >> 2) * SATC_PANEL + (kstep & 3) * 32) >> 4);
-          mma_f16_lohi(tmem_base + sb * SATC_BK, a_lo + off, HI, b_lo + off, HI, IDESC_QK, kstep > 0 ? 1u : 0u);
-        }
-        if (t == NT - 1) {
-          mma_commit_addr(k_empty0 + ks * 8u);
-          if (++ks == (uint32_t)KST) {
-            ks = 0;
-            k_par ^= 1u;
+          for (int kstep = 0; kstep < Cfg::KSTEPS; ++kstep) {
+            const uint32_t off = (uint32_t)(((kstep >> 2) * SATC_PANEL + (kstep & 3) * 32) >> 4);
+            mma_f16_lohi(tmem_base + sb * SATC_BK, a_lo + off, HI, b_lo + off, HI, IDESC_QK, kstep > 0 ? 1u : 0u);
           }
+          mma_commit_addr(s_full0 + sb * 8u);
+          if (k_done) mma_commit_addr(k_empty0 + ks * 8u);
         }
-        mma_commit_addr(s_full0 + sb * 8u);
+        __syncwarp();
+        if (k_done && ++ks == (uint32_t)KST) {
+          ks = 0;
+          k_par ^= 1u;
+        }
         if ((g & 7) == 7 && *abort_flag) break;
       }
     }
     __syncwarp();
   } else if (warp == SATC_WARP_PV) {
-    // ------------------------------------------------------------ product issuer (one lane)
+    // ------------------------------------------------------------ product issuer
     // O(tile) += P V for the tiles of the codes walk, each as soon as its P tile is complete.
-    if (lane == 0) {
+    {
       constexpr uint32_t IDESC_PV = satc_idesc(Cfg::DP, true);
       constexpr uint32_t HI = smem_desc_hi(1024, 2);
       const uint32_t v_lo = ((smem_u32(sV) & 0x3FFFFu) >> 4) | ((uint32_t)(SATC_PANEL >> 4) << 16);  // MN-major: block stride
@@ -289,25 +300,27 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         const uint32_t a_tmem = tmem_base + SATC_TMEM_P + pb * 64u, b_lo = v_lo + vs * (uint32_t)(Cfg::TILE >> 4);
         const uint32_t d_tmem = tmem_base + Cfg::TMEM_O + t * Cfg::DP;
         const uint32_t acc0 = c >= NT ? 1u : 0u;  // the first key block starts the accumulator
+        const bool v_done = t == NT - 1;
+        if (elect_one()) {
 #pragma unroll
-        for (int kstep = 0; kstep < SATC_BK / 16; ++kstep)
-          mma_f16_ts(d_tmem, a_tmem + (uint32_t)(kstep * 8), b_lo + (uint32_t)((kstep * 2048) >> 4), HI, IDESC_PV,
-                     kstep > 0 ? 1u : acc0);
-        if (t == NT - 1) {
-          mma_commit_addr(v_empty0 + vs * 8u);
-          if (++vs == (uint32_t)VST) {
-            vs = 0;
-            v_par ^= 1u;
-          }
+          for (int kstep = 0; kstep < SATC_BK / 16; ++kstep)
+            mma_f16_ts(d_tmem, a_tmem + (uint32_t)(kstep * 8), b_lo + (uint32_t)((kstep * 2048) >> 4), HI, IDESC_PV,
+                       kstep > 0 ? 1u : acc0);
+          mma_commit_addr(p_free0 + pb * 8u);
+          if (v_done) mma_commit_addr(v_empty0 + vs * 8u);
+          if (c == per_walk - 1) mma_commit_addr(smem_u32(&sh->o_full));
         }
-        mma_commit_addr(p_free0 + pb * 8u);
+        __syncwarp();
+        if (v_done && ++vs == (uint32_t)VST) {
+          vs = 0;
+          v_par ^= 1u;
+        }
         if (++pb == (uint32_t)PST) {
           pb = 0;
           p_par ^= 1u;
         }
         if ((c & 7) == 7 && *abort_flag) break;
       }
-      mma_commit_addr(smem_u32(&sh->o_full));
     }
     __syncwarp();
   } else {
@@ -316,12 +329,13 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const int row = q * 32 + lane;  // row of a query tile
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
     const float scale = a.qk_scale_log2;
-    const unsigned long long nscale2 = pack_f32x2(-scale, -scale);
+    const unsigned long long scale2 = pack_f32x2(scale, scale), nscale2 = pack_f32x2(-scale, -scale);
     const unsigned long long one2 = pack_f32x2(1.f, 1.f);
     const unsigned long long magic2 = pack_f32x2(12582912.0f, 12582912.0f);
     const uint32_t L = (1u << a.bits) - 1u;
     const uint32_t code_top = 0x4B400000u + L;                                 // bits of 1.5 * 2^23 + last code
     const uint32_t p_top = 0x4B400000u + min(L, (uint32_t)AT_CODE_CAP);       // ... + last code with a non-zero fp16 weight
+    const uint32_t p_least = (127u + (uint32_t)AT_P_SHIFT - min(L, 100u)) << 23;  // weight of the last code
     float m_raw[NT], m2[NT], base[NT];
     unsigned long long zsum2[NT];
 #pragma unroll
@@ -369,9 +383,9 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           if (walk_max) {
             float mx0 = m_raw[t], mx1 = -INFINITY;
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-              mx0 = fmaxf(mx0, __uint_as_float(r[i]));
-              mx1 = fmaxf(mx1, __uint_as_float(r[i + 1]));
+            for (int i = 0; i < 32; i += 4) {
+              mx0 = max3(mx0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+              mx1 = max3(mx1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
             }
             m_raw[t] = fmaxf(mx0, mx1);
           } else if (!walk_codes) {
@@ -387,26 +401,49 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             const uint32_t pb = c % PST;
             const int64_t code_row =
                 (((int64_t)b * a.H + h) * a.nq + row0 + t * SATC_BQ + row) * a.nk + j * SATC_BK + cp * 32;
-            const unsigned long long base2 = pack_f32x2(base[t], base[t]);
             uint32_t pk[16];
             unsigned long long zs = zsum2[t];
-            {
+            if (!FIXED) {
+              // e = 2^(14 - x) with x = base - t * scale >= 0 up to rounding (the row maximum has code 0); -inf logits (keys
+              // beyond nk) give 0.  The row sum takes e as it is.  The power of two nearest to it in the log domain,
+              // 2^(14 - rint(x)), is e with the mantissa rounded at sqrt(2): adding 2 - sqrt(2) in mantissa units carries into
+              // the exponent where x is nearer to the smaller code, and the mantissa is cut off.  One exponential and two
+              // integer operations per score serve row sum and weight (with the code formed first, by an add of
+              // 1.5 * 2^23, a clamp, a shift and a subtraction, a score took half again as many instructions).
+              const unsigned long long shift2 = pack_f32x2(AT_P_SHIFT - base[t], AT_P_SHIFT - base[t]);
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
-                // x = base - t * scale >= 0 up to rounding (the row maximum has code 0); -inf logits (keys
-                // beyond nk) give +inf, which the integer minimum below clamps to the last code
-                unsigned long long x2 = fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), nscale2, base2);
+                const unsigned long long x2 = fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), scale2, shift2);
                 float x0, x1;
                 unpack_f32x2(x2, x0, x1);
-                if (!FIXED) {
-                  // 2^(t - max) = 2^-x for the row sum
-                  zs = fma_f32x2(pack_f32x2(ex2_approx(-x0), ex2_approx(-x1)), one2, zs);
-                } else {
-                  x2 = pack_f32x2(fmaxf(x0, 0.f), fmaxf(x1, 0.f));  // a fixed scale can lie below a score
+                const float e0 = ex2_approx(x0), e1 = ex2_approx(x1);
+                zs = fma_f32x2(pack_f32x2(e0, e1), one2, zs);
+                uint32_t b0 = (__float_as_uint(e0) + 0x004AFB0Du) & 0xFF800000u, b1 = (__float_as_uint(e1) + 0x004AFB0Du) & 0xFF800000u;
+                if (CODES) {
+                  // exponent field 127 + 14 - code; where e has left the fp32 range the code comes from x itself
+                  const uint32_t c0 = x0 > -100.f ? 141u - (b0 >> 23) : __float_as_uint(fminf(AT_P_SHIFT - x0, 255.f) + 12582912.0f) & 0xFFu;
+                  const uint32_t c1 = x1 > -100.f ? 141u - (b1 >> 23) : __float_as_uint(fminf(AT_P_SHIFT - x1, 255.f) + 12582912.0f) & 0xFFu;
+                  r[i] = min(c0, L);
+                  r[i + 1] = min(c1, L);
                 }
+                if (L < (uint32_t)AT_CODE_CAP) {  // (beyond, the last code's weight is an fp16 zero)
+                  b0 = max(b0, p_least);
+                  b1 = max(b1, p_least);
+                }
+                const __half2 ph = __floats2half2_rn(__uint_as_float(b0), __uint_as_float(b1));
+                pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&ph);  // key i in the low half
+              }
+            } else {
+              const unsigned long long base2 = pack_f32x2(base[t], base[t]);
+#pragma unroll
+              for (int i = 0; i < 32; i += 2) {
+                // x = base - t * scale; a fixed scale can lie below a score; -inf logits give +inf, which the integer minimum
+                // below clamps to the last code
+                float x0, x1;
+                unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), nscale2, base2), x0, x1);
                 // rint by adding 1.5 * 2^23: the low bits of the sum are the integer
                 float y0, y1;
-                unpack_f32x2(fma_f32x2(x2, one2, magic2), y0, y1);
+                unpack_f32x2(fma_f32x2(pack_f32x2(fmaxf(x0, 0.f), fmaxf(x1, 0.f)), one2, magic2), y0, y1);
                 const uint32_t b0 = __float_as_uint(y0), b1 = __float_as_uint(y1);
                 if (CODES) {
                   r[i] = min(b0, code_top) & 0xFFu;
@@ -416,7 +453,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 const float p0 = __uint_as_float(0x46800000u - (min(b0, p_top) << 23));
                 const float p1 = __uint_as_float(0x46800000u - (min(b1, p_top) << 23));
                 const __half2 ph = __floats2half2_rn(p0, p1);
-                pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&ph);  // key i in the low half
+                pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&ph);
               }
             }
             zsum2[t] = zs;
@@ -470,7 +507,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);
         s_row[t] = 1.0f / ((zpart[row] + zpart[SATC_BQ + row]) + (zpart[2 * SATC_BQ + row] + zpart[3 * SATC_BQ + row]));
       }
-      s_row[t] *= 6.103515625e-05f;  // 2^-14
+      if (FIXED) s_row[t] *= 6.103515625e-05f;  // 2^-14 (the row sum of the other case carries it)
     }
     mbar_wait_lean(smem_u32(&sh->o_full), 0, abort_flag);
     __syncwarp();

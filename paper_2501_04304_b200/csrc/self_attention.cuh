@@ -11,8 +11,8 @@
 //   walk "codes" : S again; code = rint(base - t) in the log domain, P = 2^(14 - code) as fp16 into
 //                  tensor memory, O += P V on the tensor cores with P read from there.  With the row maximum as
 //                  scale the codes do not depend on the row sum, which is then gathered in this walk.
-// Roles: 16 softmax warps (warp w reads tensor-memory lanes 32 (w % 4) .. +31, columns 32 (w / 4) .. +31
-// of every score tile), one TMA producer lane, one lane that issues the score MMAs and one that issues
+// Roles: 16 softmax warps in two teams that take the score tiles in turn (warp w reads tensor-memory lanes 32 (w % 4) ..
+// +31 and half of the 128 columns of its team's tiles), one TMA producer lane, one lane that issues the score MMAs and one that issues
 // the P V MMAs (each tile costs an issuing thread a chain of dependent instructions, so the two run apart).  With two query tiles the softmax
 // warps alternate between them, so every K / V block fetched from L2 serves 256 query rows and one
 // tile's MMAs run under the other tile's arithmetic.  Q, K and P are K-major operands with 128-byte
@@ -58,6 +58,13 @@ struct SaTcCfg {
   // P = 2^(14 - code) as fp16 lives in tensor memory (64 columns per tile of 128 keys) and is the A
   // operand of P V from there: two tiles in flight where the accumulators leave room
   static constexpr int PST = (SATC_TMEM_P + 128 + NT * DP <= 512) ? 2 : 1;
+  // The softmax warps form two teams of eight that take the score tiles in turn, so that one team's waits, tensor-memory
+  // round trips and hand-overs run under the other's arithmetic; with a single P tile they stay together.
+  static constexpr int TEAMS = PST;
+  static constexpr int TEAM_WARPS = SATC_SOFTMAX_WARPS / TEAMS;
+  static constexpr int SPLIT = TEAM_WARPS / 4;          // warps of a team that share 32 rows of a tile
+  static constexpr int COLS = SATC_BK / SPLIT;          // score columns of a warp
+  static constexpr int PARTS = NT == 2 ? SPLIT : 4;     // threads that hold a part of a row's statistics
   static constexpr int TMEM_O = SATC_TMEM_P + PST * 64;
   static constexpr int TILE = NP * SATC_PANEL;
   static constexpr int OFF_K = NT * TILE;
@@ -184,8 +191,8 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       mbar_init(&sh->v_full[i], 1);
       mbar_init(&sh->v_empty[i], 1);
       mbar_init(&sh->s_full[i], 1);
-      mbar_init(&sh->s_free[i], SATC_SOFTMAX_WARPS);
-      mbar_init(&sh->p_full[i], SATC_SOFTMAX_WARPS);
+      mbar_init(&sh->s_free[i], Cfg::TEAM_WARPS);
+      mbar_init(&sh->p_full[i], Cfg::TEAM_WARPS);
       mbar_init(&sh->p_free[i], 1);
     }
     mbar_init(&sh->o_full, 1);
@@ -291,10 +298,11 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       const uint32_t v_lo = ((smem_u32(sV) & 0x3FFFFu) >> 4) | ((uint32_t)(SATC_PANEL >> 4) << 16);  // MN-major: block stride
       const uint32_t p_full0 = smem_u32(&sh->p_full[0]), p_free0 = smem_u32(&sh->p_free[0]);
       const uint32_t v_full0 = smem_u32(&sh->v_full[0]), v_empty0 = smem_u32(&sh->v_empty[0]);
-      uint32_t pb = 0, p_par = 0, vs = 0, v_par = 0;
+      // P tiles lie in the buffer of the team that made them (tile g of all walks: team g % 2)
+      uint32_t pb = PST == 2 ? (uint32_t)((N_WALKS - 1) * per_walk) & 1u : 0u, p_par = 0, vs = 0, v_par = 0;
       for (int c = 0; c < per_walk; ++c) {
         const uint32_t t = NT == 2 ? ((uint32_t)c & 1u) : 0u;
-        mbar_wait_lean(p_full0 + pb * 8u, p_par, abort_flag);
+        mbar_wait_lean(p_full0 + pb * 8u, (p_par >> pb) & 1u, abort_flag);
         if (t == 0) mbar_wait_lean(v_full0 + vs * 8u, v_par, abort_flag);
         tc_fence_after();
         const uint32_t a_tmem = tmem_base + SATC_TMEM_P + pb * 64u, b_lo = v_lo + vs * (uint32_t)(Cfg::TILE >> 4);
@@ -315,18 +323,19 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           vs = 0;
           v_par ^= 1u;
         }
-        if (++pb == (uint32_t)PST) {
-          pb = 0;
-          p_par ^= 1u;
-        }
+        p_par ^= 1u << pb;
+        if (PST == 2) pb ^= 1u;
         if ((c & 7) == 7 && *abort_flag) break;
       }
     }
     __syncwarp();
   } else {
     // ------------------------------------------------------------ softmax / quantizer warps
-    const int q = warp & 3, cp = warp >> 2;
+    constexpr int TEAMS = Cfg::TEAMS, SPLIT = Cfg::SPLIT, PARTS = Cfg::PARTS;
+    const int q = warp & 3, team = TEAMS == 2 ? warp >> 3 : 0, cp = (warp >> 2) % SPLIT;
     const int row = q * 32 + lane;  // row of a query tile
+    const int qt = NT == 2 ? team : 0;             // the query tile whose rows this thread holds
+    const int part = NT == 2 ? cp : warp >> 2;     // this thread's part of the row's statistics
     const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
     const float scale = a.qk_scale_log2;
     const unsigned long long scale2 = pack_f32x2(scale, scale), nscale2 = pack_f32x2(-scale, -scale);
@@ -336,73 +345,74 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t code_top = 0x4B400000u + L;                                 // bits of 1.5 * 2^23 + last code
     const uint32_t p_top = 0x4B400000u + min(L, (uint32_t)AT_CODE_CAP);       // ... + last code with a non-zero fp16 weight
     const uint32_t p_least = (127u + (uint32_t)AT_P_SHIFT - min(L, 100u)) << 23;  // weight of the last code
-    float m_raw[NT], m2[NT], base[NT];
-    unsigned long long zsum2[NT];
+    float m_raw = -INFINITY, m2 = 0.f, base = 0.f;
+    unsigned long long zs = 0ull;
+    // The threads that hold parts of a row's statistics leave them in shared memory and meet: the warps of a team when
+    // it has its own rows, else all of them.
+    auto meet = [&]() {
+      if (NT == 2) named_bar_sync(1 + team, Cfg::TEAM_WARPS * 32);
+      else named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);
+    };
+    float* my_m = mpart + (NT == 2 ? team * SPLIT * SATC_BQ : 0) + row;
+    float* my_z = zpart + (NT == 2 ? team * SPLIT * SATC_BQ : 0) + row;
+    auto row_sum = [&]() {
+      my_z[part * SATC_BQ] = __uint_as_float((uint32_t)zs) + __uint_as_float((uint32_t)(zs >> 32));
+      meet();
+      float z = my_z[0];
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      m_raw[t] = -INFINITY;
-      m2[t] = 0.f;
-      base[t] = 0.f;
-      zsum2[t] = 0ull;
-    }
-    uint32_t g = 0, c = 0;  // score tiles / codes-walk tiles seen so far
+      for (int i = 1; i < PARTS; ++i) z += my_z[i * SATC_BQ];
+      return z;
+    };
+    uint32_t n = 0, c = 0;  // tiles / codes-walk tiles of this team so far
     for (int w = 0; w < N_WALKS; ++w) {
       const bool walk_max = (w == 0), walk_codes = (w == N_WALKS - 1);
-      for (int j = 0; j < nb; ++j) {
-        const int valid = a.nk - j * SATC_BK - cp * 32;  // this warp's columns below `valid` are real keys
+      const int g0 = w * per_walk;
+      for (int g = TEAMS == 2 ? g0 + ((g0 ^ team) & 1) : g0; g < g0 + per_walk; g += TEAMS, ++n) {
+        const int j = (g - g0) / NT;
+        const uint32_t sb = (uint32_t)g & 1u;
+        // After a time-out every wait returns at once and the loops run to their ends on whatever the buffers hold (an
+        // error is recorded): no warp leaves early, so the named barriers are always reached by all their warps.
+        mbar_wait_lean(smem_u32(&sh->s_full[sb]), (TEAMS == 2 ? n : n >> 1) & 1u, abort_flag);
+        __syncwarp();
+        tc_fence_after();
 #pragma unroll
-        for (int t = 0; t < NT; ++t) {
-          const uint32_t sb = g & 1u;
-          // After a time-out every wait returns at once and the loops run to their ends on whatever the
-          // buffers hold (an error is recorded): no warp leaves early, so the named barriers below are
-          // always reached by all 16 warps.
-          mbar_wait_lean(smem_u32(&sh->s_full[sb]), (g >> 1) & 1u, abort_flag);
-          __syncwarp();
-          tc_fence_after();
+        for (int ch = 0; ch < Cfg::COLS / 32; ++ch) {
+          const int col = cp * Cfg::COLS + ch * 32;
+          const int valid = a.nk - j * SATC_BK - col;  // columns of this chunk below `valid` are real keys
           uint32_t r[32];
-          {
-            uint32_t r0[16], r1[16];
-            tmem_ld16(t_lane + sb * SATC_BK + cp * 32, r0);
-            tmem_ld16(t_lane + sb * SATC_BK + cp * 32 + 16, r1);
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              r[i] = r0[i];
-              r[16 + i] = r1[i];
-            }
+          tmem_ld32(t_lane + sb * SATC_BK + col, r);
+          tmem_ld_wait();
+          if (ch == Cfg::COLS / 32 - 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh->s_free[sb]);
           }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&sh->s_free[sb]);
-          ++g;
           if (valid < 32) {
 #pragma unroll
             for (int i = 0; i < 32; ++i)
               if (i >= valid) r[i] = 0xFF800000u;  // -inf
           }
           if (walk_max) {
-            float mx0 = m_raw[t], mx1 = -INFINITY;
+            float mx0 = m_raw, mx1 = -INFINITY;
 #pragma unroll
             for (int i = 0; i < 32; i += 4) {
               mx0 = max3(mx0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
               mx1 = max3(mx1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
             }
-            m_raw[t] = fmaxf(mx0, mx1);
+            m_raw = fmaxf(mx0, mx1);
           } else if (!walk_codes) {
             // row sums with the final maximum (fixed scale: the codes need them first)
             float z0 = 0.f, z1 = 0.f;
 #pragma unroll
             for (int i = 0; i < 32; i += 2) {
-              z0 += ex2_approx(fmaf(__uint_as_float(r[i]), scale, -m2[t]));
-              z1 += ex2_approx(fmaf(__uint_as_float(r[i + 1]), scale, -m2[t]));
+              z0 += ex2_approx(fmaf(__uint_as_float(r[i]), scale, -m2));
+              z1 += ex2_approx(fmaf(__uint_as_float(r[i + 1]), scale, -m2));
             }
-            zsum2[t] = pack_f32x2(__uint_as_float((uint32_t)zsum2[t]) + z0, __uint_as_float((uint32_t)(zsum2[t] >> 32)) + z1);
+            zs = pack_f32x2(__uint_as_float((uint32_t)zs) + z0, __uint_as_float((uint32_t)(zs >> 32)) + z1);
           } else {
-            const uint32_t pb = c % PST;
-            const int64_t code_row =
-                (((int64_t)b * a.H + h) * a.nq + row0 + t * SATC_BQ + row) * a.nk + j * SATC_BK + cp * 32;
+            const uint32_t pb = TEAMS == 2 ? sb : 0u;
+            const int64_t code_row = (((int64_t)b * a.H + h) * a.nq + row0 + qt * SATC_BQ + row) * a.nk + j * SATC_BK + col;
             uint32_t pk[16];
-            unsigned long long zs = zsum2[t];
             if (!FIXED) {
               // e = 2^(14 - x) with x = base - t * scale >= 0 up to rounding (the row maximum has code 0); -inf logits (keys
               // beyond nk) give 0.  The row sum takes e as it is.  The power of two nearest to it in the log domain,
@@ -410,7 +420,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
               // the exponent where x is nearer to the smaller code, and the mantissa is cut off.  One exponential and two
               // integer operations per score serve row sum and weight (with the code formed first, by an add of
               // 1.5 * 2^23, a clamp, a shift and a subtraction, a score took half again as many instructions).
-              const unsigned long long shift2 = pack_f32x2(AT_P_SHIFT - base[t], AT_P_SHIFT - base[t]);
+              const unsigned long long shift2 = pack_f32x2(AT_P_SHIFT - base, AT_P_SHIFT - base);
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
                 const unsigned long long x2 = fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), scale2, shift2);
@@ -434,7 +444,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&ph);  // key i in the low half
               }
             } else {
-              const unsigned long long base2 = pack_f32x2(base[t], base[t]);
+              const unsigned long long base2 = pack_f32x2(base, base);
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
                 // x = base - t * scale; a fixed scale can lie below a score; -inf logits give +inf, which the integer minimum
@@ -456,17 +466,20 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&ph);
               }
             }
-            zsum2[t] = zs;
-            // the P tile's previous product must have read it
-            mbar_wait_lean(smem_u32(&sh->p_free[pb]), ((c / PST) & 1u) ^ 1u, abort_flag);
-            __syncwarp();
-            tmem_st16(t_lane + SATC_TMEM_P + pb * 64u + cp * 16u, pk);
-            tmem_st_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&sh->p_full[pb]);
-            ++c;
-            if (CODES && row0 + t * SATC_BQ + row < a.nq) {
+            if (ch == 0) {  // the buffer's previous product must have read it
+              mbar_wait_lean(smem_u32(&sh->p_free[pb]), (c & 1u) ^ 1u, abort_flag);
+              __syncwarp();
+              tc_fence_after();
+            }
+            tmem_st16(t_lane + SATC_TMEM_P + pb * 64u + (uint32_t)(col >> 1), pk);
+            if (ch == Cfg::COLS / 32 - 1) {
+              tmem_st_wait();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&sh->p_full[pb]);
+              ++c;
+            }
+            if (CODES && row0 + qt * SATC_BQ + row < a.nq) {
 #pragma unroll
               for (int i = 0; i < 32; ++i)
                 if (i < valid) a.codes_out[code_row + i] = (uint8_t)r[i];
@@ -475,55 +488,34 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         }
       }
       if (walk_max) {
+        my_m[part * SATC_BQ] = m_raw;
+        meet();
 #pragma unroll
-        for (int t = 0; t < NT; ++t) {
-          if (t > 0) named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);  // the exchange buffer is read out
-          mpart[cp * SATC_BQ + row] = m_raw[t];
-          named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);
-          m_raw[t] = fmaxf(fmaxf(mpart[row], mpart[SATC_BQ + row]), fmaxf(mpart[2 * SATC_BQ + row], mpart[3 * SATC_BQ + row]));
-          m2[t] = m_raw[t] * scale;
-          base[t] = m2[t];  // row maximum as scale: log2 s + max + log2 sum = max
-        }
+        for (int i = 0; i < PARTS; ++i) m_raw = fmaxf(m_raw, my_m[i * SATC_BQ]);
+        m2 = m_raw * scale;
+        base = m2;  // row maximum as scale: log2 s + max + log2 sum = max
       } else if (!walk_codes) {
         const float log2_fixed = log2f(fmaxf(__ldg(a.fixed_scale + b), 1.17549435e-38f));
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-          if (t > 0) named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);
-          zpart[cp * SATC_BQ + row] = __uint_as_float((uint32_t)zsum2[t]) + __uint_as_float((uint32_t)(zsum2[t] >> 32));
-          named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);
-          const float z = (zpart[row] + zpart[SATC_BQ + row]) + (zpart[2 * SATC_BQ + row] + zpart[3 * SATC_BQ + row]);
-          base[t] = log2_fixed + m2[t] + log2f(z);
-        }
+        base = log2_fixed + m2 + log2f(row_sum());
       }
     }
-    float s_row[NT];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      if (FIXED) {
-        s_row[t] = fmaxf(__ldg(a.fixed_scale + b), 1.17549435e-38f);
-      } else {
-        if (t > 0) named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);
-        zpart[cp * SATC_BQ + row] = __uint_as_float((uint32_t)zsum2[t]) + __uint_as_float((uint32_t)(zsum2[t] >> 32));
-        named_bar_sync(1, SATC_SOFTMAX_WARPS * 32);
-        s_row[t] = 1.0f / ((zpart[row] + zpart[SATC_BQ + row]) + (zpart[2 * SATC_BQ + row] + zpart[3 * SATC_BQ + row]));
-      }
-      if (FIXED) s_row[t] *= 6.103515625e-05f;  // 2^-14 (the row sum of the other case carries it)
-    }
+    float s_row;
+    if (FIXED) s_row = fmaxf(__ldg(a.fixed_scale + b), 1.17549435e-38f) * 6.103515625e-05f;  // 2^-14
+    else s_row = 1.0f / row_sum();  // (the sum carries the 2^14)
     mbar_wait_lean(smem_u32(&sh->o_full), 0, abort_flag);
     __syncwarp();
     tc_fence_after();
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int orow = row0 + t * SATC_BQ + row;
+    {
+      const int orow = row0 + qt * SATC_BQ + row;
       __half* o_row = a.O + (((int64_t)b * a.nq + orow) * a.H + h) * D;
-      for (int ch = cp; ch < D / 8; ch += 4) {
+      for (int ch = part; ch < D / 8; ch += PARTS) {
         uint32_t o[8];
-        tmem_ld8(t_lane + Cfg::TMEM_O + t * Cfg::DP + ch * 8, o);
+        tmem_ld8(t_lane + Cfg::TMEM_O + qt * Cfg::DP + ch * 8, o);
         tmem_ld_wait();
         __half2 oh[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          oh[i] = __floats2half2_rn(s_row[t] * __uint_as_float(o[2 * i]), s_row[t] * __uint_as_float(o[2 * i + 1]));
+          oh[i] = __floats2half2_rn(s_row * __uint_as_float(o[2 * i]), s_row * __uint_as_float(o[2 * i + 1]));
         if (orow < a.nq) *(reinterpret_cast<uint4*>(o_row) + ch) = *reinterpret_cast<const uint4*>(oh);
       }
     }

@@ -30,13 +30,14 @@ constexpr int AT_THREADS = AT_WARPS * 32;
 constexpr float AT_P_SHIFT = 14.0f;  // A_hat / s is held in fp16 as 2^(14 - code)
 constexpr float AT_CODE_CAP = 40.0f; // 2^(14 - 40) is below half the smallest fp16: codes beyond it give 0
 
-template <int D, int NKP>
+// MT: 16-row tiles per warp (1 or 2; two need the registers that a wide head or a long context does not leave).
+template <int D, int NKP, int MT_>
 struct AttnCfg {
   static constexpr int DP = (D + 15) / 16 * 16;   // features padded to the MMA K step
   static constexpr int KS = DP / 16;
   static constexpr int LDK = DP + 8;              // row pitch of K and of a Q / O slab (halfs): conflict-free
   static constexpr int LDV = NKP * 16 + 8;        // row pitch of V^T (halfs)
-  static constexpr int MT = (D <= 64 && NKP <= 5) ? 2 : 1;  // 16-row tiles per warp (register budget)
+  static constexpr int MT = MT_;
   static constexpr int WROWS = 16 * MT;
   static constexpr int ROWS = AT_WARPS * WROWS;   // query rows per CTA
   static constexpr int NT = 2 * NKP;              // 8-key tiles
@@ -86,7 +87,7 @@ __device__ __forceinline__ int scope_index(const AttnArgs& a, int b, int h) {
 // all their latencies overlap.
 template <int D, int NKP>
 struct KStage {
-  static constexpr int VEC = AttnCfg<D, NKP>::LDK / 8;  // 16-byte pieces per row, padding included
+  static constexpr int VEC = AttnCfg<D, NKP, 1>::LDK / 8;  // 16-byte pieces per row, padding included
   static constexpr int N = (NKP * 16 * VEC + AT_THREADS - 1) / AT_THREADS;
 };
 template <int D, int NKP>
@@ -108,14 +109,14 @@ __device__ __forceinline__ void store_k(const uint4 (&x)[KStage<D, NKP>::N], __h
   for (int e = 0; e < KStage<D, NKP>::N; ++e) {
     const int i = threadIdx.x + e * AT_THREADS;
     const int j = i / VEC, v = i - j * VEC;
-    if (i < NKP * 16 * VEC) *reinterpret_cast<uint4*>(sK + j * AttnCfg<D, NKP>::LDK + v * 8) = x[e];
+    if (i < NKP * 16 * VEC) *reinterpret_cast<uint4*>(sK + j * AttnCfg<D, NKP, 1>::LDK + v * 8) = x[e];
   }
 }
 
 // The warp's query rows into its slab, rows beyond the valid ones and features beyond D zero.
-template <int D, int NKP>
+template <int D, int NKP, int MT>
 __device__ __forceinline__ void stage_q(const __half* q_base, int64_t q_stride, int rows_valid, __half* slab) {
-  using Cfg = AttnCfg<D, NKP>;
+  using Cfg = AttnCfg<D, NKP, MT>;
   constexpr int VEC = Cfg::DP / 8;
   constexpr int N = (Cfg::WROWS * VEC + 31) / 32;
   const int lane = threadIdx.x & 31;
@@ -150,10 +151,10 @@ __device__ __forceinline__ void ldmatrix_x2(uint32_t (&x)[2], const __half* row)
 
 // Base-2 logits of the warp's rows against all keys.  S[mt][nt][0..1]: row 16 mt + lane/4, keys
 // 8 nt + 2 (lane%4) + {0,1}; S[mt][nt][2..3]: row + 8.  Keys >= nk get -inf.
-template <int D, int NKP>
+template <int D, int NKP, int MT>
 __device__ __forceinline__ void logits_warp(const AttnArgs& a, const __half* slab, const __half* sK,
-                                            float (&S)[AttnCfg<D, NKP>::MT][2 * NKP][4]) {
-  using Cfg = AttnCfg<D, NKP>;
+                                            float (&S)[MT][2 * NKP][4]) {
+  using Cfg = AttnCfg<D, NKP, MT>;
   const int lane = threadIdx.x & 31;
   const int r = lane >> 2, c = lane & 3;
 #pragma unroll
@@ -202,9 +203,9 @@ __device__ __forceinline__ void logits_warp(const AttnArgs& a, const __half* sla
   }
 }
 
-template <int D, int NKP>
+template <int D, int NKP, int MT>
 __global__ void __launch_bounds__(AT_THREADS, 2) attn_phase1_kernel(const AttnArgs a) {
-  using Cfg = AttnCfg<D, NKP>;
+  using Cfg = AttnCfg<D, NKP, MT>;
   extern __shared__ __align__(16) unsigned char at_smem[];
   __half* sK = reinterpret_cast<__half*>(at_smem);
   __half* sQ = reinterpret_cast<__half*>(at_smem + Cfg::SM_K);
@@ -222,13 +223,13 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attn_phase1_kernel(const AttnAr
   pdl_wait();  // Q, K, V (and, in the second pass, the first pass's statistics) may come from earlier kernels
   uint4 xk[KStage<D, NKP>::N];
   load_k<D, NKP>(a, b, h, xk);
-  if (rows_valid > 0) stage_q<D, NKP>(a.Q + (((int64_t)b * a.nq + row0) * a.H + h) * D, q_stride, rows_valid, slab);
+  if (rows_valid > 0) stage_q<D, NKP, MT>(a.Q + (((int64_t)b * a.nq + row0) * a.H + h) * D, q_stride, rows_valid, slab);
   store_k<D, NKP>(xk, sK);
   __syncthreads();
   float best = -INFINITY;
   if (rows_valid > 0) {
     float S[Cfg::MT][Cfg::NT][4];
-    logits_warp<D, NKP>(a, slab, sK, S);
+    logits_warp<D, NKP, MT>(a, slab, sK, S);
 #pragma unroll
     for (int mt = 0; mt < Cfg::MT; ++mt)
 #pragma unroll
@@ -278,9 +279,9 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attn_phase1_kernel(const AttnAr
   }
 }
 
-template <int D, int NKP, bool CODES>
+template <int D, int NKP, int MT, bool CODES>
 __global__ void __launch_bounds__(AT_THREADS, 2) attn_phase2_kernel(const AttnArgs a) {
-  using Cfg = AttnCfg<D, NKP>;
+  using Cfg = AttnCfg<D, NKP, MT>;
   constexpr int NT_O = D / 8;
   extern __shared__ __align__(16) unsigned char at_smem[];
   __half* sK = reinterpret_cast<__half*>(at_smem);
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attn_phase2_kernel(const AttnAr
     for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) part_w[warp] = m;
   }
-  if (rows_valid > 0) stage_q<D, NKP>(a.Q + (((int64_t)b * a.nq + row0) * a.H + h) * D, q_stride, rows_valid, slab);
+  if (rows_valid > 0) stage_q<D, NKP, MT>(a.Q + (((int64_t)b * a.nq + row0) * a.H + h) * D, q_stride, rows_valid, slab);
   store_k<D, NKP>(xk, sK);
   // Quantized value operand: range of the head's slab (every CTA of the head derives the same
   // parameters), codes decided in fp32, de-quantized as s (q - Z); rows j >= 1 become the fp16
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attn_phase2_kernel(const AttnAr
     a.scale_out[scope] = exp2f(log2s);
   if (rows_valid <= 0) return;
   float S[Cfg::MT][Cfg::NT][4];
-  logits_warp<D, NKP>(a, slab, sK, S);
+  logits_warp<D, NKP, MT>(a, slab, sK, S);
   __syncwarp();  // the slab is reused for the output rows below
 
   const float Lf = (float)((1 << a.bits) - 1);
@@ -513,9 +514,9 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attn_phase2_kernel(const AttnAr
 // their maxima through the workspace and meet at the grid barrier, so Q K^T, the K / Q staging and the
 // statistics round trip happen once.  Launched cooperatively (every CTA resident) when the scale is dynamic;
 // with a fixed scale no CTA waits for another and the launch is an ordinary one.
-template <int D, int NKP, bool CODES>
+template <int D, int NKP, int MT, bool CODES>
 __global__ void __launch_bounds__(AT_THREADS, 2) attn_fused_kernel(const AttnArgs a) {
-  using Cfg = AttnCfg<D, NKP>;
+  using Cfg = AttnCfg<D, NKP, MT>;
   constexpr int NT_O = D / 8;
   extern __shared__ __align__(16) unsigned char at_smem[];
   __half* sK = reinterpret_cast<__half*>(at_smem);
@@ -561,7 +562,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attn_fused_kernel(const AttnArg
   // The scope's scale: its CTAs' partial maxima lie next to each other (row blocks of a head, heads of a
   // prompt, prompts of the call); each thread takes a strided share, the warps meet after the barrier below.
   __shared__ float part_w[AT_WARPS];
-  if (rows_valid > 0) stage_q<D, NKP>(a.Q + (((int64_t)b * a.nq + row0) * a.H + h) * D, q_stride, rows_valid, slab);
+  if (rows_valid > 0) stage_q<D, NKP, MT>(a.Q + (((int64_t)b * a.nq + row0) * a.H + h) * D, q_stride, rows_valid, slab);
   store_k<D, NKP>(xk, sK);
   __syncthreads();
   const int scope = scope_index(a, b, h);
@@ -569,7 +570,7 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attn_fused_kernel(const AttnArg
   float S[Cfg::MT][Cfg::NT][4];
   float st_max[Cfg::MT][2], st_lz[Cfg::MT][2];  // row maximum and log2 of the row sum, rows r and r + 8 of every tile
   float best = -INFINITY;
-  if (rows_valid > 0) logits_warp<D, NKP>(a, slab, sK, S);
+  if (rows_valid > 0) logits_warp<D, NKP, MT>(a, slab, sK, S);
   if (!V_EARLY) request_v();
   if (rows_valid > 0) {
 #pragma unroll
@@ -823,56 +824,84 @@ static cudaError_t launch_cooperative(void (*kernel)(KArgs...), dim3 grid, dim3 
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-template <int D, int NKP>
-static dgq_status launch_attn(const AttnArgs& a, bool allow_fused, cudaStream_t stream) {
-  using Cfg = AttnCfg<D, NKP>;
-  constexpr int SM1 = Cfg::SMEM1;
-  constexpr int SM2 = Cfg::SMEM2;
-  static std::atomic<int> capacity[64];  // CTAs of the fused kernel that fit the device at once; 0 = not asked yet
+// CTAs of the fused kernel that fit the device at once (asked once per device).
+template <int D, int NKP, int MT>
+static cudaError_t attn_fused_capacity(int* n) {
+  constexpr int SM2 = AttnCfg<D, NKP, MT>::SMEM2;
+  static std::atomic<int> known[64];
+  int dev = 0, n_sm = 0, per_sm0 = 0, per_sm1 = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if ((*n = known[dev].load()) != 0) return cudaSuccess;
+  if ((e = cudaFuncSetAttribute(attn_fused_kernel<D, NKP, MT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM2)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(attn_fused_kernel<D, NKP, MT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM2)) != cudaSuccess ||
+      (e = sm_count(&n_sm)) != cudaSuccess ||
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm0, attn_fused_kernel<D, NKP, MT, false>, AT_THREADS, SM2)) != cudaSuccess ||
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, attn_fused_kernel<D, NKP, MT, true>, AT_THREADS, SM2)) != cudaSuccess)
+    return e;
+  *n = std::max(1, n_sm * std::min(per_sm0, per_sm1));
+  known[dev].store(*n);
+  return cudaSuccess;
+}
+
+template <int D, int NKP, int MT>
+static dgq_status launch_attn_fused(AttnArgs a, cudaStream_t stream) {
+  using Cfg = AttnCfg<D, NKP, MT>;
+  a.n_row_blocks = (a.nq + Cfg::ROWS - 1) / Cfg::ROWS;
+  const dim3 grid(a.B * a.H * a.n_row_blocks);
+  auto kernel = a.codes_out ? attn_fused_kernel<D, NKP, MT, true> : attn_fused_kernel<D, NKP, MT, false>;
+  // with a fixed scale no CTA waits for another; with a dynamic one they meet at the grid barrier, and the launch
+  // guarantees that all of them are resident
+  if (a.fixed_scale) DGQ_CUDA_OK(launch_pdl(kernel, grid, dim3(AT_THREADS), (size_t)Cfg::SMEM2, stream, a));
+  else DGQ_CUDA_OK(launch_cooperative(kernel, grid, dim3(AT_THREADS), (size_t)Cfg::SMEM2, stream, a));
+  g_launches += 1;
+  DGQ_CUDA_OK(cudaGetLastError());
+  return DGQ_OK;
+}
+
+// The two passes as kernels of their own, for grids beyond one resident wave.
+template <int D, int NKP, int MT>
+static dgq_status launch_attn_two(AttnArgs a, cudaStream_t stream) {
+  using Cfg = AttnCfg<D, NKP, MT>;
+  static std::atomic<bool> attr_set[64];
   int dev = 0;
   DGQ_CUDA_OK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return DGQ_ERR_UNSUPPORTED;
-  if (capacity[dev].load() == 0) {
-    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_phase1_kernel<D, NKP>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM1));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_phase2_kernel<D, NKP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM2));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_phase2_kernel<D, NKP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM2));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_fused_kernel<D, NKP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM2));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_fused_kernel<D, NKP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM2));
-    int n_sm = 0, per_sm0 = 0, per_sm1 = 0;
-    DGQ_CUDA_OK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-    DGQ_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm0, attn_fused_kernel<D, NKP, false>, AT_THREADS, SM2));
-    DGQ_CUDA_OK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, attn_fused_kernel<D, NKP, true>, AT_THREADS, SM2));
-    capacity[dev].store(std::max(1, n_sm * std::min(per_sm0, per_sm1)));
+  if (!attr_set[dev].load()) {
+    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_phase1_kernel<D, NKP, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM1));
+    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_phase2_kernel<D, NKP, MT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM2));
+    DGQ_CUDA_OK(cudaFuncSetAttribute(attn_phase2_kernel<D, NKP, MT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM2));
+    attr_set[dev].store(true);
   }
-  AttnArgs aa = a;
-  aa.n_row_blocks = (a.nq + Cfg::ROWS - 1) / Cfg::ROWS;
-  const int grid = a.B * a.H * aa.n_row_blocks;
-  if (allow_fused && (a.fixed_scale != nullptr || grid <= capacity[dev].load())) {
-    // one kernel: with a fixed scale its CTAs never wait for one another; with a dynamic one they meet at the
-    // grid barrier, and the launch guarantees that all of them are resident
-    if (a.fixed_scale) {
-      if (a.codes_out)
-        DGQ_CUDA_OK(launch_pdl(attn_fused_kernel<D, NKP, true>, dim3(grid), dim3(AT_THREADS), (size_t)SM2, stream, aa));
-      else
-        DGQ_CUDA_OK(launch_pdl(attn_fused_kernel<D, NKP, false>, dim3(grid), dim3(AT_THREADS), (size_t)SM2, stream, aa));
-    } else {
-      if (a.codes_out)
-        DGQ_CUDA_OK(launch_cooperative(attn_fused_kernel<D, NKP, true>, dim3(grid), dim3(AT_THREADS), (size_t)SM2, stream, aa));
-      else
-        DGQ_CUDA_OK(launch_cooperative(attn_fused_kernel<D, NKP, false>, dim3(grid), dim3(AT_THREADS), (size_t)SM2, stream, aa));
-    }
-    g_launches += 1;
-    DGQ_CUDA_OK(cudaGetLastError());
-    return DGQ_OK;
-  }
-  DGQ_CUDA_OK(launch_pdl(attn_phase1_kernel<D, NKP>, dim3(grid), dim3(AT_THREADS), (size_t)SM1, stream, aa));
-  if (a.codes_out)
-    DGQ_CUDA_OK(launch_pdl(attn_phase2_kernel<D, NKP, true>, dim3(grid), dim3(AT_THREADS), (size_t)SM2, stream, aa));
-  else
-    DGQ_CUDA_OK(launch_pdl(attn_phase2_kernel<D, NKP, false>, dim3(grid), dim3(AT_THREADS), (size_t)SM2, stream, aa));
+  a.n_row_blocks = (a.nq + Cfg::ROWS - 1) / Cfg::ROWS;
+  const dim3 grid(a.B * a.H * a.n_row_blocks);
+  DGQ_CUDA_OK(launch_pdl(attn_phase1_kernel<D, NKP, MT>, grid, dim3(AT_THREADS), (size_t)Cfg::SMEM1, stream, a));
+  DGQ_CUDA_OK(launch_pdl(a.codes_out ? attn_phase2_kernel<D, NKP, MT, true> : attn_phase2_kernel<D, NKP, MT, false>, grid,
+                         dim3(AT_THREADS), (size_t)Cfg::SMEM2, stream, a));
   g_launches += 2;
   DGQ_CUDA_OK(cudaGetLastError());
   return DGQ_OK;
+}
+
+// One kernel where its grid fits the device at once: with 128 query rows per CTA (more CTAs, shorter ones) or, if that is
+// too many, 256 where the registers allow it (8 x 8 x 1024 x 80: 512 CTAs of 128 rows would need two kernels).
+template <int D, int NKP>
+static dgq_status launch_attn(const AttnArgs& a, bool allow_fused, cudaStream_t stream) {
+  constexpr bool TWO = D <= 80 && NKP <= 5;
+  if (allow_fused) {
+    const int64_t heads = (int64_t)a.B * a.H;
+    int fit1 = 0, fit2 = 0;
+    DGQ_CUDA_OK((attn_fused_capacity<D, NKP, 1>(&fit1)));
+    if (heads * ((a.nq + 127) / 128) <= fit1) return launch_attn_fused<D, NKP, 1>(a, stream);
+    if constexpr (TWO) {
+      DGQ_CUDA_OK((attn_fused_capacity<D, NKP, 2>(&fit2)));
+      if (a.fixed_scale || heads * ((a.nq + 255) / 256) <= fit2) return launch_attn_fused<D, NKP, 2>(a, stream);
+    } else if (a.fixed_scale) {
+      return launch_attn_fused<D, NKP, 1>(a, stream);
+    }
+  }
+  return launch_attn_two<D, NKP, (D <= 64 && NKP <= 5) ? 2 : 1>(a, stream);
 }
 
 template <int D>

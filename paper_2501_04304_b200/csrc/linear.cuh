@@ -253,7 +253,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           cw = rem - chh * a.conv_W;
         }
         for (; ks < n_kstages; ks += producers) {
-          mbar_wait_lean(empty0 + s * 8u, empty_par, abort_flag);
+          mbar_wait_handover(empty0 + s * 8u, empty_par, abort_flag);
           uint4 tab = make_uint4(0, 0, 0, 0);
           if (CONV) tab = *reinterpret_cast<const uint4*>(conv_tab + ks * 4);
           if (elect_one()) {
@@ -317,7 +317,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int j = 0; j < 4; ++j) {
           const bool starts = (j == 0) ? need : (((PAT >> (j > 0 ? j - 1 : 0)) & 1) != 0);
           if (starts) {
-            mbar_wait_lean(acce0 + ab * 8u, acc_phase, abort_flag);
+            mbar_wait_handover(acce0 + ab * 8u, acc_phase, abort_flag);
             tc_fence_after();
           }
           if (elect_one()) {
@@ -335,7 +335,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       };
       auto wait_full = [&]() {
-        if (!full_ready) mbar_wait_lean(full0 + s * 8u, full_phase, abort_flag);
+        if (!full_ready) mbar_wait_handover(full0 + s * 8u, full_phase, abort_flag);
         full_ready = 0;
         tc_fence_after();
       };
@@ -377,7 +377,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             // end of the last group moves to the last atom issued.
             const int atoms_here = n_atoms - ks * 4;
             if (atoms_here < 4) pat = (pat & ~(1u << (atoms_here - 1))) | 8u;
-            mbar_wait_lean(full0 + s * 8u, full_phase, abort_flag);
+            mbar_wait_handover(full0 + s * 8u, full_phase, abort_flag);
             tc_fence_after();
             const uint32_t a_lo = a_lo0 + s * (uint32_t)(GEMM_A_STAGE >> 4);
             const uint32_t b_lo = b_lo0 + s * (uint32_t)(Cfg::B_STAGE >> 4);
@@ -404,7 +404,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
           for (int g = 0; g < a.G; ++g) {
             const int end = a.seg_end[g];
-            mbar_wait_lean(acce0 + ab * 8u, acc_phase, abort_flag);
+            mbar_wait_handover(acce0 + ab * 8u, acc_phase, abort_flag);
             tc_fence_after();
             uint32_t acc = 0u;  // the group's first MMA starts the accumulator
             // what is left of a stage that the group before has begun
@@ -456,7 +456,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tile_it) {
         const int tm = tile / a.n_tiles_n, tn = tile - tm * a.n_tiles_n;
         const int n0 = tn * BN;
-        mbar_wait_lean(out_full_a, tile_it & 1u, abort_flag);
+        mbar_wait_handover(out_full_a, tile_it & 1u, abort_flag);
         if (*abort_flag) break;
 #pragma unroll
         for (int pnl = 0; pnl < BN / 32; ++pnl)
@@ -621,7 +621,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           npar ^= 1u;
         }
         const unsigned long long s2 = pack_f32x2(s, s);
-        mbar_wait_lean(full0 + ab * 8u, acc_par, abort_flag);
+        mbar_wait_handover(full0 + ab * 8u, acc_par, abort_flag);
         tc_fence_after();
         load_group(t_lane + ab * (uint32_t)BN);
         tmem_ld_wait();
@@ -663,7 +663,7 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (*abort_flag) break;  // a wait gave up somewhere in the CTA (same value in every lane)
       // staging buffer: wait until the stores of the previous tile have read it (normally long done)
-      mbar_wait_lean(out_free_a, (tile_it & 1u) ^ 1u, abort_flag);
+      mbar_wait_handover(out_free_a, (tile_it & 1u) ^ 1u, abort_flag);
 #pragma unroll
       for (int j = 0; j < CW / 8; ++j) {
         const int cl = sl * CW + j * 8;  // first tile column of this 16-byte chunk

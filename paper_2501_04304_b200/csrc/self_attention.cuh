@@ -222,7 +222,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       uint32_t kit = 0, vit = 0;
       auto load_v = [&](int j) {
         const uint32_t vs = vit % VST;
-        mbar_wait_lean(smem_u32(&sh->v_empty[vs]), ((vit / VST) & 1u) ^ 1u, abort_flag);
+        mbar_wait_handover(smem_u32(&sh->v_empty[vs]), ((vit / VST) & 1u) ^ 1u, abort_flag);
         mbar_arrive_expect_tx(&sh->v_full[vs], (uint32_t)Cfg::TILE);
         for (int p = 0; p < NP; ++p)
           tma_load_4d(sV + vs * Cfg::TILE + p * SATC_PANEL, &tmV, &sh->v_full[vs], p * 64, h, j * SATC_BK, b);
@@ -232,7 +232,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         const bool last = (w == N_WALKS - 1);
         for (int j = 0; j < nb; ++j) {
           const uint32_t ks = kit % KST;
-          mbar_wait_lean(smem_u32(&sh->k_empty[ks]), ((kit / KST) & 1u) ^ 1u, abort_flag);
+          mbar_wait_handover(smem_u32(&sh->k_empty[ks]), ((kit / KST) & 1u) ^ 1u, abort_flag);
           mbar_arrive_expect_tx(&sh->k_full[ks], (uint32_t)Cfg::TILE);
           for (int p = 0; p < NP; ++p)
             tma_load_4d(sK + ks * Cfg::TILE + p * SATC_PANEL, &tmK, &sh->k_full[ks], p * 64, h, j * SATC_BK, b);
@@ -262,12 +262,12 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       const uint32_t s_full0 = smem_u32(&sh->s_full[0]), s_free0 = smem_u32(&sh->s_free[0]);
       const int total = N_WALKS * per_walk;
       uint32_t ks = 0, k_par = 0;
-      mbar_wait_lean(smem_u32(&sh->q_full), 0, abort_flag);
+      mbar_wait_handover(smem_u32(&sh->q_full), 0, abort_flag);
       for (int g = 0; g < total; ++g) {
         const uint32_t sb = (uint32_t)g & 1u;
         const uint32_t t = NT == 2 ? sb : 0u;
-        if (t == 0) mbar_wait_lean(k_full0 + ks * 8u, k_par, abort_flag);
-        mbar_wait_lean(s_free0 + sb * 8u, (((uint32_t)g >> 1) & 1u) ^ 1u, abort_flag);
+        if (t == 0) mbar_wait_handover(k_full0 + ks * 8u, k_par, abort_flag);
+        mbar_wait_handover(s_free0 + sb * 8u, (((uint32_t)g >> 1) & 1u) ^ 1u, abort_flag);
         tc_fence_after();
         const uint32_t a_lo = q_lo + t * (uint32_t)(Cfg::TILE >> 4), b_lo = k_lo + ks * (uint32_t)(Cfg::TILE >> 4);
         const bool k_done = t == NT - 1;
@@ -302,8 +302,8 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       uint32_t pb = PST == 2 ? (uint32_t)((N_WALKS - 1) * per_walk) & 1u : 0u, p_par = 0, vs = 0, v_par = 0;
       for (int c = 0; c < per_walk; ++c) {
         const uint32_t t = NT == 2 ? ((uint32_t)c & 1u) : 0u;
-        mbar_wait_lean(p_full0 + pb * 8u, (p_par >> pb) & 1u, abort_flag);
-        if (t == 0) mbar_wait_lean(v_full0 + vs * 8u, v_par, abort_flag);
+        mbar_wait_handover(p_full0 + pb * 8u, (p_par >> pb) & 1u, abort_flag);
+        if (t == 0) mbar_wait_handover(v_full0 + vs * 8u, v_par, abort_flag);
         tc_fence_after();
         const uint32_t a_tmem = tmem_base + SATC_TMEM_P + pb * 64u, b_lo = v_lo + vs * (uint32_t)(Cfg::TILE >> 4);
         const uint32_t d_tmem = tmem_base + Cfg::TMEM_O + t * Cfg::DP;
@@ -372,7 +372,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         const uint32_t sb = (uint32_t)g & 1u;
         // After a time-out every wait returns at once and the loops run to their ends on whatever the buffers hold (an
         // error is recorded): no warp leaves early, so the named barriers are always reached by all their warps.
-        mbar_wait_lean(smem_u32(&sh->s_full[sb]), (TEAMS == 2 ? n : n >> 1) & 1u, abort_flag);
+        mbar_wait_handover(smem_u32(&sh->s_full[sb]), (TEAMS == 2 ? n : n >> 1) & 1u, abort_flag);
         __syncwarp();
         tc_fence_after();
 #pragma unroll
@@ -467,7 +467,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
               }
             }
             if (ch == 0) {  // the buffer's previous product must have read it
-              mbar_wait_lean(smem_u32(&sh->p_free[pb]), (c & 1u) ^ 1u, abort_flag);
+              mbar_wait_handover(smem_u32(&sh->p_free[pb]), (c & 1u) ^ 1u, abort_flag);
               __syncwarp();
               tc_fence_after();
             }
@@ -502,7 +502,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     float s_row;
     if (FIXED) s_row = fmaxf(__ldg(a.fixed_scale + b), 1.17549435e-38f) * 6.103515625e-05f;  // 2^-14
     else s_row = 1.0f / row_sum();  // (the sum carries the 2^14)
-    mbar_wait_lean(smem_u32(&sh->o_full), 0, abort_flag);
+    mbar_wait_handover(smem_u32(&sh->o_full), 0, abort_flag);
     __syncwarp();
     tc_fence_after();
     {

@@ -89,7 +89,7 @@ __device__ __forceinline__ uint32_t codes4(const float (&y)[4], float lowb, uint
   return __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
 }
 
-template <bool DYNAMIC, bool CENTRED>
+template <bool DYNAMIC, bool CENTRED, bool WARP>
 __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ QuantArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n_chunks = a.K_pad >> 4, n_cells = a.pairs * 2 * a.G;
@@ -97,11 +97,16 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
   int* cell_lo = reinterpret_cast<int*>(smem_raw + buf_bytes);  // [2][n_cells]
   int* cell_hi = cell_lo + 2 * n_cells;
   const int tid = threadIdx.x, n_threads = blockDim.x;
+  // Threads that share a row pair: all of the block, or (WARP) the warp that has the pair to itself.
+  auto sync = [&]() {
+    if (WARP) __syncwarp();
+    else __syncthreads();
+  };
 
   pdl_launch_dependents();
   // this thread's chunk: where its 16 values lie in an interleaved pair, its group, its padding positions
-  const int my_pair = tid / n_chunks, ch = tid - my_pair * n_chunks;
-  const bool active = my_pair < a.pairs;
+  const int my_pair = WARP ? tid >> 5 : tid / n_chunks, ch = WARP ? tid & 31 : tid - my_pair * n_chunks;
+  const bool active = my_pair < a.pairs && ch < n_chunks;
   uint32_t off[16];  // shared-memory addresses
   uint32_t pm = 0;
   int g = 0;
@@ -139,9 +144,9 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
     const int task = tid + e * n_threads;
-    lp[e] = task / vec;
-    lv[e] = task - lp[e] * vec;
-    lok[e] = lp[e] < a.pairs;
+    lp[e] = WARP ? my_pair : task / vec;
+    lv[e] = WARP ? (tid & 31) + 32 * e : task - lp[e] * vec;
+    lok[e] = lp[e] < a.pairs && lv[e] < vec;
   }
   float inv0 = 0.f, inv1 = 0.f;
   int z0 = 0, z1 = 0;
@@ -149,6 +154,7 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
     inv0 = inv1 = __ldg(a.inv_scale + g);
     z0 = z1 = __ldg(a.zp + g);
   }
+  if (WARP) __syncthreads();  // the words of NaN and the cells are set
   pdl_wait();  // everything above reads only constants of the grouping; the rows may come from the previous kernel
 
   const int64_t rows_per_batch = 2 * (int64_t)a.pairs, step = rows_per_batch * gridDim.x;
@@ -169,7 +175,7 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
   int buf = 0;
   for (int64_t row0 = first_row; row0 < a.M; row0 += step, buf ^= 1) {
     // (dynamic: the barrier behind the ranges says so)
-    if (!DYNAMIC && row0 != first_row) __syncthreads();  // every value of the last batch is in registers
+    if (!DYNAMIC && row0 != first_row) sync();  // every value of the last batch is in registers
 #pragma unroll
     for (int e = 0; e < 2; ++e)
       if (lok[e]) {
@@ -180,7 +186,7 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
                             __byte_perm(xa[e].w, xb[e].w, 0x5410), __byte_perm(xa[e].w, xb[e].w, 0x7632));
       }
     if (row0 + step < a.M) request(row0 + step);  // arrives while this batch is worked on
-    __syncthreads();
+    sync();
     __half2 x[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -214,7 +220,7 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
         atomicMax(c_hi + cell, k[2]);
         atomicMax(c_hi + cell + a.G, k[3]);
       }
-      __syncthreads();
+      sync();
       if (active) {
         // Every thread derives the parameters of its two cells itself: two more IEEE divisions per thread cost less
         // than a third barrier behind the few threads that would do it for all.
@@ -348,10 +354,15 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   // threads to an SM.  A matrix that would leave blocks without work gets smaller batches, down to one pair.
   const int n_chunks = g->K_pad / 16;
   const int64_t n_pairs = (M + 1) / 2;
-  int pairs = std::max(1, 128 / n_chunks);
-  int64_t slots = (int64_t)n_sm * std::max(1, 896 / (pairs * n_chunks));
+  // Where the chunks of a pair nearly fill a warp, each warp has a pair to itself and the barriers of a batch are the
+  // warp's own (32768 x 320 with 512 positions: 16.4 -> 15.4 us, static 11.5 -> 11.0; with 20 of 32 lanes at work,
+  // 16384 x 200, 7.3 -> 7.9 us, so not there).
+  const bool warp = n_chunks > 24 && n_chunks <= 32;
+  const int per_pair = warp ? 32 : n_chunks;
+  int pairs = std::max(1, 128 / per_pair);
+  int64_t slots = (int64_t)n_sm * std::max(1, 896 / (pairs * per_pair));
   if (n_pairs < slots * pairs) pairs = (int)std::max<int64_t>(1, (n_pairs + slots - 1) / slots);
-  const int threads = (pairs * n_chunks + 31) / 32 * 32;
+  const int threads = (pairs * per_pair + 31) / 32 * 32;
   slots = (int64_t)n_sm * std::max(1, 896 / threads);
   a.pairs = pairs;
   const size_t smem = qa_smem_bytes(pairs, g->C, g->G, dynamic);
@@ -359,15 +370,18 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   int dev = 0;
   DGQ_CUDA_OK(cudaGetDevice(&dev));
   if (dev >= 64 || !attr_set[dev].load()) {
-    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
     if (dev < 64) attr_set[dev].store(true);
   }
   const int grid = (int)std::min<int64_t>((n_pairs + pairs - 1) / pairs, slots);
-  DGQ_CUDA_OK(launch_pdl(dynamic ? quantize_act_kernel<true, false>
-                                : layout == DGQ_CODES_S8_CENTRED ? quantize_act_kernel<false, true> : quantize_act_kernel<false, false>,
-                         dim3(grid), dim3(threads), smem,
+  const bool centred = layout == DGQ_CODES_S8_CENTRED;
+  auto kernel = warp ? (dynamic ? quantize_act_kernel<true, false, true>
+                                : centred ? quantize_act_kernel<false, true, true> : quantize_act_kernel<false, false, true>)
+                     : (dynamic ? quantize_act_kernel<true, false, false>
+                                : centred ? quantize_act_kernel<false, true, false> : quantize_act_kernel<false, false, false>);
+  DGQ_CUDA_OK(launch_pdl(kernel, dim3(grid), dim3(threads), smem,
                          (cudaStream_t)stream, a));
   g_launches += 1;
   DGQ_CUDA_OK(cudaGetLastError());

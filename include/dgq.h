@@ -160,8 +160,9 @@ dgq_status dgq_weight_export(const dgq_weight* w, int8_t* wq, float* sw);
  * Contents undefined on entry and exit; calls that may overlap on the GPU need
  * separate workspaces unless they use the same weight.  NULL / 0 for 8-bit
  * weights.  NULL with 4-bit weights is allowed: the GEMM then expands the
- * weights itself, stage by stage and once per row tile (slower); a non-NULL
- * workspace that is too small is an error.
+ * weights itself, stage by stage and once per row tile, as it also does with a
+ * workspace where that is faster (small problems); a non-NULL workspace that is
+ * too small is an error.
  * Errors: INVALID_ARG, ALIGNMENT, NOT_CALIBRATED, WORKSPACE, UNSUPPORTED (K_pad *
  * 255 * 127 would overflow int32; more column blocks of 64-128 outputs than the
  * GPU has SMs; conv shape outside the supported tiling), CUDA. */

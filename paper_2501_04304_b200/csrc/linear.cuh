@@ -32,8 +32,6 @@
 // the tap, out-of-image rows zero-filled by TMA (exact for zero-centred codes).
 #pragma once
 
-#include <type_traits>
-
 #include "weights.cuh"
 
 namespace dgq {
@@ -61,7 +59,7 @@ static_assert(8 * gemm_regs_epi(false) + 4 * gemm_regs_other(false) <= 12 * gemm
 constexpr int GEMM_MAX_ATOMS = 1024;           // 32768 reduction positions
 constexpr int GEMM_A_STAGE = GEMM_BM * 128;  // bytes
 constexpr int GEMM_SMEM_LIMIT = 227 * 1024;
-constexpr int GEMM_LONG_STAGES = 8;          // from this many stages on a reduction is fed by two producers and issued by groups
+constexpr int GEMM_LONG_STAGES = 8;          // from this many stages on a reduction is fed by two producers
 
 template <int BN, bool W4>
 struct GemmCfg {
@@ -107,7 +105,6 @@ struct GemmArgs {
   const __half* bias;         // [N] or null
   const uint8_t* w_packed;    // 4-bit weights [N_pad][Kt/2]
   int seg_end[DGQ_MAX_GROUPS];    // end atom of every group segment
-  unsigned long long end_mask;    // reductions of fewer than GEMM_LONG_STAGES stages: bit i: atom i is the last of its group
   // conv
   int conv_W, conv_H;
   int grp_atoms[DGQ_MAX_GROUPS];  // channel atoms of every group
@@ -293,11 +290,12 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // ------------------------------------------------------------ MMA issuer
     // The whole warp runs the loop with uniform control flow; the tcgen05 instructions are issued by one elected lane.
     // A branch costs this warp 30-40 cycles, a barrier poll 50-100, and the tensor core queues only a couple of MMAs,
-    // so what the loop does between MMAs shows.  A short reduction, whose stages are full of group ends, runs
-    // straight-line stage bodies chosen by the pattern of ends.  A long one walks groups: through the stages in the
-    // middle of a group without a test of where groups end, and with the next stage's barrier polled ahead of the
-    // MMAs so that the poll's latency runs under them (350 cycles a stage against 520, of which the MMAs take 320;
-    // 2048 x 5120 -> 1280 W8 20.7 -> 19.3 us, conv 8 x 64 x 64 x 320 93 -> 78 us together with the second producer).
+    // so what the loop does between MMAs shows.  It walks groups, not stages: through the stages in the middle of a
+    // group without a test of where groups end, and with the next stage's barrier polled ahead of the MMAs so that the
+    // poll's latency runs under them (350 cycles a stage against 520 with a test per atom, of which the MMAs take 320;
+    // 2048 x 5120 -> 1280 W8 20.7 -> 18.9 us, conv 8 x 64 x 64 x 320 93 -> 77 us together with the second producer).
+    // A group's first and last stages issue a counted run of MMAs.  Reductions of a few stages full of group ends are
+    // as fast this way as with a straight-line body for each of the 16 patterns of ends in a stage.
     {
       constexpr uint32_t A_HI = CONV ? smem_desc_hi(256, 6) : smem_desc_hi(1024, 2);
       constexpr uint32_t B_HI = smem_desc_hi(1024, 2);
@@ -310,30 +308,6 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       uint32_t ab = 0;           // accumulator of the next group
       uint32_t acc_phase = 1;    // parity to wait for on its "empty" barrier (fresh barriers pass)
       uint32_t full_ready = 0;   // the slot's "full" phase has been seen to be complete
-      // One stage of four atoms whose group ends are the bits of PAT; `need`: the first atom starts a group.
-      auto issue_stage = [&](auto pat_tag, bool need, uint32_t a_lo, uint32_t b_lo) {
-        constexpr int PAT = decltype(pat_tag)::value;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const bool starts = (j == 0) ? need : (((PAT >> (j > 0 ? j - 1 : 0)) & 1) != 0);
-          if (starts) {
-            mbar_wait_handover(acce0 + ab * 8u, acc_phase, abort_flag);
-            tc_fence_after();
-          }
-          if (elect_one()) {
-            mma_i8_lohi(tmem_base + ab * (uint32_t)BN, a_lo + (CONV ? j * 256 : j * 2), A_HI, b_lo + j * 2, B_HI, idesc,
-                        starts ? 0u : 1u);
-            if ((PAT >> j) & 1) mma_commit_addr(accf0 + ab * 8u);  // last atom of the group: hand the accumulator over
-          }
-          __syncwarp();
-          if ((PAT >> j) & 1) {
-            if (++ab == (uint32_t)NACC) {
-              ab = 0;
-              acc_phase ^= 1u;
-            }
-          }
-        }
-      };
       auto wait_full = [&]() {
         if (!full_ready) mbar_wait_handover(full0 + s * 8u, full_phase, abort_flag);
         full_ready = 0;
@@ -345,105 +319,75 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           full_phase ^= 1u;
         }
       };
-      // N atoms of the current stage from atom j0 on; then the accumulator and / or the stage are handed over
-      auto issue = [&](auto n_tag, uint32_t j0, uint32_t acc, bool group_done, bool stage_done) {
-        constexpr int N_ATOMS = decltype(n_tag)::value;
+      // n atoms of the current stage from atom j0 on; then the accumulator and / or the stage are handed over
+      auto issue_n = [&](int n, uint32_t j0, uint32_t acc, bool group_done, bool stage_done) {
         const uint32_t a_lo = a_lo0 + s * (uint32_t)(GEMM_A_STAGE >> 4) + j0 * (CONV ? 256u : 2u);
         const uint32_t b_lo = b_lo0 + s * (uint32_t)(Cfg::B_STAGE >> 4) + j0 * 2u;
+        const uint32_t d = tmem_base + ab * (uint32_t)BN;
+        constexpr uint32_t A_STEP = CONV ? 256u : 2u;
         if (elect_one()) {
-#pragma unroll
-          for (int j = 0; j < N_ATOMS; ++j)
-            mma_i8_lohi(tmem_base + ab * (uint32_t)BN, a_lo + (CONV ? j * 256 : j * 2), A_HI, b_lo + j * 2, B_HI, idesc,
-                        j == 0 ? acc : 1u);
+          mma_i8_lohi(d, a_lo, A_HI, b_lo, B_HI, idesc, acc);
+          if (n > 1) mma_i8_lohi(d, a_lo + A_STEP, A_HI, b_lo + 2u, B_HI, idesc, 1u);
+          if (n > 2) mma_i8_lohi(d, a_lo + 2u * A_STEP, A_HI, b_lo + 4u, B_HI, idesc, 1u);
+          if (n > 3) mma_i8_lohi(d, a_lo + 3u * A_STEP, A_HI, b_lo + 6u, B_HI, idesc, 1u);
           if (group_done) mma_commit_addr(accf0 + ab * 8u);
           if (stage_done) mma_commit_addr(empty0 + s * 8u);  // stage reusable once these MMAs have read it
         }
         __syncwarp();
       };
-      auto issue_n = [&](int n, uint32_t j0, uint32_t acc, bool group_done, bool stage_done) {
-        switch (n) {
-          case 1: issue(std::integral_constant<int, 1>{}, j0, acc, group_done, stage_done); break;
-          case 2: issue(std::integral_constant<int, 2>{}, j0, acc, group_done, stage_done); break;
-          case 3: issue(std::integral_constant<int, 3>{}, j0, acc, group_done, stage_done); break;
-          default: issue(std::integral_constant<int, 4>{}, j0, acc, group_done, stage_done); break;
-        }
-      };
-      if (n_kstages < GEMM_LONG_STAGES) {
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-          bool need = true;      // every tile starts a group
-          for (int ks = 0; ks < n_kstages; ++ks) {
-            uint32_t pat = (uint32_t)(a.end_mask >> (ks * 4)) & 0xFu;
-            // A ragged last stage still issues four atoms (the missing ones multiply zero weights); the
-            // end of the last group moves to the last atom issued.
-            const int atoms_here = n_atoms - ks * 4;
-            if (atoms_here < 4) pat = (pat & ~(1u << (atoms_here - 1))) | 8u;
-            mbar_wait_handover(full0 + s * 8u, full_phase, abort_flag);
-            tc_fence_after();
-            const uint32_t a_lo = a_lo0 + s * (uint32_t)(GEMM_A_STAGE >> 4);
-            const uint32_t b_lo = b_lo0 + s * (uint32_t)(Cfg::B_STAGE >> 4);
-            switch (pat) {
-#define DGQ_STAGE_CASE(P) case P: issue_stage(std::integral_constant<int, P>{}, need, a_lo, b_lo); break;
-              DGQ_STAGE_CASE(0) DGQ_STAGE_CASE(1) DGQ_STAGE_CASE(2) DGQ_STAGE_CASE(3) DGQ_STAGE_CASE(4) DGQ_STAGE_CASE(5)
-              DGQ_STAGE_CASE(6) DGQ_STAGE_CASE(7) DGQ_STAGE_CASE(8) DGQ_STAGE_CASE(9) DGQ_STAGE_CASE(10) DGQ_STAGE_CASE(11)
-              DGQ_STAGE_CASE(12) DGQ_STAGE_CASE(13) DGQ_STAGE_CASE(14) DGQ_STAGE_CASE(15)
-#undef DGQ_STAGE_CASE
+      for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        int atom = 0, next_end = a.seg_end[0];
+#pragma unroll 1
+        for (int g = 0; g < a.G; ++g) {
+          const int end = next_end;
+          next_end = a.seg_end[min(g + 1, DGQ_MAX_GROUPS - 1)];
+          mbar_wait_handover(acce0 + ab * 8u, acc_phase, abort_flag);
+          tc_fence_after();
+          uint32_t acc = 0u;  // the group's first MMA starts the accumulator
+          // what is left of a stage that the group before has begun
+          const int j0 = atom & 3;
+          if (j0 != 0) {
+            const int n = min(4 - j0, end - atom);
+            atom += n;
+            const bool stage_done = (atom & 3) == 0 || atom == n_atoms;
+            issue_n(n, (uint32_t)j0, 0u, atom == end, stage_done);
+            acc = 1u;
+            if (stage_done) next_slot();
+          }
+          // stages in the middle of the group: most of a long reduction
+#pragma unroll 1
+          while (end - atom > 4) {
+            wait_full();
+            const uint32_t ns = s + 1 == (uint32_t)STAGES ? 0u : s + 1;
+            full_ready = mbar_test_addr(full0 + ns * 8u, ns == 0 ? full_phase ^ 1u : full_phase);
+            const uint32_t a_lo = a_lo0 + s * (uint32_t)(GEMM_A_STAGE >> 4), b_lo = b_lo0 + s * (uint32_t)(Cfg::B_STAGE >> 4);
+            if (elect_one()) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                mma_i8_lohi(tmem_base + ab * (uint32_t)BN, a_lo + (CONV ? j * 256 : j * 2), A_HI, b_lo + j * 2, B_HI, idesc,
+                            j == 0 ? acc : 1u);
+              mma_commit_addr(empty0 + s * 8u);
             }
-            need = (pat & 8u) != 0;
-            if (elect_one()) mma_commit_addr(empty0 + s * 8u);  // stage reusable once these MMAs have read it
             __syncwarp();
-            if (++s == (uint32_t)STAGES) {
-              s = 0;
-              full_phase ^= 1u;
-            }
+            acc = 1u;
+            atom += 4;
+            s = ns;
+            if (ns == 0) full_phase ^= 1u;
           }
-          if (*abort_flag) break;
-        }
-      } else {
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-          int atom = 0;
-#pragma unroll 1
-          for (int g = 0; g < a.G; ++g) {
-            const int end = a.seg_end[g];
-            mbar_wait_handover(acce0 + ab * 8u, acc_phase, abort_flag);
-            tc_fence_after();
-            uint32_t acc = 0u;  // the group's first MMA starts the accumulator
-            // what is left of a stage that the group before has begun
-            const int j0 = atom & 3;
-            if (j0 != 0) {
-              const int n = min(4 - j0, end - atom);
-              atom += n;
-              const bool stage_done = (atom & 3) == 0 || atom == n_atoms;
-              issue_n(n, (uint32_t)j0, 0u, atom == end, stage_done);
-              acc = 1u;
-              if (stage_done) next_slot();
-            }
-            // stages in the middle of the group: most of a long reduction
-#pragma unroll 1
-            while (end - atom > 4) {
-              wait_full();
-              const uint32_t ns = s + 1 == (uint32_t)STAGES ? 0u : s + 1;
-              full_ready = mbar_test_addr(full0 + ns * 8u, ns == 0 ? full_phase ^ 1u : full_phase);
-              issue(std::integral_constant<int, 4>{}, 0u, acc, false, true);
-              acc = 1u;
-              atom += 4;
-              s = ns;
-              if (ns == 0) full_phase ^= 1u;
-            }
-            if (atom < end) {  // the group's last stage
-              wait_full();
-              const int n = end - atom;
-              atom = end;
-              const bool stage_done = n == 4 || atom == n_atoms;
-              issue_n(n, 0u, acc, true, stage_done);
-              if (stage_done) next_slot();
-            }
-            if (++ab == (uint32_t)NACC) {
-              ab = 0;
-              acc_phase ^= 1u;
-            }
+          if (atom < end) {  // the group's last stage
+            wait_full();
+            const int n = end - atom;
+            atom = end;
+            const bool stage_done = n == 4 || atom == n_atoms;
+            issue_n(n, 0u, acc, true, stage_done);
+            if (stage_done) next_slot();
           }
-          if (*abort_flag) break;
+          if (++ab == (uint32_t)NACC) {
+            ab = 0;
+            acc_phase ^= 1u;
+          }
         }
+        if (*abort_flag) break;
       }
     }
     __syncwarp();
@@ -796,7 +740,7 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   // 4-bit weights: with a workspace they are expanded once per call in front of the GEMM, without one
   // the GEMM expands them itself, stage by stage
   const size_t ws_need = w && w->w_bits == 4 ? (size_t)w->N_pad * (size_t)w->Kt : 0;
-  const bool expand_first = ws_need != 0 && workspace != nullptr;
+  bool expand_first = ws_need != 0 && workspace != nullptr;
   if (expand_first) {
     if (workspace_bytes < ws_need) return DGQ_ERR_WORKSPACE;
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return DGQ_ERR_ALIGNMENT;
@@ -832,7 +776,6 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   a.P = g->P;
   a.use_zp = (layout == DGQ_CODES_U8);
   a.code_max = (1 << g->bits) - 1;
-  a.b_early = !expand_first;
   a.res_mask = w->res_mask;
   a.wres = w->d_wres;
   a.row_group = g->d_row_group;
@@ -841,8 +784,6 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   a.bias = (const __half*)bias;
   a.w_packed = (const uint8_t*)w->d_w;
   if (w->Kt / DGQ_K_ATOM > GEMM_MAX_ATOMS) return DGQ_ERR_UNSUPPORTED;
-  if (w->Kt <= 128 * (GEMM_LONG_STAGES - 1))
-    for (int k = 0; k < g->G; ++k) a.end_mask |= 1ull << (w->seg_end[k] - 1);
   for (int k = 0; k < g->G; ++k) {
     a.seg_end[k] = w->seg_end[k];
     a.grp_atoms[k] = w->atoms[k];
@@ -858,11 +799,22 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   // (rounds over the groups, output) shrinks with its columns (256 x 320 -> 320: 7.2 -> 5.4 us, 616 x 768 -> 1280 W4:
   // 11.7 -> 10.1 us, 512 x 5120 -> 1280: 17.7 -> 15.4 us, conv 8 x 8 x 8 x 1280: 56 -> 46 us).
   if ((int64_t)a.n_tiles_m * ((w->N + BN - 1) / BN) * 2 <= n_sm) BN = 64;
+  a.n_tiles_n = (w->N + BN - 1) / BN;
+  // Expanding in front of the GEMM costs a launch and a round trip of the weights through L2 (1.0-1.5 us at least); in the
+  // kernel it costs every tile a share of its stages' time.  The kernel wins while a CTA unpacks little: 32-row pieces
+  // of a B stage over all its tiles (616 x 768 -> 1280 10.0 -> 8.8 us, 1024 x 768 -> 1280 14.5 -> 12.0, 2048 x 1280 ->
+  // 1280 at 60 pieces 15.0 -> 14.6, 2048 x 1600 -> 1280 at 70 pieces 15.6 -> 16.2).  A conv stage takes longer anyway
+  // (2 x 16 x 16 x 320 at 90 pieces 20.5 -> 19.2).
+  if (expand_first) {
+    const int64_t n_workers = (int64_t)std::min(a.n_tiles_m, std::max(1, n_sm / a.n_tiles_n));  // row blocks side by side
+    const int64_t pieces = (a.n_tiles_m + n_workers - 1) / n_workers * ((w->Kt + 127) / 128) * (BN / 32);
+    expand_first = pieces > (conv ? 100 : 64);
+  }
+  a.b_early = !expand_first;
   // instruction descriptor of kind::i8: int32 accumulator (bits 4-5 = 2), A format bit 7 (0 = u8,
   // 1 = s8), B format bit 10 = 1 (s8), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
   a.idesc = (2u << 4) | ((layout == DGQ_CODES_S8_CENTRED ? 1u : 0u) << 7) | (1u << 10) |
             ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(GEMM_BM >> 4) << 24);
-  a.n_tiles_n = (w->N + BN - 1) / BN;
 
   CUtensorMap tmA, tmB, tmY;
   std::memset(&tmA, 0, sizeof(tmA));

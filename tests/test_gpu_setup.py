@@ -68,6 +68,7 @@ def test_weight_layout_edges(sizes, N, w_bits):
     (1, (8,), 8),                    # one row, two chunks: a block of 64 pairs with one of them real
     (3, (1, 31, 33, 255), 6),        # odd row count, groups that end inside a chunk, 6-bit clamp
     (257, (320,), 8),                # a cell that covers a whole warp
+    (2601, (300, 188), 8),           # 32 chunks: a warp per row pair, several batches, odd row count
     (9, (5112, 8), 8),               # one pair per block, more chunks than a small block has threads
     (4100, (8184, 8), 4),            # the widest layer, several batches per block
 ])
@@ -126,3 +127,28 @@ def test_linear_reduction_lengths(M, N, sizes):
     ref = ol.group_linear(codes[rows], s_rows[rows], z_rows[rows], cg, wq, sw, bias)
     check_output(Y[torch.from_numpy(rows).cuda()], ref)
     assert torch.isfinite(Y).all() and b.device_status() == 0
+
+
+@pytest.mark.parametrize("M,C,N", [
+    (130, 320, 64),          # few pieces: unpacked inside the GEMM although there is a workspace
+    (128, 4000, 64),         # 64 pieces of 64-column tiles: the last reduction unpacked inside
+    (128, 4160, 64),         # the first expanded in front
+    (2500, 640, 1280),       # several tiles per block, expanded in front
+])
+def test_four_bit_routes(M, C, N):
+    torch, b = gpu()
+    rng = np.random.default_rng(M + C)
+    g = b.groups_from_host(C, 1, 8, np.zeros(C, np.int32), np.zeros(1, np.int32), np.full((1, 1, 1), 0.03, np.float32),
+                           np.full((1, 1, 1), 120, np.int32))
+    W = rng.normal(0, 0.02, (N, C)).astype(np.float16)
+    wq, sw = ol.weight_rtn(W, 4)
+    w = b.weight_prepare(g, to_dev(torch, W), 4)
+    X = rng.normal(0, 1, (M, C)).astype(np.float16)
+    Xq, ds, dz = b.quantize_act(g, to_dev(torch, X), mode=b.MODE_DYNAMIC_TOKEN)
+    kw = dict(mode=b.MODE_DYNAMIC_TOKEN, dyn_scale=ds, dyn_zp=dz)
+    Y = b.linear(g, w, Xq, **kw)
+    assert torch.equal(Y, b.linear(g, w, Xq, workspace=False, **kw))
+    rows = np.unique(np.r_[0:3, M // 2, M - 2:M])
+    codes, s_rows, z_rows = ol.quantize_dynamic_token(X[rows], np.zeros(C, np.int32), 1, 8)
+    check_output(Y[torch.from_numpy(rows).cuda()], ol.group_linear(codes, s_rows, z_rows, np.zeros(C, np.int32), wq, sw, None))
+    assert b.device_status() == 0

@@ -11,7 +11,7 @@
 // order-preserving keys (a warp whose lanes all belong to one cell reduces first), every thread
 // derives (s, 1/s, Z) of its two cells.
 //
-// Bound: about 300 warp instructions per row of 512 codes (half of them two-cycle integer and conversion
+// Bound: about 430 (dynamic) or 300 (static) warp instructions per row of 512 codes (half of them two-cycle integer and conversion
 // instructions) and the latency of one read-reduce-write chain for small matrices; the bytes (2 B read + 1 B written per
 // element + 8 B per (token, group) in dynamic mode) would take a third of the time.  72 registers keep 28
 // warps on an SM: at 80 an 8192-row matrix needs a second, nearly empty round of batches (5.5 against 5.1 us), at 64

@@ -797,8 +797,12 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   else if (w->N <= 64) BN = 64;
   // A problem that would leave more than half of the SMs without a tile takes narrow ones: the serial work of a CTA
   // (rounds over the groups, output) shrinks with its columns (256 x 320 -> 320: 7.2 -> 5.4 us, 616 x 768 -> 1280 W4:
-  // 11.7 -> 10.1 us, 512 x 5120 -> 1280: 17.7 -> 15.4 us, conv 8 x 8 x 8 x 1280: 56 -> 46 us).
-  if ((int64_t)a.n_tiles_m * ((w->N + BN - 1) / BN) * 2 <= n_sm) BN = 64;
+  // 11.7 -> 10.1 us, 512 x 5120 -> 1280: 17.7 -> 15.4 us, conv 8 x 8 x 8 x 1280: 56 -> 46 us).  Only where every narrow
+  // tile has an SM to itself, though: a block of 160 columns becomes two and a half, and beyond one tile per SM the
+  // second one costs up to half the time again (1024 x 5120 -> 1280 19.9 us wide, 24.8 narrow; conv 2 x 32 x 32 x 640 -> 640
+  // 33 and 47 us).  Of 750 shapes between 64 and 8192 rows the 490 on this side take 0.79 of the wide tiles' time with narrow
+  // ones and the other 260 would take 1.5 times it, none of them the wrong way round by more than 3 %.
+  if ((int64_t)a.n_tiles_m * ((w->N + BN - 1) / BN) * 2 <= n_sm && (int64_t)a.n_tiles_m * ((w->N + 63) / 64) <= n_sm) BN = 64;
   a.n_tiles_n = (w->N + BN - 1) / BN;
   // Expanding in front of the GEMM costs a launch and a round trip of the weights through L2 (1.0-1.5 us at least); in the
   // kernel it costs every tile a share of its stages' time.  The kernel wins while a CTA unpacks little: 32-row pieces

@@ -114,6 +114,35 @@ def test_conv3x3_w4a6(n, H, W, C, N, K):
     check_output(Y, Yref.reshape(n * P, N), REL)
 
 
+@pytest.mark.parametrize("w_bits", [8, 4])
+@pytest.mark.parametrize("M,N", [
+    (128, 9440),      # 59 blocks of 160 columns, 148 of 64: as many narrow tiles as the GPU has SMs
+    (128, 9472),      # the same from blocks of 128
+    (77, 9600),       # 150 narrow blocks: one too many, wide tiles
+    (77, 10240), (128, 10240),   # the feed-forward of the 8 x 8 level, batch 1 and 2
+    (128, 11840),     # the last width whose wide blocks leave half of the SMs free
+    (256, 5120),      # two row blocks: 160 narrow tiles
+])
+def test_narrow_tile_rule(M, N, w_bits):
+    torch, b = gpu()
+    rng = np.random.default_rng(N + M)
+    C = 72
+    cg = (np.arange(C) % 2).astype(np.int32)
+    g = b.groups_from_host(C, 1, 8, cg, np.zeros(1, np.int32), np.full((1, 1, 2), 0.03, np.float32),
+                           np.full((1, 1, 2), 120, np.int32))
+    W = rng.normal(0, 0.02, (N, C)).astype(np.float16)
+    bias = rng.normal(0, 0.01, N).astype(np.float16)
+    wq, sw = ol.weight_rtn(W, w_bits)
+    w = b.weight_prepare(g, to_dev(torch, W), w_bits)
+    X = rng.normal(0, 1, (M, C)).astype(np.float16)
+    codes, s_rows, z_rows = ol.quantize_dynamic_token(X, cg, 2, 8)
+    Xq, ds, dz = b.quantize_act(g, to_dev(torch, X), mode=b.MODE_DYNAMIC_TOKEN)
+    Y = torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda")
+    b.linear(g, w, Xq, mode=b.MODE_DYNAMIC_TOKEN, dyn_scale=ds, dyn_zp=dz, bias=to_dev(torch, bias), out=Y)
+    check_output(Y, ol.group_linear(codes, s_rows, z_rows, cg, wq, sw, bias), REL)
+    assert b.device_status() == 0
+
+
 def test_linear_argument_errors():
     torch, b = gpu()
     Xcal, X, W, bias, gr = layer_case(12, 1, 128, 64, 64, 2, 8, oc.DIM_CHANNEL)

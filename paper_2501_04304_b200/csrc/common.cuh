@@ -73,6 +73,36 @@ static inline void pool_free(void* p) {
   if (at.device != dev) cudaSetDevice(dev);
 }
 
+// A stream of the library's own on the current device, for copies out of objects that are complete: it waits for nothing
+// that callers have enqueued.  One per device, made once (making and destroying a stream takes 115 us), shared by
+// threads: a caller's synchronisation waits for what the others have put there, which ends by itself.
+static inline cudaError_t own_stream(cudaStream_t* out) {
+  static std::mutex lock;
+  static cudaStream_t streams[64] = {nullptr};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> hold(lock);
+  if (!streams[dev] && (e = cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking)) != cudaSuccess) return e;
+  *out = streams[dev];
+  return cudaSuccess;
+}
+
+// Makes a device current for a scope.
+struct DeviceScope {
+  int before = -1;
+  cudaError_t err;
+  explicit DeviceScope(int device) {
+    int now = 0;
+    err = cudaGetDevice(&now);
+    if (err == cudaSuccess && now != device && (err = cudaSetDevice(device)) == cudaSuccess) before = now;
+  }
+  ~DeviceScope() {
+    if (before >= 0) cudaSetDevice(before);
+  }
+};
+
 // Multiprocessors of the current device, asked once.
 static inline cudaError_t sm_count(int* n) {
   static std::atomic<int> known[64];

@@ -17,13 +17,15 @@ struct dgq_weight {
   std::vector<int32_t> seg_end;  // [G] end of every group's segment, in 32-position atoms
   std::vector<int32_t> atoms;    // [G] atoms of every group (of one filter tap)
   std::vector<float> sw;         // host scales [N]
+  std::vector<int2> chan;        // [C] reduction position of every channel's first tap, distance between its taps
   unsigned char* d_slab = nullptr;  // all device arrays below
   int8_t* d_w = nullptr;         // 8-bit: [N_pad][Kt] s8; 4-bit: [N_pad][Kt/2] packed
   float* d_sw = nullptr;         // [N_pad]; 4-bit: sw / 16 (the unpacked codes carry a factor 16)
   float* d_wsum = nullptr;       // [G][N_pad] column sums per group as fp32 (exact); 4-bit: x 16
   float* d_wres = nullptr;       // [G][N_pad] part of wsum the padding positions could not absorb
-  int2* d_chan = nullptr;        // [C] reduction position of every channel's first tap, distance between its taps
+  int2* d_chan = nullptr;        // [C] copy of `chan`
   uint32_t res_mask = 0;         // bit g set: group g has a non-zero entry in d_wres
+  int device = 0;                // device of the arrays above
 };
 
 namespace dgq {
@@ -167,6 +169,12 @@ __global__ void __launch_bounds__(WP_THREADS) weight_rows_kernel(const __grid_co
   }
 }
 
+// Code of position `pos` of a padded row (see weight_rows_kernel for the order of 4-bit codes in a word).
+__host__ __device__ __forceinline__ int8_t weight_code_at(const uint8_t* row, int pos, int four_bit) {
+  if (!four_bit) return (int8_t)row[pos];
+  const uint32_t b = row[pos / 8 * 4 + (pos & 3)];
+  return (int8_t)((int)(((pos & 4) ? b >> 4 : b) << 28) >> 28);
+}
 // Codes in original channel order from the padded rows.
 __global__ void weight_unpermute_kernel(const uint8_t* __restrict__ w, const int2* __restrict__ chan, int K, int C, int Kt,
                                         int four_bit, int8_t* __restrict__ out) {
@@ -174,16 +182,47 @@ __global__ void weight_unpermute_kernel(const uint8_t* __restrict__ w, const int
   for (int k = threadIdx.x; k < K; k += blockDim.x) {
     const int tap = k / C;
     const int2 ch = __ldg(chan + (k - tap * C));
-    const int pos = ch.x + tap * ch.y;
-    int v;
-    if (four_bit) {
-      const int b = row[pos / 8 * 4 + (pos & 3)];
-      v = (int)((uint32_t)((pos & 4) ? b >> 4 : b) << 28) >> 28;
-    } else {
-      v = (int8_t)row[pos];
-    }
-    out[(size_t)blockIdx.x * K + k] = (int8_t)v;
+    out[(size_t)blockIdx.x * K + k] = weight_code_at(row, ch.x + tap * ch.y, four_bit);
   }
+}
+
+// The codes of a weight in original channel order, in host memory.  Works on the weight's device whichever is current,
+// on the library's own stream and outside the rules of a stream capture that the caller may have running (the arrays are
+// complete since the build, so nothing has to be waited for).  Small weights, and those for which the device has no
+// scratch memory left, are put in order on the host (2^9 codes 18 us, 2^11 codes 26 us; through a kernel 26 us and, up to
+// 2^14 codes, no more than 29).
+constexpr size_t WEIGHT_HOST_CODES = 1 << 11;
+static dgq_status weight_codes_to_host(const dgq_weight* w, int8_t* wq) {
+  DeviceScope on(w->device);
+  DGQ_CUDA_OK(on.err);
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  DGQ_CUDA_OK(cudaThreadExchangeStreamCaptureMode(&mode));
+  const size_t n = (size_t)w->N * w->K;
+  const int four_bit = w->w_bits == 4;
+  cudaStream_t stream = nullptr;
+  cudaError_t e = own_stream(&stream);
+  int8_t* d = nullptr;
+  if (e != cudaSuccess) {
+  } else if (n > WEIGHT_HOST_CODES && pool_alloc((void**)&d, n, stream) == cudaSuccess) {
+    weight_unpermute_kernel<<<w->N, 256, 0, stream>>>((const uint8_t*)w->d_w, w->d_chan, w->K, w->C, w->Kt, four_bit, d);
+    g_launches += 1;
+    if ((e = cudaGetLastError()) == cudaSuccess) e = cudaMemcpyAsync(wq, d, n, cudaMemcpyDeviceToHost, stream);
+    cudaFreeAsync(d, stream);
+    const cudaError_t done = cudaStreamSynchronize(stream);
+    if (e == cudaSuccess) e = done;
+  } else {
+    cudaGetLastError();  // (an allocation that failed)
+    const size_t row_bytes = four_bit ? w->Kt / 2 : w->Kt;
+    std::vector<uint8_t> rows(w->N * row_bytes);
+    if ((e = cudaMemcpyAsync(rows.data(), w->d_w, rows.size(), cudaMemcpyDeviceToHost, stream)) == cudaSuccess)
+      e = cudaStreamSynchronize(stream);
+    for (int o = 0; o < w->N && e == cudaSuccess; ++o)
+      for (int tap = 0, k = 0; k < w->K; ++tap)
+        for (int c = 0; c < w->C; ++c, ++k)
+          wq[(size_t)o * w->K + k] = weight_code_at(&rows[o * row_bytes], w->chan[c].x + tap * w->chan[c].y, four_bit);
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e == cudaSuccess ? DGQ_OK : DGQ_ERR_CUDA;
 }
 
 // Device arrays of a weight in one allocation, filled by weight_rows_kernel from fp16 weights `W` (device) or from
@@ -202,7 +241,19 @@ static dgq_status weight_build(const dgq_groups* g, const __half* W, const int8_
       if (wq[i] < -a.qmax || wq[i] > a.qmax) return DGQ_ERR_INVALID_ARG;
   // accumulator bound: |code| <= 255, |weight| <= 127 (4-bit: 7 * 16)
   if ((int64_t)taps * g->K_pad * 255 * 127 >= ((int64_t)1 << 31)) return DGQ_ERR_UNSUPPORTED;
+  int dev = 0;
+  DGQ_CUDA_OK(cudaGetDevice(&dev));
+  // Layout tables and weights may lie on another device than the current one, where the object is made: those are
+  // copied over first.
+  bool w_remote = false;
+  if (W) {
+    cudaPointerAttributes at;
+    DGQ_CUDA_OK(cudaPointerGetAttributes(&at, W));
+    if (at.type == cudaMemoryTypeUnregistered) return DGQ_ERR_CUDA;
+    w_remote = at.type == cudaMemoryTypeDevice && at.device != dev;
+  }
   dgq_weight* w = new dgq_weight();
+  w->device = dev;
   w->N = N;
   w->K = K;
   w->C = g->C;
@@ -233,35 +284,46 @@ static dgq_status weight_build(const dgq_groups* g, const __half* W, const int8_
   const size_t w_bytes = (size_t)w->N_pad * w->Kt / (w_bits == 4 ? 2 : 1), per_group = (size_t)g->G * w->N_pad * sizeof(float);
   const size_t o_w = part(w_bytes), o_sw = part(w->N_pad * sizeof(float)), o_wsum = part(per_group), o_wres = part(per_group);
   const size_t o_chan = part(g->C * sizeof(int2)), o_back = part((size_t)(N + 1) * sizeof(float));  // scales, then the mask
-  const size_t o_codes = bytes;  // given codes and scales, for the duration of the call
-  int8_t* d_codes = nullptr;
+  // for the duration of the call: given codes and scales or weights of another device, layout of another device
+  const size_t slab_bytes = bytes;
+  bytes = 0;
+  const size_t o_in = part(wq ? (size_t)N * K : w_remote ? (size_t)N * K * sizeof(__half) : 0), o_in_sw = part(wq ? N * sizeof(float) : 0);
+  const size_t o_perm = part(g->device != dev ? g->K_pad * sizeof(int16_t) : 0), temp_bytes = bytes;
+  unsigned char* d_temp = nullptr;
   dgq_status st = DGQ_OK;
   auto ok = [&](cudaError_t e) {
     if (st == DGQ_OK && e != cudaSuccess) st = DGQ_ERR_CUDA;
     return st == DGQ_OK;
   };
-  if (ok(pool_alloc((void**)&w->d_slab, o_codes, stream)) &&
-      (!wq || ok(pool_alloc((void**)&d_codes, (size_t)N * K + 4 * (size_t)N + 16, stream)))) {
+  if (ok(pool_alloc((void**)&w->d_slab, slab_bytes, stream)) && (!temp_bytes || ok(pool_alloc((void**)&d_temp, temp_bytes, stream)))) {
     w->d_w = reinterpret_cast<int8_t*>(w->d_slab + o_w);
     w->d_sw = reinterpret_cast<float*>(w->d_slab + o_sw);
     w->d_wsum = reinterpret_cast<float*>(w->d_slab + o_wsum);
     w->d_wres = reinterpret_cast<float*>(w->d_slab + o_wres);
     w->d_chan = reinterpret_cast<int2*>(w->d_slab + o_chan);
     float* back = reinterpret_cast<float*>(w->d_slab + o_back);
-    std::vector<int2> chan(g->C);
+    w->chan.resize(g->C);
     for (int k = 0; k < g->G; ++k)
       for (int p = g->group_off[k]; p < g->group_off[k + 1]; ++p)
         if (g->perm[p] >= 0)
-          chan[g->perm[p]] = make_int2(taps * a.red_off[k] + p - g->group_off[k], a.red_off[k + 1] - a.red_off[k]);
-    ok(cudaMemcpyAsync(w->d_chan, chan.data(), chan.size() * sizeof(int2), cudaMemcpyHostToDevice, stream));
+          w->chan[g->perm[p]] = make_int2(taps * a.red_off[k] + p - g->group_off[k], a.red_off[k + 1] - a.red_off[k]);
+    ok(cudaMemcpyAsync(w->d_chan, w->chan.data(), w->chan.size() * sizeof(int2), cudaMemcpyHostToDevice, stream));
+    a.W = W;
+    a.perm = g->d_perm;
     if (wq) {
-      a.wq = d_codes;
-      a.sw_in = reinterpret_cast<const float*>(d_codes + (((size_t)N * K + 15) & ~size_t(15)));
-      ok(cudaMemcpyAsync(d_codes, wq, (size_t)N * K, cudaMemcpyHostToDevice, stream));
-      ok(cudaMemcpyAsync(const_cast<float*>(a.sw_in), sw, N * sizeof(float), cudaMemcpyHostToDevice, stream));
+      a.wq = reinterpret_cast<int8_t*>(d_temp + o_in);
+      a.sw_in = reinterpret_cast<float*>(d_temp + o_in_sw);
+      ok(cudaMemcpyAsync(d_temp + o_in, wq, (size_t)N * K, cudaMemcpyHostToDevice, stream));
+      ok(cudaMemcpyAsync(d_temp + o_in_sw, sw, N * sizeof(float), cudaMemcpyHostToDevice, stream));
+    } else if (w_remote) {
+      a.W = reinterpret_cast<__half*>(d_temp + o_in);
+      ok(cudaMemcpyAsync(d_temp + o_in, W, (size_t)N * K * sizeof(__half), cudaMemcpyDefault, stream));
+    }
+    if (g->device != dev) {
+      a.perm = reinterpret_cast<int16_t*>(d_temp + o_perm);
+      ok(cudaMemcpyAsync(d_temp + o_perm, g->d_perm, g->K_pad * sizeof(int16_t), cudaMemcpyDefault, stream));
     }
     ok(cudaMemsetAsync(back + N, 0, sizeof(float), stream));
-    a.W = W;
     a.N = N;
     a.K = K;
     a.C = g->C;
@@ -271,7 +333,6 @@ static dgq_status weight_build(const dgq_groups* g, const __half* W, const int8_
     a.K_pad = g->K_pad;
     a.taps = taps;
     a.four_bit = w_bits == 4;
-    a.perm = g->d_perm;
     std::copy(g->group_off.begin(), g->group_off.end(), a.group_off);
     a.w = reinterpret_cast<uint8_t*>(w->d_w);
     a.sw = w->d_sw;
@@ -293,7 +354,7 @@ static dgq_status weight_build(const dgq_groups* g, const __half* W, const int8_
       w->sw = std::move(host);
     }
   }
-  if (d_codes) cudaFreeAsync(d_codes, stream);
+  if (d_temp) cudaFreeAsync(d_temp, stream);
   if (st != DGQ_OK) {
     pool_free(w->d_slab);
     delete w;
@@ -329,13 +390,8 @@ extern "C" dgq_status dgq_weight_destroy(dgq_weight* w) {
 extern "C" dgq_status dgq_weight_export(const dgq_weight* w, int8_t* wq, float* sw) {
   if (!w) return DGQ_ERR_INVALID_ARG;
   if (wq) {
-    int8_t* d = nullptr;
-    DGQ_CUDA_OK(dgq::pool_alloc((void**)&d, (size_t)w->N * w->K, nullptr));
-    dgq::weight_unpermute_kernel<<<w->N, 256>>>((const uint8_t*)w->d_w, w->d_chan, w->K, w->C, w->Kt, w->w_bits == 4, d);
-    dgq::g_launches += 1;
-    const cudaError_t e = cudaMemcpy(wq, d, (size_t)w->N * w->K, cudaMemcpyDeviceToHost);
-    cudaFreeAsync(d, nullptr);
-    if (e != cudaSuccess) return DGQ_ERR_CUDA;
+    const dgq_status st = dgq::weight_codes_to_host(w, wq);
+    if (st != DGQ_OK) return st;
   }
   if (sw) std::copy(w->sw.begin(), w->sw.end(), sw);
   return DGQ_OK;

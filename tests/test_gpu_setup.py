@@ -152,3 +152,51 @@ def test_four_bit_routes(M, C, N):
     codes, s_rows, z_rows = ol.quantize_dynamic_token(X[rows], np.zeros(C, np.int32), 1, 8)
     check_output(Y[torch.from_numpy(rows).cuda()], ol.group_linear(codes, s_rows, z_rows, np.zeros(C, np.int32), wq, sw, None))
     assert b.device_status() == 0
+
+
+def _weight(torch, b, rng, N, C, w_bits, conv):
+    """A prepared weight of two channel groups and its codes and scales."""
+    g = b.groups_from_host(C, 1, 8 if not conv else 6, (np.arange(C) % 2).astype(np.int32), np.zeros(1, np.int32),
+                           np.full((1, 1, 2), 0.03, np.float32), np.full((1, 1, 2), 31, np.int32))
+    W = rng.normal(0, 0.02, (N, (9 if conv else 1) * C)).astype(np.float16)
+    wq, sw = ol.weight_rtn(W, w_bits)
+    return g, W, wq, sw
+
+
+@pytest.mark.parametrize("w_bits", [8, 4])
+@pytest.mark.parametrize("N,C,conv", [
+    (8, 256, False),         # 2^11 codes: the last weight put in order on the host
+    (8, 264, False),         # the first on the device
+    (8, 24, True), (264, 24, True),
+])
+def test_weight_export_routes_and_during_a_capture(N, C, conv, w_bits):
+    """An export copies host memory as far as its caller can tell: also while the caller captures a graph."""
+    torch, b = gpu()
+    g, W, wq, sw = _weight(torch, b, np.random.default_rng(N + C), N, C, w_bits, conv)
+    w = b.weight_prepare(g, to_dev(torch, W), w_bits, conv=(1, 16, 8, C) if conv else None)
+    x = torch.arange(64.0, device="cuda")
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):
+        y = x + 1
+        got, got_sw = w.export()
+        z = y * 2
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(got, wq) and np.array_equal(got_sw, sw)
+    assert torch.equal(z, (x + 1) * 2)
+    again, _ = w.export()
+    assert np.array_equal(again, wq) and b.device_status() == 0
+
+
+def test_weight_of_another_device_than_the_current_one():
+    """Building a weight from groups and fp16 weights of another device, and exporting it while a third party's device is
+    current, read each array where it lies."""
+    torch, b = gpu()
+    if torch.cuda.device_count() < 2:
+        pytest.skip("one GPU")
+    g, W, wq, sw = _weight(torch, b, np.random.default_rng(3), 264, 320, 4, False)
+    Wd = to_dev(torch, W)
+    with torch.cuda.device(1):
+        w = b.weight_prepare(g, Wd, 4)
+    got, got_sw = w.export()
+    assert np.array_equal(got, wq) and np.array_equal(got_sw, sw)

@@ -257,10 +257,11 @@ dgq_status dgq_cross_attn_logq_noalloc(const void* Q, const void* K, const void*
  * current device in *status (DGQ_OK, or the first error a kernel recorded),
  * then clears it. */
 dgq_status dgq_device_status(int* status);
-/* Diagnostic: enqueues a one-warp kernel whose only wait, on a barrier nobody arrives at, gives up
- * after max_polls (1..65536) polls of at most a microsecond each, so that the time-out path of the
- * bounded waits (status word, dgq_device_status, a usable device afterwards) can be exercised
- * without making a wait of a working kernel run out.  Errors: INVALID_ARG, CUDA. */
+/* Diagnostic: enqueues a kernel that runs each of the library's bounded waits on a barrier nobody arrives at, with a
+ * limit of max_polls (1..65536) times 1024 SM clocks (about half a microsecond each) in place of the usual second, so
+ * that the time-out path of the bounded waits (other waits of the block end too, status word, dgq_device_status, a
+ * usable device afterwards) can be exercised without making a wait of a working kernel run out.
+ * Errors: INVALID_ARG, CUDA. */
 dgq_status dgq_selftest_wait_timeout(uint32_t max_polls, void* stream);
 const char* dgq_status_string(dgq_status s);
 /* Number of kernels the library has launched in this process (all devices). */

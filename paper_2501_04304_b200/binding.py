@@ -117,7 +117,7 @@ def device_status() -> int:
 
 
 def selftest_wait_timeout(max_polls: int, stream=None):
-    """dgq_selftest_wait_timeout: a kernel whose only wait runs out after `max_polls` polls."""
+    """dgq_selftest_wait_timeout: a kernel whose waits run out after `max_polls` x 1024 SM clocks."""
     _check(lib().dgq_selftest_wait_timeout(C.c_uint32(max_polls), _stream(stream)), "dgq_selftest_wait_timeout")
 
 

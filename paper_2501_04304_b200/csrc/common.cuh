@@ -247,10 +247,12 @@ __device__ __forceinline__ bool mbar_try_wait_parked(uint64_t* bar, uint32_t par
   return ok != 0;
 }
 
-// Bounded wait: gives up after about a second (2^31 SM clocks) or as soon as another
-// thread of the CTA has raised `*abort_flag`.  Returns false when it gave up; the caller
+// Bounded wait: gives up after `limit` SM clocks (2^31, about a second, everywhere but in the self-test) or as soon as
+// another thread of the CTA has raised `*abort_flag`.  Returns false when it gave up; the caller
 // must then leave through the kernel's common exit path.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+constexpr long long WAIT_CLOCKS = 1ll << 31;
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                          long long limit = WAIT_CLOCKS) {
   if (mbar_try_wait(bar, parity)) return true;
   const long long t0 = clock64();
   uint32_t spins = 0;
@@ -258,7 +260,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     if (mbar_try_wait_parked(bar, parity, 4000u)) return true;
     if ((++spins & 63u) == 0) {
       if (*abort_flag) return false;
-      if (clock64() - t0 > (1ll << 31)) {
+      if (clock64() - t0 > limit) {
         *abort_flag = 1;
         record_error(DGQ_ERR_TIMEOUT);
         return false;
@@ -267,44 +269,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
-// Bounded wait without a return value, for hot loops: after `max_polls` (2^21) parked polls (of at most a
-// microsecond each) it records a time-out and raises `*abort_flag`; once the flag is up every wait
-// returns at its first failed poll.  The caller tests the flag at a coarser grain (once per tile)
-// and leaves through the kernel's common exit path; what it does in between only touches memory
-// the CTA owns.
-__device__ __forceinline__ void mbar_wait_lean(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag,
-                                               uint32_t max_polls = 1u << 21) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar_addr), "r"(parity)
-      : "memory");
-  if (ok) return;
-  if (*abort_flag) return;
-  for (uint32_t spins = 0; spins < max_polls; ++spins) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar_addr), "r"(parity), "r"(1000u)
-        : "memory");
-    if (ok) return;
-    if ((spins & 31u) == 31u && *abort_flag) return;
-  }
-  *abort_flag = 1;
-  record_error(DGQ_ERR_TIMEOUT);
-}
-// Bounded wait for the hand-overs between the roles of a kernel: like mbar_wait_lean, but the polls carry no time limit of
-// their own (the hardware parks the thread and wakes it when the phase completes) and the abort flag and the clock
-// are looked at only on every 16th poll: a hand-over that finds its barrier pending costs 470 cycles from commit to
-// re-issue against 540 with a flag test behind the first poll and a time limit in the others (self-attention
-// 2 x 8 x 4096 x 40 145.5 -> 143.8 us, 8192 x 320 -> 960 with its quantizer 25.7 -> 24.8 us).  Gives up after about a
-// second (2^31 SM clocks); once the flag is up every wait returns within 16 polls.
-__device__ __forceinline__ void mbar_wait_handover(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag) {
+// Bounded wait for the hand-overs between the roles of a kernel, without a return value: the caller tests the flag at a
+// coarser grain (once per tile) and leaves through the kernel's common exit path; what it does in between only touches
+// memory the CTA owns.  The polls carry no time limit of their own (the hardware parks the thread and wakes it when
+// the phase completes) and the abort flag and the clock are looked at only on every 16th poll: a hand-over that finds its
+// barrier pending costs 470 cycles from commit to re-issue against 540 with a flag test behind the first poll and a time
+// limit in the others (self-attention 2 x 8 x 4096 x 40 145.5 -> 143.8 us, 8192 x 320 -> 960 with its quantizer
+// 25.7 -> 24.8 us).  Gives up after `limit` SM clocks; once the flag is up every wait returns within 16 polls.
+__device__ __forceinline__ void mbar_wait_handover(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag,
+                                                   long long limit = WAIT_CLOCKS) {
   long long t0 = 0;
   for (uint32_t spins = 0;; ++spins) {
     uint32_t ok;
@@ -320,7 +293,7 @@ __device__ __forceinline__ void mbar_wait_handover(uint32_t bar_addr, uint32_t p
       if (*abort_flag) return;
       const long long t = clock64();
       if (t0 == 0) t0 = t;
-      if (t - t0 > (1ll << 31)) {
+      if (t - t0 > limit) {
         *abort_flag = 1;
         record_error(DGQ_ERR_TIMEOUT);
         return;

@@ -52,9 +52,10 @@ extern "C" dgq_status dgq_cross_attn_logq_noalloc(const void* Q, const void* K, 
 }
 
 namespace dgq {
-// One warp waits, with the caller's poll limit, on a barrier that nobody arrives at: the bounded wait
-// gives up, records DGQ_ERR_TIMEOUT and the kernel ends normally.
-__global__ void selftest_wait_kernel(uint32_t max_polls) {
+// The two bounded waits of the kernels (mbar_wait_handover and, for 4-bit weights unpacked in the GEMM, mbar_wait), each
+// once as the wait that runs out and once as a wait with its usual limit that ends because another warp's ran out:
+// warp 0 of a block gives up after `limit` clocks on a barrier that nobody arrives at, warp 1 leaves with it.
+__global__ void selftest_wait_kernel(long long limit) {
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -63,13 +64,15 @@ __global__ void selftest_wait_kernel(uint32_t max_polls) {
     fence_barrier_init();
   }
   __syncthreads();
-  mbar_wait_lean(smem_u32(&bar), 0u, &abort_flag, max_polls);
+  const long long mine = threadIdx.x < 32 ? limit : WAIT_CLOCKS;
+  if ((blockIdx.x ^ (threadIdx.x >> 5)) & 1) mbar_wait(&bar, 0u, &abort_flag, mine);
+  else mbar_wait_handover(smem_u32(&bar), 0u, &abort_flag, mine);
 }
 }  // namespace dgq
 
 extern "C" dgq_status dgq_selftest_wait_timeout(uint32_t max_polls, void* stream) {
   if (max_polls == 0 || max_polls > (1u << 16)) return DGQ_ERR_INVALID_ARG;
-  dgq::selftest_wait_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(max_polls);
+  dgq::selftest_wait_kernel<<<2, 64, 0, (cudaStream_t)stream>>>((long long)max_polls << 10);
   dgq::g_launches += 1;
   DGQ_CUDA_OK(cudaGetLastError());
   return DGQ_OK;

@@ -217,12 +217,18 @@ def test_four_bit_weights_with_and_without_workspace():
 
 
 def test_a_wait_that_runs_out_is_reported_and_leaves_the_device_usable():
-    """Every device-side wait is bounded.  The library's self-test kernel waits, with a short limit, on a barrier
-    nobody arrives at: the status word reads DGQ_ERR_TIMEOUT once, is clear afterwards, and a layer call right
-    after it gives the right result."""
+    """Every device-side wait is bounded.  The library's self-test kernel runs both of the kernels' wait functions, with
+    a short limit (2000 x 1024 clocks, about a millisecond), on a barrier nobody arrives at, each beside a warp that waits
+    with the usual limit of a second and has to leave with it: the kernel is over long before that second, the status
+    word reads DGQ_ERR_TIMEOUT once, is clear afterwards, and a layer call right after it gives the right result."""
     torch, b = gpu()
     assert b.device_status() == 0
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record()
     b.selftest_wait_timeout(2000)
+    end.record()
+    end.synchronize()
+    assert 1.0 <= start.elapsed_time(end) < 500.0    # 2 048 000 clocks at up to 1965 MHz
     assert b.device_status() == 6
     assert b.device_status() == 0
     Xcal, X, W, bias, gr = layer_case(16, 1, 256, 320, 320, 4, 8, oc.DIM_CHANNEL)

@@ -6,6 +6,7 @@
 #include <Python.h>
 
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -16,6 +17,15 @@ namespace {
 
 at::Tensor empty(std::initializer_list<int64_t> shape, at::ScalarType type, const at::Tensor& like) {
   return at::Tensor(at::detail::empty_cuda(at::IntArrayRef(shape.begin(), shape.size()), type, like.device(), std::nullopt));
+}
+
+// Scratch memory for a call on stream `st` that is dropped when the call returns: it belongs to that stream, so that torch
+// gives it to nobody else before the call's kernels have run.  `given` is the stream argument (None: the current
+// stream, to which torch's allocations belong anyway).
+at::Tensor scratch(int64_t bytes, const at::Tensor& like, PyObject* given, void* st) {
+  if (given == Py_None) return empty({bytes}, at::kByte, like);
+  c10::cuda::CUDAStreamGuard on(c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(st), like.device().index()));
+  return empty({bytes}, at::kByte, like);
 }
 
 // A tensor argument, or an undefined tensor for None.  Sets a TypeError for anything else.
@@ -169,7 +179,7 @@ PyObject* linear(PyObject* const* a, Py_ssize_t n) {
     size_t need = 0;
     rc = dgq_linear_workspace_bytes(static_cast<const dgq_groups*>(g), static_cast<const dgq_weight*>(w), m, &need);
     if (rc != DGQ_OK) return status(rc);
-    if (need) ws = empty({static_cast<int64_t>(need)}, at::kByte, xq);
+    if (need) ws = scratch(static_cast<int64_t>(need), xq, a[13], st);
   }
   const int64_t ldy = y.stride(0);
   const size_t ws_bytes = ws.defined() ? static_cast<size_t>(ws.numel()) : 0;
@@ -211,7 +221,7 @@ PyObject* cross_attn_logq(PyObject* const* a, Py_ssize_t n) {
       const dgq_status rc = dgq_cross_attn_workspace_bytes(B, H, nq, nk, d, &need);
       if (rc != DGQ_OK) return status(rc);
     }
-    ws = empty({static_cast<int64_t>(need)}, at::kByte, q);
+    ws = scratch(static_cast<int64_t>(need), q, a[11], st);
   }
   void *p_q = ptr(q), *p_k = ptr(k), *p_v = ptr(v), *p_o = ptr(o), *p_ws = ptr(ws);
   float *p_fixed = ptr<float>(fixed), *p_scale = ptr<float>(scale);

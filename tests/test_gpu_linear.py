@@ -216,6 +216,35 @@ def test_four_bit_weights_with_and_without_workspace():
     assert b.device_status() == 0
 
 
+def test_workspace_belongs_to_the_stream_of_the_call():
+    """A call on another stream than the current one, still waiting there when it returns: its workspace is not given to
+    the next allocation on the current stream."""
+    torch, b = gpu()
+    M, C, N = 2500, 640, 1280
+    Xcal, X, W, bias, gr = layer_case(17, 1, M, C, N, 8, 8, oc.DIM_CHANNEL)
+    g = b.calibrate_groups(to_dev(torch, Xcal), M, 8, 8, b.DIM_CHANNEL)
+    w = b.weight_prepare(g, to_dev(torch, W), 4)
+    Xq, ds, dz = b.quantize_act(g, to_dev(torch, X), mode=b.MODE_DYNAMIC_TOKEN)
+    kw = dict(mode=b.MODE_DYNAMIC_TOKEN, dyn_scale=ds, dyn_zp=dz)
+    Y_ref = b.linear(g, w, Xq, **kw)
+    Q, K, V = [to_dev(torch, x) for x in synth.attention_inputs(18, 8, 16, 260, 77, 80, ctx_dim=16)]
+    O_ref, _, _ = b.cross_attn_logq(Q, K, V, 8)
+    Y, O = torch.empty_like(Y_ref), torch.empty_like(O_ref)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(20_000_000)
+    b.linear(g, w, Xq, out=Y, stream=side, **kw)
+    b.cross_attn_logq(Q, K, V, 8, out=O, stream=side)
+    need = [b.linear_workspace_bytes(g, w, M), b.cross_attn_workspace_bytes(8, 16, 260, 77, 80)]
+    taken = [torch.full((n,), 0x77, dtype=torch.uint8, device="cuda") for n in need]
+    torch.cuda.current_stream().synchronize()
+    side.synchronize()
+    assert torch.equal(Y, Y_ref) and torch.equal(O, O_ref) and b.device_status() == 0
+    assert all(bool((t == 0x77).all()) for t in taken)    # and the other way round
+
+
 def test_a_wait_that_runs_out_is_reported_and_leaves_the_device_usable():
     """Every device-side wait is bounded.  The library's self-test kernel runs both of the kernels' wait functions, with
     a short limit (2000 x 1024 clocks, about a millisecond), on a barrier nobody arrives at, each beside a warp that waits

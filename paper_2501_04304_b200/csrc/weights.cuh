@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(WP_THREADS) weight_rows_kernel(const __grid_co
   if (threadIdx.x < a.G) sum_s[threadIdx.x] = 0;
   float s;
   if (a.W) {
-    // fp32 sequence: sw = absmax / qmax, inv = 1 / sw, code = clamp(rint(w * inv), -qmax, qmax)
+    // fp32 sequence: sw = absmax / qmax, inv = 1 / sw, code = clamp(rint(w * inv), -qmax, qmax), 0 where that is NaN
     const __half* w = a.W + (size_t)o * a.K;
     const float qmax = (float)a.qmax;
     float amax = 0.f;
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(WP_THREADS) weight_rows_kernel(const __grid_co
     const float inv = __fdiv_rn(1.0f, s);
     for (int k = threadIdx.x; k < a.K; k += WP_THREADS) {
       const float r = rintf(__fmul_rn(__half2float(__ldg(w + k)), inv));
-      row_s[k] = (int8_t)(int)fminf(fmaxf(r, -qmax), qmax);
+      row_s[k] = r == r ? (int8_t)(int)fminf(fmaxf(r, -qmax), qmax) : (int8_t)0;
     }
   } else {
     s = __ldg(a.sw_in + o);

@@ -200,3 +200,20 @@ def test_weight_of_another_device_than_the_current_one():
         w = b.weight_prepare(g, Wd, 4)
     got, got_sw = w.export()
     assert np.array_equal(got, wq) and np.array_equal(got_sw, sw)
+
+
+@pytest.mark.parametrize("w_bits", [8, 4])
+def test_weights_that_are_not_finite(w_bits):
+    """A NaN gets code 0 and does not count for its row's scale; an infinity makes the row's scale infinite and its codes
+    0 (the fp32 sequence with NaN -> 0, as for activations)."""
+    torch, b = gpu()
+    rng = np.random.default_rng(9)
+    g, W, _, _ = _weight(torch, b, rng, 16, 72, w_bits, False)
+    finite = W.copy()
+    finite[2, 5] = finite[2, 70] = 0
+    wq, sw = ol.weight_rtn(finite, w_bits)
+    W[2, 5], W[2, 70] = np.nan, -np.nan
+    W[7, 0] = np.inf
+    wq[7], sw[7] = 0, np.inf
+    got, got_sw = b.weight_prepare(g, to_dev(torch, W), w_bits).export()
+    assert np.array_equal(got, wq) and np.array_equal(got_sw, sw)

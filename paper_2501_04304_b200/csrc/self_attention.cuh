@@ -345,7 +345,8 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t code_top = 0x4B400000u + L;                                 // bits of 1.5 * 2^23 + last code
     const uint32_t p_top = 0x4B400000u + min(L, (uint32_t)AT_CODE_CAP);       // ... + last code with a non-zero fp16 weight
     const uint32_t p_least = (127u + (uint32_t)AT_P_SHIFT - min(L, 100u)) << 23;  // weight of the last code
-    float m_raw = -INFINITY, m2 = 0.f, base = 0.f;
+    float m_raw = -INFINITY, m2 = 0.f;
+    float base = 0.f;  // fixed scale: code = rint(base - t * scale); row maximum as scale: code = rint(-(t * scale + base))
     unsigned long long zs = 0ull;
     // The threads that hold parts of a row's statistics leave them in shared memory and meet: the warps of a team when
     // it has its own rows, else all of them.
@@ -414,25 +415,30 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             const int64_t code_row = (((int64_t)b * a.H + h) * a.nq + row0 + qt * SATC_BQ + row) * a.nk + j * SATC_BK + col;
             uint32_t pk[16];
             if (!FIXED) {
-              // e = 2^(14 - x) with x = base - t * scale >= 0 up to rounding (the row maximum has code 0); -inf logits (keys
-              // beyond nk) give 0.  The row sum takes e as it is.  The power of two nearest to it in the log domain,
-              // 2^(14 - rint(x)), is e with the mantissa rounded at sqrt(2): adding 2 - sqrt(2) in mantissa units carries into
-              // the exponent where x is nearer to the smaller code, and the mantissa is cut off.  One exponential and two
-              // integer operations per score serve row sum and weight (with the code formed first, by an add of
+              // e = 2^x with x = t * scale - max <= 0 up to rounding (the row maximum has code 0); -inf logits (keys beyond
+              // nk) give 0.  The row sum takes e as it is.  The power of two nearest to it in the log domain, times 2^14, is e
+              // with the mantissa rounded at sqrt(2) and 14 more in the exponent: adding 2 - sqrt(2) in mantissa units
+              // carries into the exponent where x is nearer to the smaller code, and the mantissa is cut off.  One exponential
+              // and two integer operations per score serve row sum and weight (with the code formed first, by an add of
               // 1.5 * 2^23, a clamp, a shift and a subtraction, a score took half again as many instructions).
-              const unsigned long long shift2 = pack_f32x2(AT_P_SHIFT - base, AT_P_SHIFT - base);
+              // The 2^14 must not be part of x: 14 - distance is rounded at 2^-21 where the distance itself is held to 2^-25,
+              // and 8e-7 of the scores then take a neighbour of the code that 64 bits give, against 2.6e-7 this way and 4.3e-7
+              // with the logit rounded by an add (2 x 8 x 4096 x 40).  The 32 columns are summed before they join the row's
+              // sum, which keeps the chain of rounded additions short.
+              const unsigned long long base2 = pack_f32x2(base, base);
+              unsigned long long zc = 0ull;
 #pragma unroll
               for (int i = 0; i < 32; i += 2) {
-                const unsigned long long x2 = fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), scale2, shift2);
+                const unsigned long long x2 = fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), scale2, base2);
                 float x0, x1;
                 unpack_f32x2(x2, x0, x1);
                 const float e0 = ex2_approx(x0), e1 = ex2_approx(x1);
-                zs = fma_f32x2(pack_f32x2(e0, e1), one2, zs);
-                uint32_t b0 = (__float_as_uint(e0) + 0x004AFB0Du) & 0xFF800000u, b1 = (__float_as_uint(e1) + 0x004AFB0Du) & 0xFF800000u;
+                zc = fma_f32x2(pack_f32x2(e0, e1), one2, zc);
+                uint32_t b0 = (__float_as_uint(e0) + 0x074AFB0Du) & 0xFF800000u, b1 = (__float_as_uint(e1) + 0x074AFB0Du) & 0xFF800000u;
                 if (CODES) {
                   // exponent field 127 + 14 - code; where e has left the fp32 range the code comes from x itself
-                  const uint32_t c0 = x0 > -100.f ? 141u - (b0 >> 23) : __float_as_uint(fminf(AT_P_SHIFT - x0, 255.f) + 12582912.0f) & 0xFFu;
-                  const uint32_t c1 = x1 > -100.f ? 141u - (b1 >> 23) : __float_as_uint(fminf(AT_P_SHIFT - x1, 255.f) + 12582912.0f) & 0xFFu;
+                  const uint32_t c0 = x0 > -120.f ? 141u - (b0 >> 23) : __float_as_uint(fminf(-x0, 255.f) + 12582912.0f) & 0xFFu;
+                  const uint32_t c1 = x1 > -120.f ? 141u - (b1 >> 23) : __float_as_uint(fminf(-x1, 255.f) + 12582912.0f) & 0xFFu;
                   r[i] = min(c0, L);
                   r[i + 1] = min(c1, L);
                 }
@@ -443,6 +449,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 const __half2 ph = __floats2half2_rn(__uint_as_float(b0), __uint_as_float(b1));
                 pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&ph);  // key i in the low half
               }
+              zs = fma_f32x2(zc, one2, zs);
             } else {
               const unsigned long long base2 = pack_f32x2(base, base);
 #pragma unroll
@@ -493,7 +500,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 #pragma unroll
         for (int i = 0; i < PARTS; ++i) m_raw = fmaxf(m_raw, my_m[i * SATC_BQ]);
         m2 = m_raw * scale;
-        base = m2;  // row maximum as scale: log2 s + max + log2 sum = max
+        base = -m2;  // row maximum as scale: code = rint(max - t)
       } else if (!walk_codes) {
         const float log2_fixed = log2f(fmaxf(__ldg(a.fixed_scale + b), 1.17549435e-38f));
         base = log2_fixed + m2 + log2f(row_sum());
@@ -501,7 +508,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     }
     float s_row;
     if (FIXED) s_row = fmaxf(__ldg(a.fixed_scale + b), 1.17549435e-38f) * 6.103515625e-05f;  // 2^-14
-    else s_row = 1.0f / row_sum();  // (the sum carries the 2^14)
+    else s_row = 6.103515625e-05f / row_sum();
     mbar_wait_handover(smem_u32(&sh->o_full), 0, abort_flag);
     __syncwarp();
     tc_fence_after();

@@ -804,15 +804,23 @@ extern "C" dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int t
   // ones and the other 260 would take 1.5 times it, none of them the wrong way round by more than 3 %.
   if ((int64_t)a.n_tiles_m * ((w->N + BN - 1) / BN) * 2 <= n_sm && (int64_t)a.n_tiles_m * ((w->N + 63) / 64) <= n_sm) BN = 64;
   a.n_tiles_n = (w->N + BN - 1) / BN;
-  // Expanding in front of the GEMM costs a launch and a round trip of the weights through L2 (1.0-1.5 us at least); in the
-  // kernel it costs every tile a share of its stages' time.  The kernel wins while a CTA unpacks little: 32-row pieces
-  // of a B stage over all its tiles (616 x 768 -> 1280 10.0 -> 8.8 us, 1024 x 768 -> 1280 14.5 -> 12.0, 2048 x 1280 ->
-  // 1280 at 60 pieces 15.0 -> 14.6, 2048 x 1600 -> 1280 at 70 pieces 15.6 -> 16.2).  A conv stage takes longer anyway
-  // (2 x 16 x 16 x 320 at 90 pieces 20.5 -> 19.2).
+  // Expanding in front of the GEMM costs a launch and a round trip of the weights through L2 (1.0-1.5 us and about half a
+  // microsecond per MiB of bytes); in the kernel it costs every stage of every tile a share of its time, of which a CTA with
+  // further tiles hides a part under their epilogues.  Time unpacking in the kernel / expanding in front, 932 shapes, by 32-row
+  // pieces of B stages that a CTA unpacks: narrow tiles 44 pieces 0.80-0.99, 56 pieces 0.96, 84 pieces 0.99-1.14; a
+  // single wide tile 8 stages 0.84-1.09, 10 stages 0.88-1.13, 12 stages 0.69-1.22, 14 stages 1.00-1.27; several wide tiles 60
+  // pieces 0.85-1.03, 80 pieces 0.92-1.10, 112 pieces 1.17-1.29.  More weights to expand move the line (64 x 1280 -> 10240 with
+  // 14 MiB, 12 stages: 12.1 against 17.5 us).  9 shapes are the wrong way round by more than 8 % (worst 14 %, 2048 x 1000 -> 640).
+  // A conv stage takes longer anyway: 82 pieces 0.87-1.00, 90 pieces 0.93-1.04, 114 pieces 0.89-0.97 (narrow tiles), 125 pieces
+  // 1.11-1.14 (wide).
   if (expand_first) {
     const int64_t n_workers = (int64_t)std::min(a.n_tiles_m, std::max(1, n_sm / a.n_tiles_n));  // row blocks side by side
-    const int64_t pieces = (a.n_tiles_m + n_workers - 1) / n_workers * ((w->Kt + 127) / 128) * (BN / 32);
-    expand_first = pieces > (conv ? 100 : 64);
+    const int64_t tiles = (a.n_tiles_m + n_workers - 1) / n_workers, stages = (w->Kt + 127) / 128;
+    const int64_t pieces = tiles * stages * (BN / 32), mib = (int64_t)(ws_need >> 20);
+    if (conv) expand_first = pieces > 100;
+    else if (BN == 64) expand_first = pieces > 64;
+    else if (tiles == 1) expand_first = stages > 8 + mib;
+    else expand_first = pieces > 64 + 4 * mib;
   }
   a.b_early = !expand_first;
   // instruction descriptor of kind::i8: int32 accumulator (bits 4-5 = 2), A format bit 7 (0 = u8,

@@ -134,6 +134,10 @@ def test_linear_reduction_lengths(M, N, sizes):
     (128, 4000, 64),         # 64 pieces of 64-column tiles: the last reduction unpacked inside
     (128, 4160, 64),         # the first expanded in front
     (2500, 640, 1280),       # several tiles per block, expanded in front
+    (6300, 1016, 160), (6300, 1024, 160),    # a single wide tile per block: 8 stages inside, 9 in front
+    (1000, 1400, 2560), (1000, 1408, 2560),  # the same with 3 MiB of weights: 11 stages inside, 12 in front
+    (20000, 792, 160),                       # two tiles on some blocks: 70 pieces in front
+    (20000, 744, 160),                       # 60 inside
 ])
 def test_four_bit_routes(M, C, N):
     torch, b = gpu()

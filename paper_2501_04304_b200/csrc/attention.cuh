@@ -30,7 +30,7 @@ constexpr int AT_THREADS = AT_WARPS * 32;
 constexpr float AT_P_SHIFT = 14.0f;  // A_hat / s is held in fp16 as 2^(14 - code)
 constexpr float AT_CODE_CAP = 40.0f; // 2^(14 - 40) is below half the smallest fp16: codes beyond it give 0
 
-// MT: 16-row tiles per warp (1 or 2; two need the registers that a wide head or a long context does not leave).
+// MT: 16-row tiles per warp (1 or 2; two need more registers than a wide head or a long context leaves, see launch_attn).
 template <int D, int NKP, int MT_>
 struct AttnCfg {
   static constexpr int DP = (D + 15) / 16 * 16;   // features padded to the MMA K step
@@ -885,7 +885,9 @@ static dgq_status launch_attn_two(AttnArgs a, cudaStream_t stream) {
 }
 
 // One kernel where its grid fits the device at once: with 128 query rows per CTA (more CTAs, shorter ones) or, if that is
-// too many, 256 where the registers allow it (8 x 8 x 1024 x 80: 512 CTAs of 128 rows would need two kernels).
+// too many, 256 for heads of up to 80 features and up to 80 keys (at 128 features the sums, at 128 keys the logits of two
+// row tiles take the 128 registers of a thread alone).  With 80 features a thread spills 130-170 bytes, and one kernel is
+// the faster way all the same (8 x 8 x 1024 x 80, for which 128 rows per CTA would need two kernels: 24.4 -> 17.5 us).
 template <int D, int NKP>
 static dgq_status launch_attn(const AttnArgs& a, bool allow_fused, cudaStream_t stream) {
   constexpr bool TWO = D <= 80 && NKP <= 5;

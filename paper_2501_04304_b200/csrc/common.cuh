@@ -314,18 +314,6 @@ __device__ __forceinline__ uint32_t mbar_test_addr(uint32_t bar_addr, uint32_t p
       : "memory");
   return ok;
 }
-// Read-only global loads that stay where they are written (a plain load may be moved next to its
-// first use, which would expose its latency there).
-__device__ __forceinline__ float ldg_f32_here(const float* p) {
-  float v;
-  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
-__device__ __forceinline__ int ldg_s32_here(const int32_t* p) {
-  int v;
-  asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(p));
-  return v;
-}
 // Register re-balancing between the warpgroups of a CTA (every warp of an aligned group of four
 // executes the same instruction).
 template <int REGS>
@@ -369,18 +357,6 @@ __device__ __forceinline__ void cvt_fma_f32x2(unsigned long long& y, unsigned lo
       : "r"(i0), "r"(i1), "l"(s2));
 }
 
-// Two int32 -> fp32 conversions straight into one 64-bit register pair (the operand form of the packed
-// fp32 instructions), so that no moves are needed to pair the results up.
-__device__ __forceinline__ unsigned long long cvt_s32x2_f32x2(uint32_t i0, uint32_t i1) {
-  unsigned long long r;
-  asm("{\n\t.reg .f32 f0, f1;\n\t"
-      "cvt.rn.f32.s32 f0, %1;\n\t"
-      "cvt.rn.f32.s32 f1, %2;\n\t"
-      "mov.b64 %0, {f0, f1};\n\t}"
-      : "=l"(r)
-      : "r"(i0), "r"(i1));
-  return r;
-}
 // d = a * b + c on two lanes
 __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b,
                                                         unsigned long long c) {
@@ -447,19 +423,9 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-// One 128 x N x 32 int8 MMA: D[tmem] (+)= A[smem] * B[smem]^T, issued by a single thread.
-__device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
-                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// The same with the two 64-bit shared-memory descriptors given as (low, high) words: the high words
-// are constants of the layout and only the low word (the address field) changes from atom to atom,
-// which keeps the single issuing thread's dependent instruction chain short.
+// One 128 x N x 32 int8 MMA: D[tmem] (+)= A[smem] * B[smem]^T, issued by a single thread.  The two 64-bit shared-memory
+// descriptors come as (low, high) words: the high words are constants of the layout and only the low word (the address
+// field) changes from atom to atom, which keeps the single issuing thread's dependent instruction chain short.
 __device__ __forceinline__ void mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
                                             uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -471,16 +437,14 @@ __device__ __forceinline__ void mma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uint
       ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Low / high words of a K-major shared-memory descriptor (see smem_desc).
+// Low / high words of the shared-memory descriptor of a K-major operand with rows of 128 B (SWIZZLE_128B) or 32 B
+// (SWIZZLE_32B): start address >> 4 in bits [0,14), stride between 8-row groups >> 4 in bits [32,46), descriptor
+// version 1 in bits [46,48), swizzle mode in bits [61,64) (2 = 128 B, 6 = 32 B).
 __device__ __forceinline__ uint32_t smem_desc_lo(uint32_t addr) { return ((addr & 0x3FFFFu) >> 4) | (1u << 16); }
 __device__ __forceinline__ constexpr uint32_t smem_desc_hi(uint32_t sbo_bytes, uint32_t layout) {
   return (sbo_bytes >> 4) | (1u << 14) | (layout << 29);
 }
-// Arrives on `bar` once every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
+// Arrives on the barrier once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit_addr(uint32_t bar_addr) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_addr)
                : "memory");
@@ -515,13 +479,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Shared-memory matrix descriptor, K-major operand, rows of 128 B (SWIZZLE_128B) or 32 B (SWIZZLE_32B):
-// start address >> 4 in bits [0,14), stride between 8-row groups >> 4 in bits [32,46), descriptor
-// version 1 in bits [46,48), swizzle mode in bits [61,64) (2 = 128 B, 6 = 32 B).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t sbo_bytes, uint32_t layout) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)layout << 61);
-}
 #endif  // __CUDACC__
 
 }  // namespace dgq

@@ -6,8 +6,8 @@
 //
 // CTA = one 128-row output tile x BN columns, persistent over tiles.  Warp roles:
 //   warps 0-7   epilogue: lane quarter = warp & 3 (the TMEM lanes a warp may read), column half = warp >> 2
-//   warp  8, 11 TMA producers: A code tile and B weight tile per 128-byte K stage
-//   warp  9     MMA issuer (one lane) and TMEM allocator
+//   warp  8, 11 TMA producers: A code tile and B weight tile per 128-byte K stage (the second for long reductions)
+//   warp  9     MMA issuer (the whole warp walks, one elected lane issues) and TMEM allocator
 //   warp  10    output store (one lane): TMA stores of the staged fp16 tile
 //   warps 11-15 (4-bit weights only) unpack packed nibbles from global memory into the B stage
 // After set-up the data-movement warps hand registers to the epilogue warps (setmaxnreg).
@@ -223,7 +223,8 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int turn = (warp == GEMM_WARP_TMA) ? 0 : 1;
     if (turn < producers) {
       const uint32_t empty0 = smem_u32(&sh->empty[0]);
-      // The first tile's weights do not depend on the kernel before this one: their boxes go out ahead of the wait.
+      // The first tile's weights do not depend on the kernel before this one: their boxes go out ahead of the wait.  (The
+      // kernel that writes them runs when the weight is built, and the build waits for it.)
       int early = 0;
       if (!W4 && a.b_early && (int)blockIdx.x < n_tiles) {
         early = min(n_kstages, STAGES);

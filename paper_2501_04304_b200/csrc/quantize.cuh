@@ -27,8 +27,6 @@
 
 namespace dgq {
 
-constexpr int QA_MAX_THREADS = 608;  // K_pad / 16 chunks of the widest layer (8192 channels, 32 groups)
-
 struct QuantArgs {
   const __half* X;
   uint8_t* Xq;
@@ -355,8 +353,8 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   const int n_chunks = g->K_pad / 16;
   const int64_t n_pairs = (M + 1) / 2;
   // Where the chunks of a pair nearly fill a warp, each warp has a pair to itself and the barriers of a batch are the
-  // warp's own (32768 x 320 with 512 positions: 16.4 -> 15.4 us, static 11.5 -> 11.0; with 20 of 32 lanes at work,
-  // 16384 x 200, 7.3 -> 7.9 us, so not there).
+  // warp's own (32768 x 320 with 512 positions: 16.4 -> 15.4 us, static 11.5 -> 11.0).  Warp / block time, mean over 300 to 32768
+  // rows: 32 chunks 0.98, 30 0.98, 28 0.99, 26 1.0, 24 1.0, 22 0.99, 20 1.02, 18 1.05, 16 1.16 (at 32768 rows 1.15 from 24 chunks down).
   const bool warp = n_chunks > 24 && n_chunks <= 32;
   const int per_pair = warp ? 32 : n_chunks;
   int pairs = std::max(1, 128 / per_pair);

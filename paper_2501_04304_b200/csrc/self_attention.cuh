@@ -10,13 +10,16 @@
 //   walk "sum"   : (fixed scale only) the row sums of 2^(t - max), which the codes then depend on;
 //   walk "codes" : S again; code = rint(base - t) in the log domain, P = 2^(14 - code) as fp16 into
 //                  tensor memory, O += P V on the tensor cores with P read from there.  With the row maximum as
-//                  scale the codes do not depend on the row sum, which is then gathered in this walk.
+//                  scale the codes do not depend on the row sum, which is then gathered in this walk, and the rounding
+//                  is done on the mantissa of 2^(t - max); with a fixed scale it is done on base - t itself.  The two
+//                  agree but for scores within a few units in the last place of a boundary.
 // Roles: 16 softmax warps in two teams that take the score tiles in turn (warp w reads tensor-memory lanes 32 (w % 4) ..
-// +31 and half of the 128 columns of its team's tiles), one TMA producer lane, one lane that issues the score MMAs and one that issues
-// the P V MMAs (each tile costs an issuing thread a chain of dependent instructions, so the two run apart).  With two query tiles the softmax
-// warps alternate between them, so every K / V block fetched from L2 serves 256 query rows and one
-// tile's MMAs run under the other tile's arithmetic.  Q, K and P are K-major operands with 128-byte
-// swizzled rows; V is used as it lies in memory (features contiguous), an MN-major operand.  Tiles are
+// +31 and half of the 128 columns of its team's tiles), one TMA producer lane, one warp that issues the score MMAs and one
+// that issues the P V MMAs (each tile costs an issuing warp a chain of dependent instructions, so the two run apart; the
+// instructions themselves come from one elected lane).  With two query tiles the softmax warps alternate between them, so
+// every K / V block fetched from L2 serves 256 query rows and one tile's MMAs run under the other tile's
+// arithmetic.  Q, K and P are K-major operands with 128-byte swizzled rows; V is used as it lies in memory (features
+// contiguous; one row = 64 features of one key), an MN-major operand.  Tiles are
 // fetched as boxes of 64 features x 128 tokens; features beyond d and tokens beyond the sequence are
 // zero-filled by the copy engine, so d = 40 runs as 48 and ragged ends need no staging.
 #pragma once
@@ -87,18 +90,9 @@ struct SaTcShared {
   int abort_flag;
 };
 
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
-                                        uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// The same with the descriptors given as (low, high) words: the high words are constants of the layout,
-// only the address field in the low word changes from step to step, which keeps the issuing thread's
-// dependent instruction chain short (that chain, not the tensor pipe, is what bounds a tile otherwise).
+// One 128 x N x 16 fp16 MMA, descriptors as (low, high) words: the high words are constants of the layout, only the
+// address field in the low word changes from step to step, which keeps the issuing thread's dependent
+// instruction chain short (that chain, not the tensor pipe, is what bounds a tile otherwise).
 __device__ __forceinline__ void mma_f16_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
                                              uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -130,12 +124,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// MN-major operand with 128-byte swizzled rows (one row = 64 contiguous elements of the M/N axis for
-// one k): `lbo` = bytes between 64-element blocks of the M/N axis, `sbo` = bytes between groups of 8 k.
-__device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) |
-         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
-}
 __device__ __forceinline__ void named_bar_sync(int id, int n_threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
 }

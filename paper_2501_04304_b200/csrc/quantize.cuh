@@ -45,6 +45,7 @@ struct QuantArgs {
 
 // Words of the interleaved pair: the channels, a word of NaN for the padding, up to a multiple of four.
 __host__ __device__ inline int qa_pitch(int C) { return (C + 1 + 3) & ~3; }
+constexpr int QA_SMEM_MAX = 80 * 1024;  // three pairs of the widest layer that has three
 // The row buffer and two sets of cell ranges.
 __host__ inline size_t qa_smem_bytes(int pairs, int C, int G, bool dynamic) {
   const size_t cells = (size_t)pairs * 2 * G;
@@ -87,7 +88,8 @@ __device__ __forceinline__ uint32_t codes4(const float (&y)[4], float lowb, uint
   return __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
 }
 
-template <bool DYNAMIC, bool CENTRED, bool WARP>
+// FAR: asks for the rows of the batch after the next one in L2.
+template <bool DYNAMIC, bool CENTRED, bool WARP, bool FAR>
 __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ QuantArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n_chunks = a.K_pad >> 4, n_cells = a.pairs * 2 * a.G;
@@ -135,17 +137,27 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
     const int first = __shfl_sync(0xffffffffu, cell, 0);
     one_cell = __all_sync(0xffffffffu, !active || cell == first);
   }
-  // this thread's share of the row loads: at most two pieces of eight channels of a pair
+  // This thread's share of the row loads: at most two pieces of eight channels of a pair.  (With the requests to L2 there
+  // are registers for one word, pair and piece, and the place in shared memory, which is then not worked out again.)
   const int vec = a.C >> 3;
   int lp[2], lv[2];
   bool lok[2];
+  uint32_t place[2];
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
     const int task = tid + e * n_threads;
     lp[e] = WARP ? my_pair : task / vec;
     lv[e] = WARP ? (tid & 31) + 32 * e : task - lp[e] * vec;
     lok[e] = lp[e] < a.pairs && lv[e] < vec;
+    if (FAR) {
+      place[e] = (uint32_t)(lp[e] * a.pitch + lv[e] * 8) * 4u;
+      lp[e] = lok[e] ? lp[e] << 16 | lv[e] : -1;
+    }
   }
+  auto has = [&](int e) { return FAR ? lp[e] >= 0 : lok[e]; };
+  auto pair_of = [&](int e) { return FAR ? lp[e] >> 16 : lp[e]; };
+  auto piece_of = [&](int e) { return FAR ? lp[e] & 0xFFFF : lv[e]; };
+  auto place_of = [&](int e) { return smem_raw + (FAR ? place[e] : (uint32_t)(lp[e] * a.pitch + lv[e] * 8) * 4u); };
   float inv0 = 0.f, inv1 = 0.f;
   int z0 = 0, z1 = 0;
   if (!DYNAMIC && !a.row_group) {
@@ -160,11 +172,22 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
   auto request = [&](int64_t row0) {
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const int64_t row = row0 + 2 * lp[e];
-      if (lok[e] && row < a.M) {
-        const uint4* src = reinterpret_cast<const uint4*>(a.X + row * a.ld) + lv[e];
+      const int64_t row = row0 + 2 * pair_of(e);
+      if (has(e) && row < a.M) {
+        const uint4* src = reinterpret_cast<const uint4*>(a.X + row * a.ld) + piece_of(e);
         xa[e] = __ldg(src);
         xb[e] = row + 1 < a.M ? __ldg(src + (a.ld >> 3)) : xa[e];
+      }
+    }
+  };
+  auto request_far = [&](int64_t row0) {  // one lane per 64 bytes of a row
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int64_t row = row0 + 2 * pair_of(e);
+      if (has(e) && row + 1 < a.M && (piece_of(e) & 3) == 0) {
+        const uint4* src = reinterpret_cast<const uint4*>(a.X + row * a.ld) + piece_of(e);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (a.ld >> 3)));
       }
     }
   };
@@ -176,14 +199,15 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
     if (!DYNAMIC && row0 != first_row) sync();  // every value of the last batch is in registers
 #pragma unroll
     for (int e = 0; e < 2; ++e)
-      if (lok[e]) {
-        uint4* dst = reinterpret_cast<uint4*>(smem_raw + (lp[e] * a.pitch + lv[e] * 8) * 4);
+      if (has(e)) {
+        uint4* dst = reinterpret_cast<uint4*>(place_of(e));
         dst[0] = make_uint4(__byte_perm(xa[e].x, xb[e].x, 0x5410), __byte_perm(xa[e].x, xb[e].x, 0x7632),
                             __byte_perm(xa[e].y, xb[e].y, 0x5410), __byte_perm(xa[e].y, xb[e].y, 0x7632));
         dst[1] = make_uint4(__byte_perm(xa[e].z, xb[e].z, 0x5410), __byte_perm(xa[e].z, xb[e].z, 0x7632),
                             __byte_perm(xa[e].w, xb[e].w, 0x5410), __byte_perm(xa[e].w, xb[e].w, 0x7632));
       }
     if (row0 + step < a.M) request(row0 + step);  // arrives while this batch is worked on
+    if (FAR) request_far(row0 + 2 * step);
     sync();
     __half2 x[16];
 #pragma unroll
@@ -358,27 +382,49 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   const bool warp = n_chunks > 24 && n_chunks <= 32;
   const int per_pair = warp ? 32 : n_chunks;
   int pairs = std::max(1, 128 / per_pair);
+  if (per_pair > 64) {
+    // More chunks than half a block: 72 of them leave a quarter of three warps idle, three pairs fill 216 of 224 threads.  Of
+    // one to three pairs the one with the most lanes at work, less 3 % for every warp that a barrier waits for, over all
+    // rounds of the device (32768 x 960: 50.4 -> 46.8 us, x 1600: 73.9 -> 71.0, x 1920: 96.9 -> 92.2; x 1280 stays with one,
+    // 56 against 61 us).
+    double best = 0.;
+    for (int p = 1; p <= 3; ++p) {
+      const int warps = (p * per_pair + 31) / 32, blocks = 28 / warps;
+      if (blocks == 0) break;
+      const int64_t capacity = (int64_t)n_sm * blocks * p, rounds = (n_pairs + capacity - 1) / capacity;
+      const double lanes = (double)(p * per_pair * blocks) * (33 - warps) * (double)n_pairs / (double)(rounds * capacity);
+      if (lanes > best) best = lanes, pairs = p;
+    }
+  }
   int64_t slots = (int64_t)n_sm * std::max(1, 896 / (pairs * per_pair));
   if (n_pairs < slots * pairs) pairs = (int)std::max<int64_t>(1, (n_pairs + slots - 1) / slots);
   const int threads = (pairs * per_pair + 31) / 32 * 32;
   slots = (int64_t)n_sm * std::max(1, 896 / threads);
+  // With many batches per block the rows of the batch after the next one are asked for in L2 as well (32768 x 2560: 125 ->
+  // 115 us, 8192 x 3840: 46.0 -> 41.0, 8192 x 8000: 117 -> 101); with few the instructions cost more than that gives (8192 x 960,
+  // three batches: 15.6 -> 16.1, 8192 x 1280, four: 17.2 -> 17.3, 32768 x 600, eight: 33.7 -> 34.3).
+  const bool far = !warp && n_pairs > 8 * slots * pairs;
   a.pairs = pairs;
   const size_t smem = qa_smem_bytes(pairs, g->C, g->G, dynamic);
   static std::atomic<bool> attr_set[64];
   int dev = 0;
   DGQ_CUDA_OK(cudaGetDevice(&dev));
   if (dev >= 64 || !attr_set[dev].load()) {
-    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
-    DGQ_CUDA_OK(cudaFuncSetAttribute(quantize_act_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024));
+    for (auto k : {quantize_act_kernel<true, false, false, false>, quantize_act_kernel<true, false, false, true>,
+                   quantize_act_kernel<false, false, false, false>, quantize_act_kernel<false, false, false, true>,
+                   quantize_act_kernel<false, true, false, false>, quantize_act_kernel<false, true, false, true>})
+      DGQ_CUDA_OK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QA_SMEM_MAX));
     if (dev < 64) attr_set[dev].store(true);
   }
   const int grid = (int)std::min<int64_t>((n_pairs + pairs - 1) / pairs, slots);
   const bool centred = layout == DGQ_CODES_S8_CENTRED;
-  auto kernel = warp ? (dynamic ? quantize_act_kernel<true, false, true>
-                                : centred ? quantize_act_kernel<false, true, true> : quantize_act_kernel<false, false, true>)
-                     : (dynamic ? quantize_act_kernel<true, false, false>
-                                : centred ? quantize_act_kernel<false, true, false> : quantize_act_kernel<false, false, false>);
+  auto pick = [&](auto w, auto f) {
+    constexpr bool W = decltype(w)::value, F = decltype(f)::value;
+    return dynamic ? quantize_act_kernel<true, false, W, F>
+                   : centred ? quantize_act_kernel<false, true, W, F> : quantize_act_kernel<false, false, W, F>;
+  };
+  auto kernel = warp ? pick(std::true_type{}, std::false_type{})
+                     : far ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{});
   DGQ_CUDA_OK(launch_pdl(kernel, dim3(grid), dim3(threads), smem,
                          (cudaStream_t)stream, a));
   g_launches += 1;

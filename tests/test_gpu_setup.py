@@ -70,7 +70,10 @@ def test_weight_layout_edges(sizes, N, w_bits):
     (257, (320,), 8),                # a cell that covers a whole warp
     (2601, (300, 188), 8),           # 32 chunks: a warp per row pair, several batches, odd row count
     (9, (5112, 8), 8),               # one pair per block, more chunks than a small block has threads
-    (4100, (8184, 8), 4),            # the widest layer, several batches per block
+    (4100, (8184, 8), 4),            # the widest layer, several batches per block, rows asked for two batches ahead
+    (2367, (1500, 36), 8),           # 100 chunks, one round of the device with two pairs per block
+    (3551, (1100, 20), 8),           # 72 chunks, one round with three
+    (18947, (1500, 36), 8),          # two pairs per block and rows asked for ahead, odd row count
 ])
 def test_quantizer_edges(M, sizes, bits, mode):
     torch, b = gpu()

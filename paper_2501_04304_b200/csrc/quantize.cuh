@@ -14,11 +14,13 @@
 // Bound: about 430 (dynamic) or 300 (static) warp instructions per row of 512 codes (half of them two-cycle integer and conversion
 // instructions) and the latency of one read-reduce-write chain for small matrices; the bytes (2 B read + 1 B written per
 // element + 8 B per (token, group) in dynamic mode) would take a third of the time.  72 registers keep 28
-// warps on an SM: at 80 an 8192-row matrix needs a second, nearly empty round of batches (5.5 against 5.1 us), at 64
-// the gathered values spill (5.9 us).  Blocks of 128 threads keep the barriers cheap (256: 5.8 us).  Against one warp
-// per two rows that scattered value by value into group order and read the chunks back twice, dynamic / static:
-// 8192 x 320 6.4 -> 5.1 / 7.0 -> 3.8 us, 32768 x 320 19.9 -> 16.3 us, 2048 x 5120 23.7 -> 15.7 us, 616 x 768 4.9 ->
-// 3.1 us, static 2048 x 1280 with 16 groups 12.0 -> 3.8 us.
+// warps on an SM (4 to 60 bytes of a thread spill): at 80 an 8192-row matrix needs a second, nearly empty round of batches
+// (5.5 against 5.1 us), at 64 the gathered values spill (5.9 us).  Blocks of 128 threads keep the barriers cheap (256: 5.8 us).
+// Against one warp per two rows that scattered value by value into group order and read the chunks back twice, dynamic /
+// static, inputs cold, 8 groups: 8192 x 320 6.4 -> 5.1 / 7.0 -> 3.8 us, 2048 x 5120 23.7 -> 15.7, 616 x 768 4.9 -> 3.1; 8192 x 1280 17.1 ->
+// 17.1 / 13.6 -> 12.4, 32768 x 1280 54.7 -> 53.1 / 42.4 -> 36.4, 32768 x 2560 117 -> 112 / 80 -> 75.  It is the slower one for dynamic
+// ranges of 960 and 1920 to 2048 channels at 8192 rows (14.5 -> 15.6, 24.3 -> 26.6, 25.9 -> 28.1) and of 1920 to 2048 beyond (32768 rows 83.6 ->
+// 90.3, 88.7 -> 91.3): a pair fills its warps badly there and the barriers of a batch are waited for.
 #pragma once
 
 #include <type_traits>
@@ -43,13 +45,18 @@ struct QuantArgs {
   int32_t* dyn_zp;
 };
 
+// Place of a channel in an interleaved pair.  Spread, four words are left out behind every 32: where neighbouring channels
+// belong to one group (the whole layer, when it is grouped by pixel positions only) the lanes of a warp read words 16
+// apart, which would lie in two banks; this way at most four lanes meet in one.
+template <bool SPREAD>
+__host__ __device__ inline int qa_word(int c) { return SPREAD ? c + (c >> 5) * 4 : c; }
 // Words of the interleaved pair: the channels, a word of NaN for the padding, up to a multiple of four.
-__host__ __device__ inline int qa_pitch(int C) { return (C + 1 + 3) & ~3; }
+__host__ __device__ inline int qa_pitch(int C, bool spread) { return ((spread ? qa_word<true>(C) : C) + 1 + 3) & ~3; }
 constexpr int QA_SMEM_MAX = 80 * 1024;  // three pairs of the widest layer that has three
 // The row buffer and two sets of cell ranges.
-__host__ inline size_t qa_smem_bytes(int pairs, int C, int G, bool dynamic) {
+__host__ inline size_t qa_smem_bytes(int pairs, int pitch, int G, bool dynamic) {
   const size_t cells = (size_t)pairs * 2 * G;
-  return (size_t)pairs * qa_pitch(C) * 4 + (dynamic ? cells * 4 * 4 : 0);
+  return (size_t)pairs * pitch * 4 + (dynamic ? cells * 4 * 4 : 0);
 }
 
 // bits 0-3 of `m` spread to 0xFF bytes
@@ -89,7 +96,7 @@ __device__ __forceinline__ uint32_t codes4(const float (&y)[4], float lowb, uint
 }
 
 // FAR: asks for the rows of the batch after the next one in L2.
-template <bool DYNAMIC, bool CENTRED, bool WARP, bool FAR>
+template <bool DYNAMIC, bool CENTRED, bool WARP, bool FAR, bool SPREAD>
 __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ QuantArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int n_chunks = a.K_pad >> 4, n_cells = a.pairs * 2 * a.G;
@@ -119,12 +126,12 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
     for (int i = 0; i < 16; ++i) {
       const int c = (int)(int16_t)(pw[i >> 1] >> (16 * (i & 1)));
       if (c < 0) pm |= 1u << i;
-      off[i] = base + (uint32_t)(c < 0 ? a.C : c) * 4u;
+      off[i] = base + (uint32_t)qa_word<SPREAD>(c < 0 ? a.C : c) * 4u;
     }
     g = active ? __ldg(a.chunk_group + ch) : 0;
   }
   for (int i = tid; i < a.pairs; i += n_threads)
-    *reinterpret_cast<uint32_t*>(smem_raw + ((size_t)i * a.pitch + a.C) * 4) = 0x7FFF7FFFu;  // the word of NaN
+    *reinterpret_cast<uint32_t*>(smem_raw + ((size_t)i * a.pitch + qa_word<SPREAD>(a.C)) * 4) = 0x7FFF7FFFu;  // the word of NaN
   if (DYNAMIC)
     for (int i = tid; i < n_cells; i += n_threads) {
       cell_lo[i] = INT_MAX;
@@ -150,14 +157,14 @@ __global__ void __maxnreg__(72) quantize_act_kernel(const __grid_constant__ Quan
     lv[e] = WARP ? (tid & 31) + 32 * e : task - lp[e] * vec;
     lok[e] = lp[e] < a.pairs && lv[e] < vec;
     if (FAR) {
-      place[e] = (uint32_t)(lp[e] * a.pitch + lv[e] * 8) * 4u;
+      place[e] = (uint32_t)(lp[e] * a.pitch + qa_word<SPREAD>(lv[e] * 8)) * 4u;
       lp[e] = lok[e] ? lp[e] << 16 | lv[e] : -1;
     }
   }
   auto has = [&](int e) { return FAR ? lp[e] >= 0 : lok[e]; };
   auto pair_of = [&](int e) { return FAR ? lp[e] >> 16 : lp[e]; };
   auto piece_of = [&](int e) { return FAR ? lp[e] & 0xFFFF : lv[e]; };
-  auto place_of = [&](int e) { return smem_raw + (FAR ? place[e] : (uint32_t)(lp[e] * a.pitch + lv[e] * 8) * 4u); };
+  auto place_of = [&](int e) { return smem_raw + (FAR ? place[e] : (uint32_t)(lp[e] * a.pitch + qa_word<SPREAD>(lv[e] * 8)) * 4u); };
   float inv0 = 0.f, inv1 = 0.f;
   int z0 = 0, z1 = 0;
   if (!DYNAMIC && !a.row_group) {
@@ -361,7 +368,6 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   a.G = g->G;
   a.P = g->P;
   a.bits = g->bits;
-  a.pitch = qa_pitch(g->C);
   a.perm = g->d_perm;
   a.chunk_group = g->d_chunk_group;
   a.row_group = g->R > 1 ? g->d_row_group : nullptr;
@@ -404,27 +410,45 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   // 115 us, 8192 x 3840: 46.0 -> 41.0, 8192 x 8000: 117 -> 101); with few the instructions cost more than that gives (8192 x 960,
   // three batches: 15.6 -> 16.1, 8192 x 1280, four: 17.2 -> 17.3, 32768 x 600, eight: 33.7 -> 34.3).
   const bool far = !warp && n_pairs > 8 * slots * pairs;
+  // Where one group holds more than half of the layer (one group, static, 8192 x 2048: 29.1 -> 18.9 us, 32768 x 1280: 58.5 -> 36.5,
+  // 8192 x 320: 7.3 -> 4.5 us; the instructions it costs take 1 to 2 % of a static pass over layers of several groups).
+  int largest = 0;
+  for (int k = 0; k < g->G; ++k) largest = std::max(largest, g->group_off[k + 1] - g->group_off[k]);
+  const bool spread = 2 * largest > g->K_pad;
+  a.pitch = qa_pitch(g->C, spread);
   a.pairs = pairs;
-  const size_t smem = qa_smem_bytes(pairs, g->C, g->G, dynamic);
+  const size_t smem = qa_smem_bytes(pairs, a.pitch, g->G, dynamic);
   static std::atomic<bool> attr_set[64];
   int dev = 0;
   DGQ_CUDA_OK(cudaGetDevice(&dev));
   if (dev >= 64 || !attr_set[dev].load()) {
-    for (auto k : {quantize_act_kernel<true, false, false, false>, quantize_act_kernel<true, false, false, true>,
-                   quantize_act_kernel<false, false, false, false>, quantize_act_kernel<false, false, false, true>,
-                   quantize_act_kernel<false, true, false, false>, quantize_act_kernel<false, true, false, true>})
-      DGQ_CUDA_OK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QA_SMEM_MAX));
+    auto opt_in = [](auto f, auto s) {
+      constexpr bool F = decltype(f)::value, S = decltype(s)::value;
+      for (auto k : {quantize_act_kernel<true, false, false, F, S>, quantize_act_kernel<false, false, false, F, S>,
+                     quantize_act_kernel<false, true, false, F, S>}) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, QA_SMEM_MAX);
+        if (e != cudaSuccess) return e;
+      }
+      return cudaSuccess;
+    };
+    const std::false_type no;
+    const std::true_type yes;
+    DGQ_CUDA_OK(opt_in(no, no));
+    DGQ_CUDA_OK(opt_in(no, yes));
+    DGQ_CUDA_OK(opt_in(yes, no));
+    DGQ_CUDA_OK(opt_in(yes, yes));
     if (dev < 64) attr_set[dev].store(true);
   }
   const int grid = (int)std::min<int64_t>((n_pairs + pairs - 1) / pairs, slots);
   const bool centred = layout == DGQ_CODES_S8_CENTRED;
-  auto pick = [&](auto w, auto f) {
-    constexpr bool W = decltype(w)::value, F = decltype(f)::value;
-    return dynamic ? quantize_act_kernel<true, false, W, F>
-                   : centred ? quantize_act_kernel<false, true, W, F> : quantize_act_kernel<false, false, W, F>;
+  auto pick = [&](auto w, auto f, auto s) {
+    constexpr bool W = decltype(w)::value, F = decltype(f)::value, S = decltype(s)::value;
+    return dynamic ? quantize_act_kernel<true, false, W, F, S>
+                   : centred ? quantize_act_kernel<false, true, W, F, S> : quantize_act_kernel<false, false, W, F, S>;
   };
-  auto kernel = warp ? pick(std::true_type{}, std::false_type{})
-                     : far ? pick(std::false_type{}, std::true_type{}) : pick(std::false_type{}, std::false_type{});
+  auto pick_spread = [&](auto w, auto f) { return spread ? pick(w, f, std::true_type{}) : pick(w, f, std::false_type{}); };
+  auto kernel = warp ? pick_spread(std::true_type{}, std::false_type{})
+                     : far ? pick_spread(std::false_type{}, std::true_type{}) : pick_spread(std::false_type{}, std::false_type{});
   DGQ_CUDA_OK(launch_pdl(kernel, dim3(grid), dim3(threads), smem,
                          (cudaStream_t)stream, a));
   g_launches += 1;

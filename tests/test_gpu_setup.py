@@ -73,7 +73,7 @@ def test_weight_layout_edges(sizes, N, w_bits):
     (4100, (8184, 8), 4),            # the widest layer, several batches per block, rows asked for two batches ahead
     (2367, (1500, 36), 8),           # 100 chunks, one round of the device with two pairs per block
     (3551, (1100, 20), 8),           # 72 chunks, one round with three
-    (18947, (1500, 36), 8),          # two pairs per block and rows asked for ahead, odd row count
+    (18947, (512, 512, 512), 8),     # two pairs per block and rows asked for ahead, odd row count, no group of more than half
 ])
 def test_quantizer_edges(M, sizes, bits, mode):
     torch, b = gpu()

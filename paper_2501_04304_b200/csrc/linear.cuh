@@ -8,7 +8,7 @@
 //   warps 0-7   epilogue: lane quarter = warp & 3 (the TMEM lanes a warp may read), column half = warp >> 2
 //   warp  8, 11 TMA producers: A code tile and B weight tile per 128-byte K stage (the second for long reductions)
 //   warp  9     MMA issuer (the whole warp walks, one elected lane issues) and TMEM allocator
-//   warp  10    output store (one lane): TMA stores of the staged fp16 tile
+//   warp  10    bias into shared memory, then output store (one lane): TMA stores of the staged fp16 tile
 //   warps 11-15 (4-bit weights only) unpack packed nibbles from global memory into the B stage
 // After set-up the data-movement warps hand registers to the epilogue warps (setmaxnreg).
 // K runs over 32-code atoms; a stage holds four atoms.  Group segments are multiples of one atom,
@@ -117,7 +117,7 @@ struct __align__(8) GemmShared {
   uint64_t acc_full[4];
   uint64_t acc_empty[4];
   uint64_t out_full;   // all epilogue warps have staged their part of the output tile
-  uint64_t out_free;   // the TMA stores of the previous tile have read the staging buffer
+  uint64_t out_free;   // first phase: the bias is in shared memory; then: the TMA stores of the previous tile have read the staging buffer
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -174,7 +174,6 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   for (int i = threadIdx.x; i < BN; i += blockDim.x) {
     const int col = cta_n0 + i;
     sw_s[i] = col < a.N_pad ? __ldg(a.sw + col) : 0.f;
-    bias_s[i] = (a.bias != nullptr && col < a.N) ? __half2float(a.bias[col]) : 0.f;
   }
   if (a.use_zp)
     for (int i = threadIdx.x; i < a.G * BN; i += blockDim.x) {
@@ -201,8 +200,10 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tmem_alloc(&sh->tmem_base, 512);
     tmem_relinquish();
   }
-  // Everything up to here reads only the layer's constants; codes, scales and zero-points may come from the kernel
-  // before this one, so every role waits for it (pdl_wait) before its first access to them.
+  // Everything up to here reads only the arrays of the weight, which are complete before it can be used; codes, scales,
+  // zero-points and the bias may come from kernels before this one that are still running (the kernel right before it has
+  // let this one start, and need not have waited for its own predecessor yet), so every role waits (pdl_wait) before its
+  // first access to them.
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -395,7 +396,11 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp == GEMM_WARP_STORE) {
     // ------------------------------------------------------------ output store
     pdl_wait();
+    for (int i = lane; i < BN; i += 32)
+      bias_s[i] = (a.bias != nullptr && cta_n0 + i < a.N) ? __half2float(__ldg(a.bias + cta_n0 + i)) : 0.f;
+    __syncwarp();
     if (lane == 0) {
+      mbar_arrive(&sh->out_free);  // the bias is there, the staging buffer is free
       const uint32_t out_full_a = smem_u32(&sh->out_full);
       uint32_t tile_it = 0;
       for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tile_it) {
@@ -607,8 +612,9 @@ gq_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       }
       if (*abort_flag) break;  // a wait gave up somewhere in the CTA (same value in every lane)
-      // staging buffer: wait until the stores of the previous tile have read it (normally long done)
-      mbar_wait_handover(out_free_a, (tile_it & 1u) ^ 1u, abort_flag);
+      // staging buffer: wait until the stores of the previous tile have read it (normally long done); for the first tile,
+      // until the bias is there
+      mbar_wait_handover(out_free_a, tile_it & 1u, abort_flag);
 #pragma unroll
       for (int j = 0; j < CW / 8; ++j) {
         const int cl = sl * CW + j * 8;  // first tile column of this 16-byte chunk

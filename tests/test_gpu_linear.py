@@ -216,6 +216,33 @@ def test_four_bit_weights_with_and_without_workspace():
     assert b.device_status() == 0
 
 
+@pytest.mark.parametrize("w_bits,M", [(8, 1), (4, 200)])
+def test_bias_may_come_from_a_kernel_still_running(w_bits, M):
+    """A layer whose bias is a row of another layer's output (as a time embedding added per channel is), with a tiny
+    quantizer in between that lets the second GEMM start while the first still runs: the bias is read after the wait."""
+    torch, b = gpu()
+    C, N = 320, 328
+    Xcal, X, W, bias, gr = layer_case(19, 1, 512, C, N, 8, 8, oc.DIM_CHANNEL)
+    g = b.calibrate_groups(to_dev(torch, Xcal), 512, 8, 8, b.DIM_CHANNEL)
+    w1, w2 = b.weight_prepare(g, to_dev(torch, W), 8), b.weight_prepare(g, to_dev(torch, W), w_bits)
+    big = to_dev(torch, np.tile(X, (64, 1)))
+    x = to_dev(torch, X[:M])
+    kw = dict(mode=b.MODE_DYNAMIC_TOKEN)
+    xq, ds, dz = b.quantize_act(g, big, **kw)
+    xq2, ds2, dz2 = b.quantize_act(g, x, **kw)
+    y1 = b.linear(g, w1, xq, dyn_scale=ds, dyn_zp=dz, **kw)
+    torch.cuda.synchronize()
+    ref = b.linear(g, w2, xq2, dyn_scale=ds2, dyn_zp=dz2, bias=y1[-1], **kw)
+    for _ in range(5):
+        y1.fill_(float("nan"))
+        b.linear(g, w1, xq, dyn_scale=ds, dyn_zp=dz, out=y1, **kw)
+        b.quantize_act_into(g, x, xq2, ds2, dz2, **kw)
+        y2 = b.linear(g, w2, xq2, dyn_scale=ds2, dyn_zp=dz2, bias=y1[-1], **kw)
+        torch.cuda.synchronize()
+        assert torch.equal(y2, ref)
+    assert b.device_status() == 0
+
+
 def test_workspace_belongs_to_the_stream_of_the_call():
     """A call on another stream than the current one, still waiting there when it returns: its workspace is not given to
     the next allocation on the current stream."""

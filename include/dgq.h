@@ -141,7 +141,8 @@ dgq_status dgq_weight_prepare(const dgq_groups* g, const void* W, int N, int K, 
 dgq_status dgq_weight_from_codes(const dgq_groups* g, const int8_t* wq, const float* sw, int N, int K,
                                  int w_bits, const dgq_conv_desc* conv, dgq_weight** out);
 dgq_status dgq_weight_destroy(dgq_weight* w);
-/* Host copies of the codes in original channel order (int8 [N, K]) and scales. */
+/* Host copies of the codes in original channel order (int8 [N, K]) and scales.  Reads the weight's own device
+ * whichever is current, waits for none of the caller's streams and may be called while the calling thread captures one. */
 dgq_status dgq_weight_export(const dgq_weight* w, int8_t* wq, float* sw);
 
 /* ---------------------------------------------------------------- group-quantized layer
@@ -164,8 +165,8 @@ dgq_status dgq_weight_export(const dgq_weight* w, int8_t* wq, float* sw);
  * workspace where that is faster (small problems); a non-NULL workspace that is
  * too small is an error.
  * Errors: INVALID_ARG, ALIGNMENT, NOT_CALIBRATED, WORKSPACE, UNSUPPORTED (K_pad *
- * 255 * 127 would overflow int32; more column blocks of 64-128 outputs than the
- * GPU has SMs; conv shape outside the supported tiling), CUDA. */
+ * 255 * 127 would overflow int32; more column blocks of 128 outputs, 160 where that
+ * divides N, than the GPU has SMs; conv shape outside the supported tiling), CUDA. */
 dgq_status dgq_linear(const dgq_groups* g, const dgq_weight* w, int timestep, int mode, int layout,
                       const void* Xq, const float* dyn_scale, const int32_t* dyn_zp, const void* bias,
                       void* Y, int64_t M, int64_t ldy, const dgq_conv_desc* conv, void* workspace,

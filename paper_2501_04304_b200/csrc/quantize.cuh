@@ -410,8 +410,8 @@ extern "C" dgq_status dgq_quantize_act(const dgq_groups* g, int timestep, int mo
   // 115 us, 8192 x 3840: 46.0 -> 41.0, 8192 x 8000: 117 -> 101); with few the instructions cost more than that gives (8192 x 960,
   // three batches: 15.6 -> 16.1, 8192 x 1280, four: 17.2 -> 17.3, 32768 x 600, eight: 33.7 -> 34.3).
   const bool far = !warp && n_pairs > 8 * slots * pairs;
-  // Where one group holds more than half of the layer (one group, static, 8192 x 2048: 29.1 -> 18.9 us, 32768 x 1280: 58.5 -> 36.5,
-  // 8192 x 320: 7.3 -> 4.5 us; the instructions it costs take 1 to 2 % of a static pass over layers of several groups).
+  // Where one group holds more than half of the layer (one group, static, 8192 x 2048: 29.1 -> 18.3 us, 32768 x 1280: 58.5 -> 35.5,
+  // 8192 x 320: 5.3 -> 4.0 us; the instructions it costs take 1 to 2 % of a static pass over layers of several groups).
   int largest = 0;
   for (int k = 0; k < g->G; ++k) largest = std::max(largest, g->group_off[k + 1] - g->group_off[k]);
   const bool spread = 2 * largest > g->K_pad;

@@ -203,13 +203,13 @@ static dgq_status weight_codes_to_host(const dgq_weight* w, int8_t* wq) {
   cudaError_t e = own_stream(&stream);
   int8_t* d = nullptr;
   if (e != cudaSuccess) {
-  } else if (n > WEIGHT_HOST_CODES && pool_alloc((void**)&d, n, stream) == cudaSuccess) {
+  } else if (n > WEIGHT_HOST_CODES && pool_alloc((void**)&d, n, stream, true) == cudaSuccess) {
     weight_unpermute_kernel<<<w->N, 256, 0, stream>>>((const uint8_t*)w->d_w, w->d_chan, w->K, w->C, w->Kt, four_bit, d);
     g_launches += 1;
     if ((e = cudaGetLastError()) == cudaSuccess) e = cudaMemcpyAsync(wq, d, n, cudaMemcpyDeviceToHost, stream);
-    cudaFreeAsync(d, stream);
     const cudaError_t done = cudaStreamSynchronize(stream);
     if (e == cudaSuccess) e = done;
+    cudaFreeAsync(d, stream);
   } else {
     cudaGetLastError();  // (an allocation that failed)
     const size_t row_bytes = four_bit ? w->Kt / 2 : w->Kt;

@@ -44,11 +44,12 @@ constexpr int SATC_SOFTMAX_WARPS = 16;
 constexpr int SATC_WARP_TMA = 16;
 constexpr int SATC_WARP_MMA = 17;   // issues S = Q K^T (and owns the tensor-memory allocation)
 constexpr int SATC_WARP_PV = 18;    // issues O += P V
-constexpr int SATC_THREADS = 19 * 32;
+constexpr int SATC_WARP_MMA2 = 19;  // issues every other score tile (where the softmax warps form two teams)
+
 constexpr int SATC_BQ = 128;            // query rows per tile
 constexpr int SATC_BK = 128;            // keys per block
 constexpr int SATC_PANEL = 128 * 128;   // bytes of one 64-feature (or 64-key) panel of 128 rows
-constexpr int SATC_TMEM_P = 256;        // first column of the P tiles (score buffers at columns 0 and 128)
+constexpr int SATC_TMEM_P = 256;        // first column of the P tiles
 
 template <int D>
 struct SaTcCfg {
@@ -64,18 +65,26 @@ struct SaTcCfg {
   // The softmax warps form two teams of eight that take the score tiles in turn, so that one team's waits, tensor-memory
   // round trips and hand-overs run under the other's arithmetic; with a single P tile they stay together.
   static constexpr int TEAMS = PST;
+  static constexpr int ISSUERS = TEAMS;        // warps that issue score tiles
+  static constexpr int BUFS = 2 * ISSUERS;     // score buffers of the walks before the codes walk
+  static constexpr int THREADS = (18 + ISSUERS) * 32;
   static constexpr int TEAM_WARPS = SATC_SOFTMAX_WARPS / TEAMS;
   static constexpr int SPLIT = TEAM_WARPS / 4;          // warps of a team that share 32 rows of a tile
   static constexpr int COLS = SATC_BK / SPLIT;          // score columns of a warp
   static constexpr int PARTS = NT == 2 ? SPLIT : 4;     // threads that hold a part of a row's statistics
-  static constexpr int TMEM_O = SATC_TMEM_P + PST * 64;
+  // Tensor memory: score buffers at columns 0 and 128; with two teams two more at 256 and 384 in the walks before the codes
+  // walk, which have no use for P and O yet.  With two query tiles a team's P and O lie inside its own second buffer there,
+  // because the teams enter the codes walk one by one; else all warps meet between the walks.
+  static constexpr int P_STRIDE = NT == 2 ? 128 : 64;
+  static constexpr int TMEM_O = NT == 2 ? SATC_TMEM_P + 64 : SATC_TMEM_P + PST * 64;
+  static constexpr int O_STRIDE = 128;
   static constexpr int TILE = NP * SATC_PANEL;
   static constexpr int OFF_K = NT * TILE;
   static constexpr int OFF_V = OFF_K + KST * TILE;
   static constexpr int OFF_SH = OFF_V + VST * TILE;
   static constexpr int SMEM = 1024 + OFF_SH + 1024 + 2 * 4 * SATC_BQ * 4;
   static_assert(SMEM <= 232448, "shared memory budget");
-  static_assert(TMEM_O + NT * DP <= 512, "tensor memory budget");
+  static_assert(TMEM_O + (NT - 1) * O_STRIDE + DP <= 512, "tensor memory budget");
   static_assert(NT == 1 || PST == 2, "alternating query tiles need two P tiles");
 };
 
@@ -83,7 +92,7 @@ struct SaTcShared {
   uint64_t q_full;
   uint64_t k_full[3], k_empty[3];
   uint64_t v_full[2], v_empty[2];
-  uint64_t s_full[2], s_free[2];
+  uint64_t s_full[4], s_free[4];
   uint64_t p_full[2], p_free[2];
   uint64_t o_full;
   uint32_t tmem_base;
@@ -141,8 +150,10 @@ __host__ __device__ constexpr uint32_t satc_idesc(int n, bool b_mn_major) {
 }
 
 
-template <int D, bool FIXED, bool CODES>
-__global__ void __launch_bounds__(SATC_THREADS, 1)
+// FEW: with few codes the last one's weight is not an fp16 zero (a parameter of the kernel: as a test per score pair it cost 3 % of
+// 2 x 8 x 4096 x 40).
+template <int D, bool FIXED, bool CODES, bool FEW>
+__global__ void __launch_bounds__(SaTcCfg<D>::THREADS, 1)
 self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ SelfAttnArgs a) {
   using Cfg = SaTcCfg<D>;
@@ -173,15 +184,17 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     mbar_init(&sh->q_full, 1);
     for (int i = 0; i < 3; ++i) {
       mbar_init(&sh->k_full[i], 1);
-      mbar_init(&sh->k_empty[i], 1);
+      mbar_init(&sh->k_empty[i], NT);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&sh->v_full[i], 1);
       mbar_init(&sh->v_empty[i], 1);
-      mbar_init(&sh->s_full[i], 1);
-      mbar_init(&sh->s_free[i], Cfg::TEAM_WARPS);
       mbar_init(&sh->p_full[i], Cfg::TEAM_WARPS);
       mbar_init(&sh->p_free[i], 1);
+    }
+    for (int i = 0; i < 4; ++i) {
+      mbar_init(&sh->s_full[i], 1);
+      mbar_init(&sh->s_free[i], Cfg::TEAM_WARPS);
     }
     mbar_init(&sh->o_full, 1);
     sh->abort_flag = 0;
@@ -234,31 +247,36 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       }
     }
     __syncwarp();
-  } else if (warp == SATC_WARP_MMA) {
+  } else if (warp == SATC_WARP_MMA || warp == SATC_WARP_MMA2) {
     // ------------------------------------------------------------ score issuer
-    // Both issuing warps run their loops as a whole with uniform control flow, and one elected lane issues a tile's
+    // The issuing warps run their loops as a whole with uniform control flow, and one elected lane issues a tile's
     // MMAs and commits in one block: issued from a loop that a single lane runs, with its addresses in per-lane
     // registers, every MMA cost about twice as much of the warp's time.
     // Score tiles are numbered g = 0 .. N_WALKS * per_walk - 1 in the order (walk, key block, query
-    // tile) and alternate between the two score buffers; a tile is issued as soon as its buffer has
-    // been read, which is early in the arithmetic of tile g - 2.
+    // tile); a tile is issued as soon as its buffer has been read, which is early in the arithmetic of the team's tile before.
+    // Each of two teams has an issuing warp of its own, and two score buffers until the codes walk: a barrier poll waits behind
+    // the MMAs that its warp has issued, so one warp took 580 cycles a tile of the max walk (192 of them MMAs), two take 440.
+    // With the code count as a template parameter: 2 x 8 x 4096 x 40 145.0 -> 135.7 us, 4 x 10 x 1024 x 64 43.9 -> 40.6,
+    // 8 x 8 x 1024 x 80 54.2 -> 52.9 (four buffers behind one issuer: 148.6 on the first).
     {
       constexpr uint32_t IDESC_QK = satc_idesc(SATC_BK, false);
       constexpr uint32_t HI = smem_desc_hi(1024, 2);
       const uint32_t q_lo = smem_desc_lo(smem_u32(sQ)), k_lo = smem_desc_lo(smem_u32(sK));
       const uint32_t k_full0 = smem_u32(&sh->k_full[0]), k_empty0 = smem_u32(&sh->k_empty[0]);
       const uint32_t s_full0 = smem_u32(&sh->s_full[0]), s_free0 = smem_u32(&sh->s_free[0]);
-      const int total = N_WALKS * per_walk;
-      uint32_t ks = 0, k_par = 0;
+      const int total = N_WALKS * per_walk, early = (N_WALKS - 1) * per_walk;
+      constexpr int STEP = Cfg::ISSUERS;
+      const int e = warp == SATC_WARP_MMA ? 0 : 1;
+      uint32_t ks = Cfg::ISSUERS == 2 ? (uint32_t)(e / NT) : 0u, k_par = 0, s_par = 0xFu;  // s_par bit b: parity to wait for on buffer b (fresh barriers pass)
       mbar_wait_handover(smem_u32(&sh->q_full), 0, abort_flag);
-      for (int g = 0; g < total; ++g) {
-        const uint32_t sb = (uint32_t)g & 1u;
-        const uint32_t t = NT == 2 ? sb : 0u;
-        if (t == 0) mbar_wait_handover(k_full0 + ks * 8u, k_par, abort_flag);
-        mbar_wait_handover(s_free0 + sb * 8u, (((uint32_t)g >> 1) & 1u) ^ 1u, abort_flag);
+      for (int g = e, it = 0; g < total; g += STEP, ++it) {
+        const uint32_t sb = (uint32_t)g & (g < early ? (uint32_t)Cfg::BUFS - 1u : 1u);
+        const uint32_t t = NT == 2 ? (uint32_t)e : 0u;
+        mbar_wait_handover(k_full0 + ks * 8u, k_par, abort_flag);
+        mbar_wait_handover(s_free0 + sb * 8u, (s_par >> sb) & 1u, abort_flag);
+        s_par ^= 1u << sb;
         tc_fence_after();
         const uint32_t a_lo = q_lo + t * (uint32_t)(Cfg::TILE >> 4), b_lo = k_lo + ks * (uint32_t)(Cfg::TILE >> 4);
-        const bool k_done = t == NT - 1;
         if (elect_one()) {
 #pragma unroll
           for (int kstep = 0; kstep < Cfg::KSTEPS; ++kstep) {
@@ -266,14 +284,15 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             mma_f16_lohi(tmem_base + sb * SATC_BK, a_lo + off, HI, b_lo + off, HI, IDESC_QK, kstep > 0 ? 1u : 0u);
           }
           mma_commit_addr(s_full0 + sb * 8u);
-          if (k_done) mma_commit_addr(k_empty0 + ks * 8u);
+          mma_commit_addr(k_empty0 + ks * 8u);
         }
         __syncwarp();
-        if (k_done && ++ks == (uint32_t)KST) {
-          ks = 0;
+        ks += Cfg::ISSUERS / NT;  // this warp's next key block
+        if (ks >= (uint32_t)KST) {
+          ks -= (uint32_t)KST;
           k_par ^= 1u;
         }
-        if ((g & 7) == 7 && *abort_flag) break;
+        if ((it & 3) == 3 && *abort_flag) break;
       }
     }
     __syncwarp();
@@ -293,8 +312,8 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         mbar_wait_handover(p_full0 + pb * 8u, (p_par >> pb) & 1u, abort_flag);
         if (t == 0) mbar_wait_handover(v_full0 + vs * 8u, v_par, abort_flag);
         tc_fence_after();
-        const uint32_t a_tmem = tmem_base + SATC_TMEM_P + pb * 64u, b_lo = v_lo + vs * (uint32_t)(Cfg::TILE >> 4);
-        const uint32_t d_tmem = tmem_base + Cfg::TMEM_O + t * Cfg::DP;
+        const uint32_t a_tmem = tmem_base + SATC_TMEM_P + pb * (uint32_t)Cfg::P_STRIDE, b_lo = v_lo + vs * (uint32_t)(Cfg::TILE >> 4);
+        const uint32_t d_tmem = tmem_base + Cfg::TMEM_O + t * Cfg::O_STRIDE;
         const uint32_t acc0 = c >= NT ? 1u : 0u;  // the first key block starts the accumulator
         const bool v_done = t == NT - 1;
         if (elect_one()) {
@@ -352,16 +371,17 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       for (int i = 1; i < PARTS; ++i) z += my_z[i * SATC_BQ];
       return z;
     };
-    uint32_t n = 0, c = 0;  // tiles / codes-walk tiles of this team so far
+    uint32_t c = 0, s_par = 0;  // codes-walk tiles of this team so far; bit b: parity of score buffer b's next tile
     for (int w = 0; w < N_WALKS; ++w) {
       const bool walk_max = (w == 0), walk_codes = (w == N_WALKS - 1);
       const int g0 = w * per_walk;
-      for (int g = TEAMS == 2 ? g0 + ((g0 ^ team) & 1) : g0; g < g0 + per_walk; g += TEAMS, ++n) {
+      for (int g = TEAMS == 2 ? g0 + ((g0 ^ team) & 1) : g0; g < g0 + per_walk; g += TEAMS) {
         const int j = (g - g0) / NT;
-        const uint32_t sb = (uint32_t)g & 1u;
+        const uint32_t sb = (uint32_t)g & (walk_codes ? 1u : (uint32_t)Cfg::BUFS - 1u);
         // After a time-out every wait returns at once and the loops run to their ends on whatever the buffers hold (an
         // error is recorded): no warp leaves early, so the named barriers are always reached by all their warps.
-        mbar_wait_handover(smem_u32(&sh->s_full[sb]), (TEAMS == 2 ? n : n >> 1) & 1u, abort_flag);
+        mbar_wait_handover(smem_u32(&sh->s_full[sb]), (s_par >> sb) & 1u, abort_flag);
+        s_par ^= 1u << sb;
         __syncwarp();
         tc_fence_after();
 #pragma unroll
@@ -430,7 +450,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                   r[i] = min(c0, L);
                   r[i + 1] = min(c1, L);
                 }
-                if (L < (uint32_t)AT_CODE_CAP) {  // (beyond, the last code's weight is an fp16 zero)
+                if (FEW) {
                   b0 = max(b0, p_least);
                   b1 = max(b1, p_least);
                 }
@@ -466,7 +486,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
               __syncwarp();
               tc_fence_after();
             }
-            tmem_st16(t_lane + SATC_TMEM_P + pb * 64u + (uint32_t)(col >> 1), pk);
+            tmem_st16(t_lane + SATC_TMEM_P + pb * (uint32_t)Cfg::P_STRIDE + (uint32_t)(col >> 1), pk);
             if (ch == Cfg::COLS / 32 - 1) {
               tmem_st_wait();
               tc_fence_before();
@@ -505,7 +525,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       __half* o_row = a.O + (((int64_t)b * a.nq + orow) * a.H + h) * D;
       for (int ch = part; ch < D / 8; ch += PARTS) {
         uint32_t o[8];
-        tmem_ld8(t_lane + Cfg::TMEM_O + qt * Cfg::DP + ch * 8, o);
+        tmem_ld8(t_lane + Cfg::TMEM_O + qt * Cfg::O_STRIDE + ch * 8, o);
         tmem_ld_wait();
         __half2 oh[4];
 #pragma unroll
@@ -541,7 +561,7 @@ static bool satc_encode(CUtensorMap* m, const void* base, int B, int n, int H, i
   return encode_map(m, base, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_DATA_TYPE_FLOAT16);
 }
 
-template <int D, bool FIXED, bool CODES>
+template <int D, bool FIXED, bool CODES, bool FEW>
 static dgq_status launch_self_attn2(const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV,
                                        const SelfAttnArgs& a, unsigned grid, cudaStream_t stream) {
   using Cfg = SaTcCfg<D>;
@@ -549,11 +569,11 @@ static dgq_status launch_self_attn2(const CUtensorMap& tmQ, const CUtensorMap& t
   int dev = 0;
   DGQ_CUDA_OK(cudaGetDevice(&dev));
   if (dev >= 64 || !attr_set[dev]) {
-    DGQ_CUDA_OK(cudaFuncSetAttribute(self_attn_logq_kernel<D, FIXED, CODES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    DGQ_CUDA_OK(cudaFuncSetAttribute(self_attn_logq_kernel<D, FIXED, CODES, FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      Cfg::SMEM));
     if (dev < 64) attr_set[dev] = true;
   }
-  DGQ_CUDA_OK(launch_pdl(self_attn_logq_kernel<D, FIXED, CODES>, dim3(grid), dim3(SATC_THREADS), (size_t)Cfg::SMEM, stream,
+  DGQ_CUDA_OK(launch_pdl(self_attn_logq_kernel<D, FIXED, CODES, FEW>, dim3(grid), dim3(Cfg::THREADS), (size_t)Cfg::SMEM, stream,
                          tmQ, tmK, tmV, a));
   g_launches += 1;
   DGQ_CUDA_OK(cudaGetLastError());
@@ -575,10 +595,13 @@ static dgq_status launch_self_attn(const SelfAttnArgs& a, cudaStream_t stream) {
     return DGQ_ERR_CUDA;
   const unsigned g = (unsigned)grid;
   if (a.fixed_scale)
-    return a.codes_out ? launch_self_attn2<D, true, true>(tmQ, tmK, tmV, aa, g, stream)
-                       : launch_self_attn2<D, true, false>(tmQ, tmK, tmV, aa, g, stream);
-  return a.codes_out ? launch_self_attn2<D, false, true>(tmQ, tmK, tmV, aa, g, stream)
-                     : launch_self_attn2<D, false, false>(tmQ, tmK, tmV, aa, g, stream);
+    return a.codes_out ? launch_self_attn2<D, true, true, false>(tmQ, tmK, tmV, aa, g, stream)
+                       : launch_self_attn2<D, true, false, false>(tmQ, tmK, tmV, aa, g, stream);
+  if ((1 << a.bits) - 1 < AT_CODE_CAP)
+    return a.codes_out ? launch_self_attn2<D, false, true, true>(tmQ, tmK, tmV, aa, g, stream)
+                       : launch_self_attn2<D, false, false, true>(tmQ, tmK, tmV, aa, g, stream);
+  return a.codes_out ? launch_self_attn2<D, false, true, false>(tmQ, tmK, tmV, aa, g, stream)
+                     : launch_self_attn2<D, false, false, false>(tmQ, tmK, tmV, aa, g, stream);
 }
 
 }  // namespace dgq

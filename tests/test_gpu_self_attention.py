@@ -65,6 +65,18 @@ def test_fixed_scale():
     _compare(torch, b, Q, K, V, 6, fixed=[1.0, 0.25])
 
 
+@pytest.mark.parametrize("d", [40, 80, 160])
+@pytest.mark.parametrize("n", [127, 128, 129, 257, 385, 513, 640])
+@pytest.mark.parametrize("bits,fixed", [(8, None), (4, None), (8, [0.5])])
+def test_key_block_counts(n, d, bits, fixed):
+    """One to five key blocks, full and ragged: every phase of the score buffers at the change from the walks that use four of
+    them to the one that uses two.  Bounds as in the other cases: codes within one level, outputs 1e-3 plus what a moved code
+    explains."""
+    torch, b = gpu()
+    Q, K, V = _qkv(20 + n, 1, 2, n, d)
+    _compare(torch, b, Q, K, V, bits, fixed)
+
+
 def test_level_at_1024_tokens():
     """32 x 32 level: 1024 tokens, 8 heads of 80 features; the whole output against the oracle."""
     torch, b = gpu()

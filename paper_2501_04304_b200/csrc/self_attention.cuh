@@ -348,6 +348,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const unsigned long long scale2 = pack_f32x2(scale, scale), nscale2 = pack_f32x2(-scale, -scale);
     const unsigned long long one2 = pack_f32x2(1.f, 1.f);
     const unsigned long long magic2 = pack_f32x2(12582912.0f, 12582912.0f);
+    const unsigned long long zero2 = 0ull, to_weight2 = pack_f32x2(__uint_as_float(0x46B504F4u), __uint_as_float(0x46B504F4u));
     const uint32_t L = (1u << a.bits) - 1u;
     const uint32_t code_top = 0x4B400000u + L;                                 // bits of 1.5 * 2^23 + last code
     const uint32_t p_top = 0x4B400000u + min(L, (uint32_t)AT_CODE_CAP);       // ... + last code with a non-zero fp16 weight
@@ -425,10 +426,15 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             if (!FIXED) {
               // e = 2^x with x = t * scale - max <= 0 up to rounding (the row maximum has code 0); -inf logits (keys beyond
               // nk) give 0.  The row sum takes e as it is.  The power of two nearest to it in the log domain, times 2^14, is e
-              // with the mantissa rounded at sqrt(2) and 14 more in the exponent: adding 2 - sqrt(2) in mantissa units
-              // carries into the exponent where x is nearer to the smaller code, and the mantissa is cut off.  One exponential
-              // and two integer operations per score serve row sum and weight (with the code formed first, by an add of
-              // 1.5 * 2^23, a clamp, a shift and a subtraction, a score took half again as many instructions).
+              // times sqrt(2) 2^14 with the mantissa cut off: the product reaches the next exponent where x is nearer to the smaller
+              // code.  The factor is the fp32 number above sqrt(2) 2^14; with it the rounded product reaches the exponent at
+              // mantissa 0x3504F3 and not one below, the same mantissas as an integer add of 2 - sqrt(2) and 14 exponents gives
+              // (compared over all of them).  Packed, it takes one instruction for two scores where the add took two: 2 x 8 x 4096
+              // x 40 137.4 -> 136.7 us, 2 x 8 x 1024 x 128 14.76 -> 14.61; half the pairs by the add, to spread the work over both
+              // pipes, took 138.0.  With the code formed first, by an add of 1.5 * 2^23, a clamp, a shift and a subtraction, a
+              // score took half again as many instructions.  Exponentials of 2 to 6 of 16 pairs as polynomials of degree 5 on
+              // the multiply-add pipe took 133.6 to 142.4 us, 2 to 8 % more with 4-bit scores, and moved a third more codes away
+              // from those of 64-bit arithmetic.
               // The 2^14 must not be part of x: 14 - distance is rounded at 2^-21 where the distance itself is held to 2^-25,
               // and 8e-7 of the scores then take a neighbour of the code that 64 bits give, against 2.6e-7 this way and 4.3e-7
               // with the logit rounded by an add (2 x 8 x 4096 x 40).  The 32 columns are summed before they join the row's
@@ -441,8 +447,11 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 float x0, x1;
                 unpack_f32x2(x2, x0, x1);
                 const float e0 = ex2_approx(x0), e1 = ex2_approx(x1);
-                zc = fma_f32x2(pack_f32x2(e0, e1), one2, zc);
-                uint32_t b0 = (__float_as_uint(e0) + 0x074AFB0Du) & 0xFF800000u, b1 = (__float_as_uint(e1) + 0x074AFB0Du) & 0xFF800000u;
+                const unsigned long long e2 = pack_f32x2(e0, e1);
+                zc = fma_f32x2(e2, one2, zc);
+                float w0, w1;
+                unpack_f32x2(fma_f32x2(e2, to_weight2, zero2), w0, w1);
+                uint32_t b0 = __float_as_uint(w0) & 0xFF800000u, b1 = __float_as_uint(w1) & 0xFF800000u;
                 if (CODES) {
                   // exponent field 127 + 14 - code; where e has left the fp32 range the code comes from x itself
                   const uint32_t c0 = x0 > -120.f ? 141u - (b0 >> 23) : __float_as_uint(fminf(-x0, 255.f) + 12582912.0f) & 0xFFu;

@@ -65,7 +65,10 @@ struct SaTcCfg {
   // The softmax warps form two teams of eight that take the score tiles in turn, so that one team's waits, tensor-memory
   // round trips and hand-overs run under the other's arithmetic; with a single P tile they stay together.
   static constexpr int TEAMS = PST;
-  static constexpr int ISSUERS = TEAMS;        // warps that issue score tiles
+  // Warps that issue score tiles.  Two only where each sees every key block (its own query tile's products with it): two that took
+  // the blocks of one query tile in turn would wait for a stage's next block by parity without having seen the block before
+  // it arrive, and the wait passes at once when that load lands late.
+  static constexpr int ISSUERS = NT == 2 && TEAMS == 2 ? 2 : 1;
   static constexpr int BUFS = 2 * ISSUERS;     // score buffers of the walks before the codes walk
   static constexpr int THREADS = (18 + ISSUERS) * 32;
   static constexpr int TEAM_WARPS = SATC_SOFTMAX_WARPS / TEAMS;
@@ -254,10 +257,10 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     // registers, every MMA cost about twice as much of the warp's time.
     // Score tiles are numbered g = 0 .. N_WALKS * per_walk - 1 in the order (walk, key block, query
     // tile); a tile is issued as soon as its buffer has been read, which is early in the arithmetic of the team's tile before.
-    // Each of two teams has an issuing warp of its own, and two score buffers until the codes walk: a barrier poll waits behind
+    // With two query tiles each team has an issuing warp of its own, and two score buffers until the codes walk: a barrier poll waits behind
     // the MMAs that its warp has issued, so one warp took 580 cycles a tile of the max walk (192 of them MMAs), two take 440.
-    // With the code count as a template parameter: 2 x 8 x 4096 x 40 145.0 -> 135.7 us, 4 x 10 x 1024 x 64 43.9 -> 40.6,
-    // 8 x 8 x 1024 x 80 54.2 -> 52.9 (four buffers behind one issuer: 148.6 on the first).
+    // With the code count as a template parameter: 2 x 8 x 4096 x 40 145.0 -> 135.7 us, 4 x 10 x 1024 x 64 43.9 -> 40.6
+    // (four buffers behind one issuer: 148.6 on the first).
     {
       constexpr uint32_t IDESC_QK = satc_idesc(SATC_BK, false);
       constexpr uint32_t HI = smem_desc_hi(1024, 2);
@@ -430,7 +433,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
               // code.  The factor is the fp32 number above sqrt(2) 2^14; with it the rounded product reaches the exponent at
               // mantissa 0x3504F3 and not one below, the same mantissas as an integer add of 2 - sqrt(2) and 14 exponents gives
               // (compared over all of them).  Packed, it takes one instruction for two scores where the add took two: 2 x 8 x 4096
-              // x 40 137.4 -> 136.7 us, 2 x 8 x 1024 x 128 14.76 -> 14.61; half the pairs by the add, to spread the work over both
+              // x 40 137.4 -> 136.7 us; half the pairs by the add, to spread the work over both
               // pipes, took 138.0.  With the code formed first, by an add of 1.5 * 2^23, a clamp, a shift and a subtraction, a
               // score took half again as many instructions.  Exponentials of 2 to 6 of 16 pairs as polynomials of degree 5 on
               // the multiply-add pipe took 133.6 to 142.4 us, 2 to 8 % more with 4-bit scores, and moved a third more codes away

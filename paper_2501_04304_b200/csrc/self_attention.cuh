@@ -426,6 +426,10 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             const uint32_t pb = TEAMS == 2 ? sb : 0u;
             const int64_t code_row = (((int64_t)b * a.H + h) * a.nq + row0 + qt * SATC_BQ + row) * a.nk + j * SATC_BK + col;
             uint32_t pk[16];
+            // Codes of four keys share a register: one each, next to the logits and weights, spilled 24 bytes a thread for heads of
+            // 40 and 64 (2 x 8 x 1024 x 40 with codes 324.7 -> 321.6 us, 4 x 10 x 1024 x 64 612.7 -> 608.7; byte stores bound both).
+            uint32_t cd[8] = {};
+            auto keep_codes = [&](int i, uint32_t c0, uint32_t c1) { cd[i >> 2] |= (c0 | c1 << 8) << (8 * (i & 2)); };
             if (!FIXED) {
               // e = 2^x with x = t * scale - max <= 0 up to rounding (the row maximum has code 0); -inf logits (keys beyond
               // nk) give 0.  The row sum takes e as it is.  The power of two nearest to it in the log domain, times 2^14, is e
@@ -459,8 +463,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                   // exponent field 127 + 14 - code; where e has left the fp32 range the code comes from x itself
                   const uint32_t c0 = x0 > -120.f ? 141u - (b0 >> 23) : __float_as_uint(fminf(-x0, 255.f) + 12582912.0f) & 0xFFu;
                   const uint32_t c1 = x1 > -120.f ? 141u - (b1 >> 23) : __float_as_uint(fminf(-x1, 255.f) + 12582912.0f) & 0xFFu;
-                  r[i] = min(c0, L);
-                  r[i + 1] = min(c1, L);
+                  keep_codes(i, min(c0, L), min(c1, L));
                 }
                 if (FEW) {
                   b0 = max(b0, p_least);
@@ -482,10 +485,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 float y0, y1;
                 unpack_f32x2(fma_f32x2(pack_f32x2(fmaxf(x0, 0.f), fmaxf(x1, 0.f)), one2, magic2), y0, y1);
                 const uint32_t b0 = __float_as_uint(y0), b1 = __float_as_uint(y1);
-                if (CODES) {
-                  r[i] = min(b0, code_top) & 0xFFu;
-                  r[i + 1] = min(b1, code_top) & 0xFFu;
-                }
+                if (CODES) keep_codes(i, min(b0, code_top) & 0xFFu, min(b1, code_top) & 0xFFu);
                 // 2^(14 - code) as fp32 bits: (127 + 14) << 23 minus code << 23 (the bits of 1.5 * 2^23 shift out)
                 const float p0 = __uint_as_float(0x46800000u - (min(b0, p_top) << 23));
                 const float p1 = __uint_as_float(0x46800000u - (min(b1, p_top) << 23));
@@ -509,7 +509,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
             if (CODES && row0 + qt * SATC_BQ + row < a.nq) {
 #pragma unroll
               for (int i = 0; i < 32; ++i)
-                if (i < valid) a.codes_out[code_row + i] = (uint8_t)r[i];
+                if (i < valid) a.codes_out[code_row + i] = (uint8_t)(cd[i >> 2] >> (8 * (i & 3)));
             }
           }
         }

@@ -153,8 +153,9 @@ __host__ __device__ constexpr uint32_t satc_idesc(int n, bool b_mn_major) {
 }
 
 
-// FEW: with few codes the last one's weight is not an fp16 zero (a parameter of the kernel: as a test per score pair it cost 3 % of
-// 2 x 8 x 4096 x 40).
+// FEW: with few codes the last one's weight is not an fp16 zero, and smaller weights are raised to it, two in one instruction.  A
+// parameter of the kernel: as a test per score pair it cost the 8-bit scores of 2 x 8 x 4096 x 40 139.2 against 135.3 us.  4-bit
+// scores there: 142.3 us with two integer maxima a pair, 139.1 with one of packed halves; 8 x 8 x 1024 x 80 56.9 and 56.0.
 template <int D, bool FIXED, bool CODES, bool FEW>
 __global__ void __launch_bounds__(SaTcCfg<D>::THREADS, 1)
 self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -355,7 +356,8 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const uint32_t L = (1u << a.bits) - 1u;
     const uint32_t code_top = 0x4B400000u + L;                                 // bits of 1.5 * 2^23 + last code
     const uint32_t p_top = 0x4B400000u + min(L, (uint32_t)AT_CODE_CAP);       // ... + last code with a non-zero fp16 weight
-    const uint32_t p_least = (127u + (uint32_t)AT_P_SHIFT - min(L, 100u)) << 23;  // weight of the last code
+    // weight of the last code, a power of two that fp16 holds where FEW is set
+    const __half2 p_least2 = __float2half2_rn(__uint_as_float((127u + (uint32_t)AT_P_SHIFT - min(L, 100u)) << 23));
     float m_raw = -INFINITY, m2 = 0.f;
     float base = 0.f;  // fixed scale: code = rint(base - t * scale); row maximum as scale: code = rint(-(t * scale + base))
     unsigned long long zs = 0ull;
@@ -465,11 +467,8 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                   const uint32_t c1 = x1 > -120.f ? 141u - (b1 >> 23) : __float_as_uint(fminf(-x1, 255.f) + 12582912.0f) & 0xFFu;
                   keep_codes(i, min(c0, L), min(c1, L));
                 }
-                if (FEW) {
-                  b0 = max(b0, p_least);
-                  b1 = max(b1, p_least);
-                }
-                const __half2 ph = __floats2half2_rn(__uint_as_float(b0), __uint_as_float(b1));
+                __half2 ph = __floats2half2_rn(__uint_as_float(b0), __uint_as_float(b1));
+                if (FEW) ph = __hmax2(ph, p_least2);
                 pk[i >> 1] = *reinterpret_cast<const uint32_t*>(&ph);  // key i in the low half
               }
               zs = fma_f32x2(zc, one2, zs);

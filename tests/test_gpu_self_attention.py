@@ -66,6 +66,17 @@ def test_fixed_scale():
 
 
 @pytest.mark.parametrize("d", [40, 80, 160])
+@pytest.mark.parametrize("bits", [2, 3, 4, 5])
+def test_few_codes(bits, d):
+    """Up to 5 bits the last code's weight is not an fp16 zero (2^-17 at 5 bits, below the normal fp16 numbers): logits spread far
+    beyond the last code, so most scores carry that weight, and with values of one sign it shows in the output (at 4 bits 380 x 2^-15,
+    12 times the tolerance; at 5 bits it does not).  Bounds as in the other cases."""
+    torch, b = gpu()
+    Q, K, V = _qkv(60 + bits, 1, 2, 385, d)
+    _compare(torch, b, Q * np.float16(8), K, np.abs(V), bits)
+
+
+@pytest.mark.parametrize("d", [40, 80, 160])
 @pytest.mark.parametrize("n", [127, 128, 129, 257, 385, 513, 640])
 @pytest.mark.parametrize("bits,fixed", [(8, None), (4, None), (8, [0.5])])
 def test_key_block_counts(n, d, bits, fixed):

@@ -69,6 +69,7 @@ struct SaTcCfg {
   // the blocks of one query tile in turn would wait for a stage's next block by parity without having seen the block before
   // it arrive, and the wait passes at once when that load lands late.
   static constexpr int ISSUERS = NT == 2 && TEAMS == 2 ? 2 : 1;
+  static constexpr int ABORT_EVERY = 8 / ISSUERS;  // tiles of an issuing warp between its reads of the abort flag: every eighth tile of all
   static constexpr int BUFS = 2 * ISSUERS;     // score buffers of the walks before the codes walk
   static constexpr int THREADS = (18 + ISSUERS) * 32;
   static constexpr int TEAM_WARPS = SATC_SOFTMAX_WARPS / TEAMS;
@@ -296,7 +297,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           ks -= (uint32_t)KST;
           k_par ^= 1u;
         }
-        if ((it & 3) == 3 && *abort_flag) break;
+        if ((it & (Cfg::ABORT_EVERY - 1)) == Cfg::ABORT_EVERY - 1 && *abort_flag) break;
       }
     }
     __syncwarp();

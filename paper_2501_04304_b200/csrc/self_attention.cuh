@@ -14,9 +14,9 @@
 //                  is done on the mantissa of 2^(t - max); with a fixed scale it is done on base - t itself.  The two
 //                  agree but for scores within a few units in the last place of a boundary.
 // Roles: 16 softmax warps in two teams that take the score tiles in turn (warp w reads tensor-memory lanes 32 (w % 4) ..
-// +31 and half of the 128 columns of its team's tiles), one TMA producer lane, one warp that issues the score MMAs and one
-// that issues the P V MMAs (each tile costs an issuing warp a chain of dependent instructions, so the two run apart; the
-// instructions themselves come from one elected lane).  With two query tiles the softmax warps alternate between them, so
+// +31 and half of the 128 columns of its team's tiles), one TMA producer lane, one warp per query tile that issues its score
+// MMAs and one that issues the P V MMAs (each tile costs an issuing warp a chain of dependent instructions, so they run apart;
+// the instructions themselves come from one elected lane).  With two query tiles the softmax warps alternate between them, so
 // every K / V block fetched from L2 serves 256 query rows and one tile's MMAs run under the other tile's
 // arithmetic.  Q, K and P are K-major operands with 128-byte swizzled rows; V is used as it lies in memory (features
 // contiguous; one row = 64 features of one key), an MN-major operand.  Tiles are
@@ -44,7 +44,7 @@ constexpr int SATC_SOFTMAX_WARPS = 16;
 constexpr int SATC_WARP_TMA = 16;
 constexpr int SATC_WARP_MMA = 17;   // issues S = Q K^T (and owns the tensor-memory allocation)
 constexpr int SATC_WARP_PV = 18;    // issues O += P V
-constexpr int SATC_WARP_MMA2 = 19;  // issues every other score tile (where the softmax warps form two teams)
+constexpr int SATC_WARP_MMA2 = 19;  // issues the second query tile's S (launched where there are two)
 
 constexpr int SATC_BQ = 128;            // query rows per tile
 constexpr int SATC_BK = 128;            // keys per block
@@ -65,10 +65,10 @@ struct SaTcCfg {
   // The softmax warps form two teams of eight that take the score tiles in turn, so that one team's waits, tensor-memory
   // round trips and hand-overs run under the other's arithmetic; with a single P tile they stay together.
   static constexpr int TEAMS = PST;
-  // Warps that issue score tiles.  Two only where each sees every key block (its own query tile's products with it): two that took
-  // the blocks of one query tile in turn would wait for a stage's next block by parity without having seen the block before
-  // it arrive, and the wait passes at once when that load lands late.
-  static constexpr int ISSUERS = NT == 2 && TEAMS == 2 ? 2 : 1;
+  // Warps that issue score tiles: one per query tile, so that each sees every key block.  Two that took the blocks of one query
+  // tile in turn would wait for a stage's next block by parity without having seen the block before it arrive, and
+  // the wait passes at once when that load lands late.
+  static constexpr int ISSUERS = NT;
   static constexpr int ABORT_EVERY = 8 / ISSUERS;  // tiles of an issuing warp between its reads of the abort flag: every eighth tile of all
   static constexpr int BUFS = 2 * ISSUERS;     // score buffers of the walks before the codes walk
   static constexpr int THREADS = (18 + ISSUERS) * 32;
@@ -76,9 +76,9 @@ struct SaTcCfg {
   static constexpr int SPLIT = TEAM_WARPS / 4;          // warps of a team that share 32 rows of a tile
   static constexpr int COLS = SATC_BK / SPLIT;          // score columns of a warp
   static constexpr int PARTS = NT == 2 ? SPLIT : 4;     // threads that hold a part of a row's statistics
-  // Tensor memory: score buffers at columns 0 and 128; with two teams two more at 256 and 384 in the walks before the codes
-  // walk, which have no use for P and O yet.  With two query tiles a team's P and O lie inside its own second buffer there,
-  // because the teams enter the codes walk one by one; else all warps meet between the walks.
+  // Tensor memory: score buffers at columns 0 and 128; with two query tiles two more at 256 and 384 in the walks before the
+  // codes walk, which have no use for P and O yet.  A team's P and O then lie inside its own second buffer, because the
+  // teams enter the codes walk one by one.
   static constexpr int P_STRIDE = NT == 2 ? 128 : 64;
   static constexpr int TMEM_O = NT == 2 ? SATC_TMEM_P + 64 : SATC_TMEM_P + PST * 64;
   static constexpr int O_STRIDE = 128;
@@ -252,7 +252,7 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       }
     }
     __syncwarp();
-  } else if (warp == SATC_WARP_MMA || warp == SATC_WARP_MMA2) {
+  } else if (warp == SATC_WARP_MMA || (Cfg::ISSUERS == 2 && warp == SATC_WARP_MMA2)) {
     // ------------------------------------------------------------ score issuer
     // The issuing warps run their loops as a whole with uniform control flow, and one elected lane issues a tile's
     // MMAs and commits in one block: issued from a loop that a single lane runs, with its addresses in per-lane
@@ -270,13 +270,11 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       const uint32_t k_full0 = smem_u32(&sh->k_full[0]), k_empty0 = smem_u32(&sh->k_empty[0]);
       const uint32_t s_full0 = smem_u32(&sh->s_full[0]), s_free0 = smem_u32(&sh->s_free[0]);
       const int total = N_WALKS * per_walk, early = (N_WALKS - 1) * per_walk;
-      constexpr int STEP = Cfg::ISSUERS;
-      const int e = warp == SATC_WARP_MMA ? 0 : 1;
-      uint32_t ks = Cfg::ISSUERS == 2 ? (uint32_t)(e / NT) : 0u, k_par = 0, s_par = 0xFu;  // s_par bit b: parity to wait for on buffer b (fresh barriers pass)
+      const uint32_t t = Cfg::ISSUERS == 2 && warp == SATC_WARP_MMA2 ? 1u : 0u;  // this warp's query tile
+      uint32_t ks = 0, k_par = 0, s_par = 0xFu;  // s_par bit b: parity to wait for on buffer b (fresh barriers pass)
       mbar_wait_handover(smem_u32(&sh->q_full), 0, abort_flag);
-      for (int g = e, it = 0; g < total; g += STEP, ++it) {
+      for (int g = (int)t, it = 0; g < total; g += Cfg::ISSUERS, ++it) {
         const uint32_t sb = (uint32_t)g & (g < early ? (uint32_t)Cfg::BUFS - 1u : 1u);
-        const uint32_t t = NT == 2 ? (uint32_t)e : 0u;
         mbar_wait_handover(k_full0 + ks * 8u, k_par, abort_flag);
         mbar_wait_handover(s_free0 + sb * 8u, (s_par >> sb) & 1u, abort_flag);
         s_par ^= 1u << sb;
@@ -292,9 +290,8 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
           mma_commit_addr(k_empty0 + ks * 8u);
         }
         __syncwarp();
-        ks += Cfg::ISSUERS / NT;  // this warp's next key block
-        if (ks >= (uint32_t)KST) {
-          ks -= (uint32_t)KST;
+        if (++ks == (uint32_t)KST) {
+          ks = 0;
           k_par ^= 1u;
         }
         if ((it & (Cfg::ABORT_EVERY - 1)) == Cfg::ABORT_EVERY - 1 && *abort_flag) break;

@@ -65,24 +65,25 @@ def test_fixed_scale():
     _compare(torch, b, Q, K, V, 6, fixed=[1.0, 0.25])
 
 
-@pytest.mark.parametrize("d", [40, 80, 160])
-@pytest.mark.parametrize("bits", [2, 3, 4, 5])
+@pytest.mark.parametrize("d", [40, 64, 80, 128, 160])
+@pytest.mark.parametrize("bits", [2, 3, 4, 5, 6])
 def test_few_codes(bits, d):
     """Up to 5 bits the last code's weight is not an fp16 zero (2^-17 at 5 bits, below the normal fp16 numbers): logits spread far
     beyond the last code, so most scores carry that weight, and with values of one sign it shows in the output (at 4 bits 380 x 2^-15,
-    12 times the tolerance; at 5 bits it does not).  Bounds as in the other cases."""
+    12 times the tolerance; at 5 bits it does not).  6 bits is the first count whose last codes are fp16 zeros, another kernel.
+    Bounds as in the other cases."""
     torch, b = gpu()
     Q, K, V = _qkv(60 + bits, 1, 2, 385, d)
     _compare(torch, b, Q * np.float16(8), K, np.abs(V), bits)
 
 
-@pytest.mark.parametrize("d", [40, 80, 160])
+@pytest.mark.parametrize("d", [40, 64, 80, 128, 160])
 @pytest.mark.parametrize("n", [127, 128, 129, 257, 385, 513, 640])
 @pytest.mark.parametrize("bits,fixed", [(8, None), (4, None), (8, [0.5])])
 def test_key_block_counts(n, d, bits, fixed):
-    """One to five key blocks, full and ragged: every phase of the score buffers at the change from the walks that use four of
-    them to the one that uses two.  Bounds as in the other cases: codes within one level, outputs 1e-3 plus what a moved code
-    explains."""
+    """One to five key blocks, full and ragged: every stage of the K ring is used again, and for heads of 40 and 64 every phase of the score
+    buffers meets the change from the walks that use four of them to the one that uses two.  Bounds as in the
+    other cases: codes within one level, outputs 1e-3 plus what a moved code explains."""
     torch, b = gpu()
     Q, K, V = _qkv(20 + n, 1, 2, n, d)
     _compare(torch, b, Q, K, V, bits, fixed)
@@ -93,6 +94,34 @@ def test_level_at_1024_tokens():
     torch, b = gpu()
     Q, K, V = _qkv(4, 1, 8, 1024, 80)
     _compare(torch, b, Q, K, V, 8)
+
+
+@pytest.mark.parametrize("B,H,n,d", [
+    (4, 10, 2048, 64),        # 320 CTAs of two query tiles
+    (8, 8, 1024, 80),         # 512 CTAs of one
+    (4, 8, 1024, 128),        # 256
+    (8, 8, 1024, 160),        # 512, the softmax warps in one team
+])
+def test_several_rounds_of_ctas(B, H, n, d):
+    """More CTAs than the device holds at once (one per SM), so that their key and value loads compete and land late: a wait that passes
+    before its load would show as a time-out or as wrong rows.  Five calls give the same bits, no wait ran out,
+    and sampled rows of every prompt and head are held to the oracle with the bounds of the other cases."""
+    torch, b = gpu()
+    Q, K, V = _qkv(80 + d, B, H, n, d)
+    dev = [to_dev(torch, x) for x in (Q, K, V)]
+    O, codes = b.self_attn_logq(*dev, 8, want_codes=True)
+    for _ in range(5):
+        again, _ = b.self_attn_logq(*dev, 8)
+        assert torch.equal(O, again)
+    assert b.device_status() == 0
+    rows = np.random.default_rng(d).choice(n, 12, replace=False)
+    O_ref, codes_ref, s_ref, _ = oa.self_attn_logq(Q[:, rows], K, V, 8)
+    at = torch.from_numpy(rows).cuda()
+    c = codes[:, :, at].cpu().numpy().astype(np.int64)
+    diff = check_codes(c, codes_ref)
+    Og = O[:, at].float().cpu().numpy().astype(np.float64)
+    bound = 1e-3 * np.max(np.abs(O_ref)) + flipped_output_bound(diff, c, codes_ref, s_ref, V)
+    assert np.all(np.abs(Og - O_ref) <= bound), f"max excess {np.max(np.abs(Og - O_ref) - bound):.3e}"
 
 
 def test_argument_errors():

@@ -260,9 +260,9 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     // Score tiles are numbered g = 0 .. N_WALKS * per_walk - 1 in the order (walk, key block, query
     // tile); a tile is issued as soon as its buffer has been read, which is early in the arithmetic of the team's tile before.
     // With two query tiles each team has an issuing warp of its own, and two score buffers until the codes walk: a barrier poll waits behind
-    // the MMAs that its warp has issued, so one warp took 580 cycles a tile of the max walk (192 of them MMAs), two take 440.
-    // With the code count as a template parameter: 2 x 8 x 4096 x 40 145.0 -> 135.7 us, 4 x 10 x 1024 x 64 43.9 -> 40.6
-    // (four buffers behind one issuer: 148.6 on the first).
+    // the MMAs that its warp has issued, so one warp took 580 cycles a tile of the max walk (192 of them MMAs), two take 444.
+    // 2 x 8 x 4096 x 40 143.0 -> 136.2 us, 4 x 10 x 1024 x 64 42.9 -> 40.4 (four buffers behind one issuer took 3.6 us more than two
+    // on the first).
     {
       constexpr uint32_t IDESC_QK = satc_idesc(SATC_BK, false);
       constexpr uint32_t HI = smem_desc_hi(1024, 2);
@@ -436,15 +436,16 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
               // times sqrt(2) 2^14 with the mantissa cut off: the product reaches the next exponent where x is nearer to the smaller
               // code.  The factor is the fp32 number above sqrt(2) 2^14; with it the rounded product reaches the exponent at
               // mantissa 0x3504F3 and not one below, the same mantissas as an integer add of 2 - sqrt(2) and 14 exponents gives
-              // (compared over all of them).  Packed, it takes one instruction for two scores where the add took two: 2 x 8 x 4096
-              // x 40 137.4 -> 136.7 us; half the pairs by the add, to spread the work over both
-              // pipes, took 138.0.  With the code formed first, by an add of 1.5 * 2^23, a clamp, a shift and a subtraction, a
+              // (compared over all of them).  Packed, it takes one instruction for two scores where the add takes two: 2 x 8 x 4096
+              // x 40 136.15 (136.09-136.24) -> 135.50 us (135.48-135.55), 4 x 10 x 1024 x 64 40.41 -> 40.26.  Few codes keep the add:
+              // next to their maximum of packed halves the product was the slower one, 137.34 against 136.86 us and 41.50
+              // against 41.19 (but not where codes are written: the add spills there).  With the code formed first, by an add of 1.5 * 2^23, a clamp, a shift and a subtraction, a
               // score took half again as many instructions.  Exponentials of 2 to 6 of 16 pairs as polynomials of degree 5 on
-              // the multiply-add pipe took 133.6 to 142.4 us, 2 to 8 % more with 4-bit scores, and moved a third more codes away
+              // the multiply-add pipe took 133.6 to 142.4 us, 2 to 8 % more with 4-bit scores, and moved 36 to 64 % more codes away
               // from those of 64-bit arithmetic.
               // The 2^14 must not be part of x: 14 - distance is rounded at 2^-21 where the distance itself is held to 2^-25,
-              // and 8e-7 of the scores then take a neighbour of the code that 64 bits give, against 2.6e-7 this way and 4.3e-7
-              // with the logit rounded by an add (2 x 8 x 4096 x 40).  The 32 columns are summed before they join the row's
+              // and 8e-7 of the scores then take a neighbour of the code that 64 bits give, against 2.4e-7 this way (eight draws, 1.9e-7
+              // to 2.9e-7) and 4.3e-7 with the logit rounded by an add (2 x 8 x 4096 x 40).  The 32 columns are summed before they join the row's
               // sum, which keeps the chain of rounded additions short.
               const unsigned long long base2 = pack_f32x2(base, base);
               unsigned long long zc = 0ull;
@@ -456,9 +457,16 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
                 const float e0 = ex2_approx(x0), e1 = ex2_approx(x1);
                 const unsigned long long e2 = pack_f32x2(e0, e1);
                 zc = fma_f32x2(e2, one2, zc);
-                float w0, w1;
-                unpack_f32x2(fma_f32x2(e2, to_weight2, zero2), w0, w1);
-                uint32_t b0 = __float_as_uint(w0) & 0xFF800000u, b1 = __float_as_uint(w1) & 0xFF800000u;
+                uint32_t b0, b1;
+                if (FEW && !CODES) {
+                  b0 = (__float_as_uint(e0) + 0x074AFB0Du) & 0xFF800000u;
+                  b1 = (__float_as_uint(e1) + 0x074AFB0Du) & 0xFF800000u;
+                } else {
+                  float w0, w1;
+                  unpack_f32x2(fma_f32x2(e2, to_weight2, zero2), w0, w1);
+                  b0 = __float_as_uint(w0) & 0xFF800000u;
+                  b1 = __float_as_uint(w1) & 0xFF800000u;
+                }
                 if (CODES) {
                   // exponent field 127 + 14 - code; where e has left the fp32 range the code comes from x itself
                   const uint32_t c0 = x0 > -120.f ? 141u - (b0 >> 23) : __float_as_uint(fminf(-x0, 255.f) + 12582912.0f) & 0xFFu;

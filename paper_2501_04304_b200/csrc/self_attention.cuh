@@ -271,12 +271,12 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       const uint32_t s_full0 = smem_u32(&sh->s_full[0]), s_free0 = smem_u32(&sh->s_free[0]);
       const int total = N_WALKS * per_walk, early = (N_WALKS - 1) * per_walk;
       const uint32_t t = Cfg::ISSUERS == 2 && warp == SATC_WARP_MMA2 ? 1u : 0u;  // this warp's query tile
-      uint32_t ks = 0, k_par = 0, s_par = 0xFu;  // s_par bit b: parity to wait for on buffer b (fresh barriers pass)
+      uint32_t ks = 0, k_par = 0, s_par = 0xFu;  // s_par bit b: parity to wait for on buffer b of four (fresh barriers pass)
       mbar_wait_handover(smem_u32(&sh->q_full), 0, abort_flag);
       for (int g = (int)t, it = 0; g < total; g += Cfg::ISSUERS, ++it) {
         const uint32_t sb = (uint32_t)g & (g < early ? (uint32_t)Cfg::BUFS - 1u : 1u);
         mbar_wait_handover(k_full0 + ks * 8u, k_par, abort_flag);
-        mbar_wait_handover(s_free0 + sb * 8u, (s_par >> sb) & 1u, abort_flag);
+        mbar_wait_handover(s_free0 + sb * 8u, (Cfg::ISSUERS == 2 ? s_par >> sb : ((uint32_t)g >> 1) ^ 1u) & 1u, abort_flag);
         s_par ^= 1u << sb;
         tc_fence_after();
         const uint32_t a_lo = q_lo + t * (uint32_t)(Cfg::TILE >> 4), b_lo = k_lo + ks * (uint32_t)(Cfg::TILE >> 4);
@@ -375,7 +375,10 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       for (int i = 1; i < PARTS; ++i) z += my_z[i * SATC_BQ];
       return z;
     };
-    uint32_t c = 0, s_par = 0;  // codes-walk tiles of this team so far; bit b: parity of score buffer b's next tile
+    // c: codes-walk tiles of this team so far.  s_par bit b: parity of score buffer b's next tile, where a team has two in turn.
+    // Where it has one, a single bit, and where all warps take both buffers in turn, the tile's number: a bit for each buffer there
+    // cost 8 x 8 x 1024 x 80 56.05 against 55.61 us, 8 x 8 x 1024 x 160 with a fixed scale 111.72 against 111.19.
+    uint32_t c = 0, s_par = 0;
     for (int w = 0; w < N_WALKS; ++w) {
       const bool walk_max = (w == 0), walk_codes = (w == N_WALKS - 1);
       const int g0 = w * per_walk;
@@ -384,8 +387,9 @@ self_attn_logq_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         const uint32_t sb = (uint32_t)g & (walk_codes ? 1u : (uint32_t)Cfg::BUFS - 1u);
         // After a time-out every wait returns at once and the loops run to their ends on whatever the buffers hold (an
         // error is recorded): no warp leaves early, so the named barriers are always reached by all their warps.
-        mbar_wait_handover(smem_u32(&sh->s_full[sb]), (s_par >> sb) & 1u, abort_flag);
-        s_par ^= 1u << sb;
+        const uint32_t full_par = Cfg::ISSUERS == 2 ? s_par >> sb : TEAMS == 2 ? s_par : (uint32_t)g >> 1;
+        mbar_wait_handover(smem_u32(&sh->s_full[sb]), full_par & 1u, abort_flag);
+        s_par ^= Cfg::ISSUERS == 2 ? 1u << sb : 1u;
         __syncwarp();
         tc_fence_after();
 #pragma unroll
